@@ -6,7 +6,7 @@
 // the final assignment costs at most n * eps_final more than the optimum: the
 // mean is within eps_final of the exact EMD.
 //
-// Bid kernel: one warp per unassigned point of A; the points of B and their
+// Bid kernel without lists (more than kTailMaxN points): one warp per unassigned point of A; the points of B and their
 // prices are streamed through shared memory in tiles; each lane keeps the best
 // and second-best value (-distance - price) and the warp merges them; the bid
 // (price + best - second + eps) goes to the object with a 64-bit atomic max of
@@ -133,55 +133,272 @@ __global__ void k_emd_resolve(int n, float *price, int *owner, int *assign, unsi
     price[j] = __uint_as_float((unsigned)(b >> 32));
 }
 
-// Gauss-Seidel tail: once few points are unassigned, one block finishes the
-// phase, one bid at a time, with the other set and its prices held in shared
-// memory (n <= kTailMaxN): the unassigned points are queued in index order,
-// each bid is a block-wide scan for the best and second-best object, and an
-// evicted owner joins the back of the queue.  At most max_bids bids; *active
-// gets the points still queued.
-constexpr int kTailThreads = 1024;
-constexpr int kTailQueue = 256;
+// ---------------------------------------------------------------------------
+// Candidate lists.  A point's bid needs its best and second-best value over
+// all n objects, but prices only rise within a call, so values only fall: a
+// list of the objects whose value exceeded a threshold T when it was made, with
+// their distances, still holds the best two as long as the best listed value
+// is above T and the second is not below it (everything outside is at most T).
+// Such a bid reads kListMax entries instead of n objects.  The threshold is the
+// second-best value at that time less a margin, adapted per point so that
+// about 160 objects qualify.  A list that no longer decides is made again by
+// a scan of all objects; one that cannot (more than kListMax objects within the
+// margin, e.g. coincident points) gives way to an exact scan for that bid.
+// Either way the bid is the one a full scan gives, bit for bit: the same
+// distances, the same subtraction, ties to the lowest object id.
+// ---------------------------------------------------------------------------
+constexpr int kListMax = 256;                        // entries; eight per lane
+constexpr int kListLow = 120, kListHigh = 208;       // entries aimed for
 
-__device__ __forceinline__ void block_best2(float &b1, int &j1, float &b2, float *r1, float *r2, int *rj) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        float o1 = __shfl_xor_sync(0xffffffffu, b1, o), o2 = __shfl_xor_sync(0xffffffffu, b2, o);
-        int oj = __shfl_xor_sync(0xffffffffu, j1, o);
-        merge2(b1, j1, b2, o1, oj, o2);
-    }
-    if (lane == 0) { r1[wid] = b1; r2[wid] = b2; rj[wid] = j1; }
-    __syncthreads();
-    if (wid == 0) {
-        const int nw = blockDim.x >> 5;
-        b1 = lane < nw ? r1[lane] : -INFINITY;
-        b2 = lane < nw ? r2[lane] : -INFINITY;
-        j1 = lane < nw ? rj[lane] : 0x7fffffff;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            float o1 = __shfl_xor_sync(0xffffffffu, b1, o), o2 = __shfl_xor_sync(0xffffffffu, b2, o);
-            int oj = __shfl_xor_sync(0xffffffffu, j1, o);
-            merge2(b1, j1, b2, o1, oj, o2);
-        }
-        if (lane == 0) { r1[0] = b1; r2[0] = b2; rj[0] = j1; }
-    }
-    __syncthreads();
-    b1 = r1[0]; b2 = r2[0]; j1 = rj[0];
-    __syncthreads();
+struct EmdLists {
+    int4 *entry;       // [n][kListMax / 2], two (object, distance bits) pairs each
+    float2 *hdr;       // [n] (threshold, margin); threshold +inf: no list yet
+};
+
+// Distance of a point and an object: the one expression every path values with.
+__device__ __forceinline__ float emd_d2(float4 a, float bx, float by, float bz) {
+    float dx = a.x - bx, dy = a.y - by, dz = a.z - bz;
+    return dx * dx + dy * dy + dz * dz;
 }
 
-__global__ void __launch_bounds__(kTailThreads)
-k_emd_tail(int n, const float4 *__restrict__ A4, const float4 *__restrict__ B4, float *price, int *owner,
-           int *assign, float eps, int max_bids, unsigned *active) {
-    extern __shared__ float4 tsm[];
-    float4 *sB = tsm;
-    float *sp = reinterpret_cast<float *>(sB + n);
+__device__ __forceinline__ float warp_max(float v) { return ord2f_emd(__reduce_max_sync(0xffffffffu, f2ord_emd(v))); }
+
+// Best (lowest object on ties) and second-best value of a warp from its lanes'.
+__device__ __forceinline__ void warp_best2(float &b1, int &j1, float &b2) {
+    const unsigned full = 0xffffffffu;
+    const float m = warp_max(b1);
+    const int j = (int)__reduce_min_sync(full, b1 == m ? (unsigned)j1 : 0x7fffffffu);
+    const bool owner = b1 == m && j1 == j;
+    b2 = warp_max(owner ? b2 : b1);
+    b1 = m;
+    j1 = j;
+}
+
+// The best two of a point from its list (e: this lane's eight entries) at the
+// current prices.
+template <typename Price>
+__device__ __forceinline__ void list_best2(const int4 (&e)[4], Price price, float &b1, int &j1, float &b2) {
+    b1 = b2 = -INFINITY;
+    j1 = 0x7fffffff;
+    auto take = [&](int j, int dbits) {
+        const float v = -__int_as_float(dbits) - price(j);
+        const bool better = v > b1 || (v == b1 && j < j1);
+        b2 = fmaxf(b2, better ? b1 : v);
+        if (better) { b1 = v; j1 = j; }
+    };
+#pragma unroll
+    for (int m = 0; m < 4; ++m) {
+        take(e[m].x, e[m].y);
+        take(e[m].z, e[m].w);
+    }
+    warp_best2(b1, j1, b2);
+}
+
+__device__ __forceinline__ void list_load(const EmdLists &L, int i, int lane, int4 (&e)[4]) {
+    const int4 *p = L.entry + (size_t)i * (kListMax / 2) + lane;
+#pragma unroll
+    for (int m = 0; m < 4; ++m) e[m] = p[32 * m];
+}
+
+// An object belongs on the list of threshold T when its value exceeds T; tested
+// on the squared distance (no square root) and widened for rounding, so none
+// is missed -- an extra entry does no harm.
+__device__ __forceinline__ bool list_qualifies(float d2, float price, float T) {
+    const float r = (-T - price) + 2e-6f * (fabsf(T) + fabsf(price));
+    return r > 0.0f && d2 <= r * r * 1.000002f;
+}
+
+__device__ __forceinline__ void list_append(const EmdLists &L, int i, int *cnt, int j, float d2) {
+    const int pos = atomicAdd(cnt, 1);
+    if (pos < kListMax)
+        reinterpret_cast<int2 *>(L.entry)[(size_t)i * kListMax + pos] = make_int2(j, __float_as_int(sqrtf(d2)));
+}
+
+// Closes a list of cnt entries: the rest padded with entries of value -inf
+// (thread t of nt), threshold and next margin by thread 0.
+__device__ __forceinline__ void list_close(const EmdLists &L, int i, int cnt, int n, float T, float margin, int t,
+                                           int nt) {
+    for (int k = cnt + t; k < kListMax; k += nt)
+        reinterpret_cast<int2 *>(L.entry)[(size_t)i * kListMax + k] = make_int2(0, 0x7f800000);
+    if (t != 0) return;
+    if (cnt > kListMax) { T = INFINITY; margin *= 0.5f; }            // too many: no list
+    else if (cnt == n) T = -INFINITY;                                // every object is listed
+    else if (cnt > kListHigh) margin *= 0.8f;
+    else if (cnt < kListLow) margin *= 1.25f;
+    L.hdr[i] = make_float2(T, margin);
+}
+
+// Value of an object to within about 1e-6 of its distance, for choosing a
+// threshold: one reciprocal-root instruction instead of a rounded square root.
+__device__ __forceinline__ float value_approx(float d2, float price) {
+    return -(d2 * rsqrtf(fmaxf(d2, 1e-30f))) - price;
+}
+
+__global__ void k_emd_lists_init(int n, EmdLists L, float margin) {
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) L.hdr[i] = make_float2(INFINITY, margin);
+}
+
+// One round of bids with lists (n <= kTailMaxN): one warp per unassigned point
+// reads its list; the block then scans the objects for the points whose lists
+// did not decide, two at a time, and those bid from their new lists.  B4 holds
+// the prices in w.
+__global__ void __launch_bounds__(kEmdBlock)
+k_emd_bid_lists(int n, const float4 *__restrict__ A4, const float4 *__restrict__ B4, const int *__restrict__ assign,
+                unsigned long long *bids, EmdLists L, float eps, unsigned *active) {
+    __shared__ int s_point[kEmdWarps], s_miss;
+    __shared__ float s_b1[2][kEmdWarps], s_b2[2][kEmdWarps];
+    __shared__ int s_cnt[2];
+    pdl_wait();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (threadIdx.x == 0) s_miss = 0;
+    __syncthreads();
+    auto price = [&](int j) { return __ldcg(&B4[j].w); };
+    auto place = [&](int i, float b1, int j1, float b2) {
+        if (lane != 0) return;
+        atomicAdd(active, 1u);
+        if ((unsigned)j1 >= (unsigned)n) return;      // no comparable value (NaN input): unassigned, no bid
+        const float inc = (b2 == -INFINITY ? 0.0f : b1 - b2) + eps;
+        const float bid = price(j1) + inc;
+        atomicMax(&bids[j1], ((unsigned long long)__float_as_uint(bid) << 32) | (unsigned)i);
+    };
+    // true when point i bid from its list
+    auto bid_from_list = [&](int i) {
+        const float T = L.hdr[i].x;
+        if (T == INFINITY) return false;
+        int4 e[4];
+        list_load(L, i, lane, e);
+        float b1, b2;
+        int j1;
+        list_best2(e, price, b1, j1, b2);
+        if (!(b1 > T && b2 >= T)) return false;
+        place(i, b1, j1, b2);
+        return true;
+    };
+    {
+        const int i = blockIdx.x * kEmdWarps + wid;
+        if (i < n && assign[i] < 0 && !bid_from_list(i) && lane == 0) s_point[atomicAdd(&s_miss, 1)] = i;
+    }
+    __syncthreads();
+    const int misses = s_miss;
+    for (int m0 = 0; m0 < misses; m0 += 2) {
+        const int two = min(2, misses - m0);
+        const int pt[2] = {s_point[m0], s_point[m0 + two - 1]};
+        const float4 a[2] = {A4[pt[0]], A4[pt[1]]};
+        const float margin[2] = {L.hdr[pt[0]].y, L.hdr[pt[1]].y};
+        float b1[2] = {-INFINITY, -INFINITY}, b2[2] = {-INFINITY, -INFINITY};
+        for (int j = threadIdx.x; j < n; j += kEmdBlock) {
+            const float4 b = __ldcg(&B4[j]);
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                const float v = value_approx(emd_d2(a[k], b.x, b.y, b.z), b.w);
+                b2[k] = fmaxf(b2[k], fminf(b1[k], v));
+                b1[k] = fmaxf(b1[k], v);
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            int dummy = lane;
+            warp_best2(b1[k], dummy, b2[k]);
+            if (lane == 0) { s_b1[k][wid] = b1[k]; s_b2[k][wid] = b2[k]; }
+        }
+        if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
+        __syncthreads();
+        float T[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            float c1 = lane < kEmdWarps ? s_b1[k][lane] : -INFINITY, c2 = lane < kEmdWarps ? s_b2[k][lane] : -INFINITY;
+            int dummy = lane;
+            warp_best2(c1, dummy, c2);
+            T[k] = c2 - margin[k];
+        }
+        for (int j = threadIdx.x; j < n; j += kEmdBlock) {
+            const float4 b = __ldcg(&B4[j]);
+#pragma unroll
+            for (int k = 0; k < 2; ++k) {
+                if (k >= two) break;
+                const float d2 = emd_d2(a[k], b.x, b.y, b.z);
+                if (list_qualifies(d2, b.w, T[k])) list_append(L, pt[k], &s_cnt[k], j, d2);
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < 2; ++k)
+            if (k < two) list_close(L, pt[k], s_cnt[k], n, T[k], margin[k], threadIdx.x, kEmdBlock);
+        __syncthreads();
+        if (wid < two) {
+            const int i = pt[wid];
+            if (!bid_from_list(i)) {                  // exact scan by the warp
+                float c1 = -INFINITY, c2 = -INFINITY;
+                int j1 = 0x7fffffff;
+                for (int j = lane; j < n; j += 32) {
+                    const float4 b = __ldcg(&B4[j]);
+                    merge2(c1, j1, c2, -sqrtf(emd_d2(a[wid], b.x, b.y, b.z)) - b.w, j, -INFINITY);
+                }
+                warp_best2(c1, j1, c2);
+                place(i, c1, j1, c2);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+__global__ void k_emd_resolve_lists(int n, float4 *__restrict__ B4, int *owner, int *assign,
+                                    unsigned long long *bids) {
+    pdl_wait();
+    int j = blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n) return;
+    unsigned long long b = bids[j];
+    if (b == 0ull) return;
+    bids[j] = 0ull;
+    int winner = (int)(b & 0xffffffffull);
+    int old = owner[j];
+    if (old >= 0) assign[old] = -1;
+    owner[j] = winner;
+    assign[winner] = j;
+    B4[j].w = __uint_as_float((unsigned)(b >> 32));
+}
+
+// Gauss-Seidel tail: once few points are unassigned, one block finishes the
+// phase, one bid at a time: the unassigned points are queued in index order and
+// an evicted owner joins the back of the queue.  At most max_bids bids;
+// *active gets the points still queued.
+//
+// Warp 0 commits bids: prices and owners in shared memory, the bidder's list
+// (read through L1: the points of a price war take turns, and 91 KB of shared
+// memory leave the SM room to keep theirs), the next bidder's list fetched
+// ahead while the queue holds one.  When a list does not decide, the other 31
+// warps, which hold the objects' coordinates in registers, make it again.
+// A call is a chain of ~270k dependent bids at 10k points, so the latency of
+// one bid is the time: a block-wide scan of all objects for each took 2.0 us
+// (531 of the call's 545 ms; 259 ms with lists, of which a bid from its list
+// takes about 1600 cycles, most of them the list's trip from L2, and a new
+// list about 10000).
+constexpr int kTailThreads = 1024;
+constexpr int kTailQueue = 256;
+constexpr int kScanThreads = kTailThreads - 32;      // warps 1-31
+constexpr int kScanPer = 12;                         // objects a scanning thread holds
+constexpr int kTailMaxN = 11417;                     // largest n taken (16 + 4 B of shared memory each would fit)
+static_assert(kScanThreads * kScanPer >= kTailMaxN, "every object is held by a thread");
+
+enum { kTailDone = 0, kTailList = 1, kTailExact = 2 };
+
+__device__ __forceinline__ void bar_sync(int id, int threads) {
+    asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+__global__ void __launch_bounds__(kTailThreads, 1)
+k_emd_tail(int n, const float4 *__restrict__ A4, float4 *B4, float *price, int *owner, int *assign, EmdLists L,
+           float eps, int max_bids, unsigned *active) {
+    extern __shared__ float sp[];                    // prices, then owners
+    int *s_own = reinterpret_cast<int *>(sp + n);
     __shared__ int queue[kTailQueue];
     __shared__ float r1[32], r2[32];
-    __shared__ int rj[32], s_cnt[32];
-    __shared__ int s_len;
+    __shared__ int rj[32], s_wcnt[32];
+    __shared__ int s_len, s_mode, s_point, s_cnt;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-    for (int j = tid; j < n; j += kTailThreads) { sB[j] = B4[j]; sp[j] = price[j]; }
+    const bool lists = L.entry != nullptr;
+    for (int j = tid; j < n; j += kTailThreads) { sp[j] = price ? price[j] : B4[j].w; s_own[j] = owner[j]; }
     if (tid == 0) s_len = 0;
     __syncthreads();
     // unassigned points in index order (up to the queue's size)
@@ -189,49 +406,166 @@ k_emd_tail(int n, const float4 *__restrict__ A4, const float4 *__restrict__ B4, 
         int i = c0 + tid;
         bool un = i < n && assign[i] < 0;
         unsigned ball = __ballot_sync(0xffffffffu, un);
-        if (lane == 0) s_cnt[wid] = __popc(ball);
+        if (lane == 0) s_wcnt[wid] = __popc(ball);
         __syncthreads();
         int before = s_len;
-        for (int w = 0; w < wid; ++w) before += s_cnt[w];
+        for (int w = 0; w < wid; ++w) before += s_wcnt[w];
         int pos = before + __popc(ball & ((1u << lane) - 1u));
         if (un && pos < kTailQueue) queue[pos] = i;
         __syncthreads();
         if (tid == 0) {
             int tot = s_len;
-            for (int w = 0; w < (kTailThreads >> 5); ++w) tot += s_cnt[w];
+            for (int w = 0; w < (kTailThreads >> 5); ++w) tot += s_wcnt[w];
             s_len = min(tot, kTailQueue);
         }
         __syncthreads();
     }
-    int head = 0, len = s_len;
-    for (int bids = 0; bids < max_bids && len > 0; ++bids) {
-        const int i = queue[head % kTailQueue];
-        const float4 a = A4[i];
-        float b1 = -INFINITY, b2 = -INFINITY;
-        int j1 = 0x7fffffff;
-        for (int j = tid; j < n; j += kTailThreads) {
-            float4 b = sB[j];
-            float dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z;
-            merge2(b1, j1, b2, -sqrtf(dx * dx + dy * dy + dz * dz) - sp[j], j, -INFINITY);
-        }
-        block_best2(b1, j1, b2, r1, r2, rj);
-        int old = owner[j1];                          // read by every thread, written by thread 0 below
-        __syncthreads();
-        if (tid == 0) {
-            sp[j1] += (b2 == -INFINITY ? 0.0f : b1 - b2) + eps;
-            owner[j1] = i;
-            assign[i] = j1;
-            if (old >= 0) {
-                assign[old] = -1;
-                queue[(head + len) % kTailQueue] = old;
+    if (wid == 0) {
+        int head = 0, len = s_len, bids = 0, mode = kTailDone;
+        auto commit = [&](int i, float b1, int j1, float b2) {
+            const int old = s_own[j1];
+            __syncwarp();
+            if (lane == 0) {
+                sp[j1] += (b2 == -INFINITY ? 0.0f : b1 - b2) + eps;
+                s_own[j1] = i;
+                assign[i] = j1;
+                if (old >= 0) {
+                    assign[old] = -1;
+                    queue[(head + len) % kTailQueue] = old;
+                }
+            }
+            ++head;
+            ++bids;
+            if (old < 0) --len;
+            __syncwarp();
+        };
+        auto price_of = [&](int j) { return sp[j]; };
+        bool fresh = false;                          // the head's list was just made
+        while (true) {
+            mode = kTailDone;
+            int i = -1;
+            if (lists) {
+                int4 e[4];
+                float T = 0.0f;
+                int have = -1;                       // the point whose list e and T hold
+                while (bids < max_bids && len > 0) {
+                    i = queue[head % kTailQueue];
+                    if (have != i) {
+                        T = L.hdr[i].x;
+                        list_load(L, i, lane, e);
+                    }
+                    int4 f[4];
+                    float Tn = 0.0f;
+                    int next = -1;
+                    if (len > 1) {
+                        next = queue[(head + 1) % kTailQueue];
+                        Tn = L.hdr[next].x;
+                        list_load(L, next, lane, f);
+                    }
+                    mode = kTailList;
+                    if (T == INFINITY) break;
+                    float b1, b2;
+                    int j1;
+                    list_best2(e, price_of, b1, j1, b2);
+                    if (!(b1 > T && b2 >= T)) break;
+                    commit(i, b1, j1, b2);
+                    mode = kTailDone;
+                    fresh = false;
+                    have = next;
+                    T = Tn;
+                    if (next >= 0) {
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) e[m] = f[m];
+                    }
+                }
+                if (mode == kTailList && fresh) mode = kTailExact;
+            } else if (bids < max_bids && len > 0) {
+                i = queue[head % kTailQueue];
+                mode = kTailExact;
+            }
+            if (lane == 0) { s_mode = mode; s_point = i; }
+            bar_sync(1, kTailThreads);
+            if (mode == kTailDone) break;
+            bar_sync(1, kTailThreads);               // the scan is done
+            fresh = mode == kTailList;
+            if (mode == kTailExact) {
+                float b1 = lane > 0 ? r1[lane] : -INFINITY, b2 = lane > 0 ? r2[lane] : -INFINITY;
+                int j1 = lane > 0 ? rj[lane] : 0x7fffffff;
+                warp_best2(b1, j1, b2);
+                if ((unsigned)j1 >= (unsigned)n) {   // no comparable value (NaN input): leave the point queued
+                    max_bids = bids;
+                    continue;
+                }
+                commit(i, b1, j1, b2);
             }
         }
-        ++head;
-        if (old < 0) --len;
-        __syncthreads();
+        if (lane == 0) *active = (unsigned)len;
+    } else {
+        const int t = tid - 32;
+        float bx[kScanPer], by[kScanPer], bz[kScanPer];
+#pragma unroll
+        for (int k = 0; k < kScanPer; ++k) {
+            const int j = t + k * kScanThreads;
+            const float4 b = j < n ? B4[j] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            bx[k] = b.x; by[k] = b.y; bz[k] = b.z;
+        }
+        while (true) {
+            bar_sync(1, kTailThreads);
+            const int mode = s_mode, i = s_point;
+            if (mode == kTailDone) break;
+            const float4 a = A4[i];
+            float b1 = -INFINITY, b2 = -INFINITY;
+            if (mode == kTailExact) {
+                int j1 = 0x7fffffff;
+#pragma unroll
+                for (int k = 0; k < kScanPer; ++k) {
+                    const int j = t + k * kScanThreads;
+                    if (j < n) merge2(b1, j1, b2, -sqrtf(emd_d2(a, bx[k], by[k], bz[k])) - sp[j], j, -INFINITY);
+                }
+                warp_best2(b1, j1, b2);
+                if (lane == 0) { r1[wid] = b1; r2[wid] = b2; rj[wid] = j1; }
+                bar_sync(1, kTailThreads);
+                continue;
+            }
+            const float margin = L.hdr[i].y;
+            if (t == 0) s_cnt = 0;
+#pragma unroll
+            for (int k = 0; k < kScanPer; ++k) {
+                const int j = t + k * kScanThreads;
+                if (j < n) {
+                    const float v = value_approx(emd_d2(a, bx[k], by[k], bz[k]), sp[j]);
+                    b2 = fmaxf(b2, fminf(b1, v));
+                    b1 = fmaxf(b1, v);
+                }
+            }
+            int dummy = lane;
+            warp_best2(b1, dummy, b2);
+            if (lane == 0) { r1[wid] = b1; r2[wid] = b2; }
+            bar_sync(2, kScanThreads);
+            b1 = lane > 0 ? r1[lane] : -INFINITY;
+            b2 = lane > 0 ? r2[lane] : -INFINITY;
+            dummy = lane;
+            warp_best2(b1, dummy, b2);
+            const float T = b2 - margin;
+#pragma unroll
+            for (int k = 0; k < kScanPer; ++k) {
+                const int j = t + k * kScanThreads;
+                if (j < n) {
+                    const float d2 = emd_d2(a, bx[k], by[k], bz[k]);
+                    if (list_qualifies(d2, sp[j], T)) list_append(L, i, &s_cnt, j, d2);
+                }
+            }
+            bar_sync(2, kScanThreads);
+            list_close(L, i, s_cnt, n, T, margin, t, kScanThreads);
+            bar_sync(1, kTailThreads);
+        }
     }
-    for (int j = tid; j < n; j += kTailThreads) price[j] = sp[j];
-    if (tid == 0) *active = (unsigned)len;
+    __syncthreads();
+    for (int j = tid; j < n; j += kTailThreads) {
+        if (price) price[j] = sp[j];
+        else B4[j].w = sp[j];
+        owner[j] = s_own[j];
+    }
 }
 
 // Mean cost of the assignment in float64, summed in a fixed order.
@@ -269,6 +603,8 @@ k_emd_cost(int n, const float4 *__restrict__ A4, const float4 *__restrict__ B4, 
 }
 
 struct EmdWs {
+    EmdLists L;
+    size_t base_bytes;             // without the lists
     float4 *A4, *B4;
     float *price;
     int *owner, *assign;
@@ -296,6 +632,12 @@ static EmdWs emd_ws(void *ws, int64_t n) {
     w.active = w.box + 8;
     w.ticket = w.box + 9;
     w.partial = (double *)(b + oPart);
+    w.base_bytes = off;
+    w.L = EmdLists{nullptr, nullptr};
+    if (n <= kTailMaxN) {
+        size_t oE = take(8 * (size_t)kListMax * m), oH = take(8 * m);
+        w.L = EmdLists{(int4 *)(b + oE), (float2 *)(b + oH)};
+    }
     w.bytes = off;
     return w;
 }
@@ -324,7 +666,11 @@ mesh_status mesh_emd(const float *d_A, const float *d_B, int64_t n, float eps_re
         return check_launch();
     }
     EmdWs w = emd_ws(d_ws, n);
-    if (!d_ws || ws_bytes < w.bytes || ((uintptr_t)d_ws & 255u)) return MESH_ERR_WORKSPACE;
+    if (!d_ws || ws_bytes < w.base_bytes || ((uintptr_t)d_ws & 255u)) return MESH_ERR_WORKSPACE;
+    // Lists where they fit: to kTailMaxN points (2 KB each; beyond that the tail, which
+    // makes most bids, does not run), and not in a workspace without room for them.
+    const bool lists = n <= kTailMaxN && ws_bytes >= w.bytes;
+    if (!lists) w.L = EmdLists{nullptr, nullptr};
     const int N = (int)n;
     unsigned init_box[10] = {0xffffffffu, 0xffffffffu, 0xffffffffu, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
     if (cudaMemcpyAsync(w.box, init_box, sizeof(init_box), cudaMemcpyHostToDevice, s) != cudaSuccess)
@@ -347,17 +693,13 @@ mesh_status mesh_emd(const float *d_A, const float *d_B, int64_t n, float eps_re
     if (!(C > 0.0)) C = 1.0;
     const double eps_final = eps_rel * C;
     const unsigned bid_grid = grid_for(N, kEmdWarps);
-    static int64_t tail_max = -1;                    // largest n whose set fits the tail's shared memory
-    auto tail_smem = [](int m) { return (size_t)m * (sizeof(float4) + sizeof(float)); };
-    if (tail_max < 0) {
-        int dev = 0, optin = 0;
-        tail_max = 0;
-        if (cudaGetDevice(&dev) == cudaSuccess &&
-            cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) == cudaSuccess &&
-            optin > 4096 && cudaFuncSetAttribute(k_emd_tail, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                 optin - 4096) == cudaSuccess)
-            tail_max = (optin - 4096) / (int64_t)(sizeof(float4) + sizeof(float));
-        cudaGetLastError();
+    static const bool tail_ok =                       // the dynamic shared memory the tail takes
+        cudaFuncSetAttribute(k_emd_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kTailMaxN) == cudaSuccess;
+    if (!tail_ok) return MESH_ERR_CUDA;
+    if (lists) {
+        // a first guess of the margin: about 1 % of the box diagonal's objects at 10k points
+        k_emd_lists_init<<<grid_for(N, 256), 256, 0, s>>>(N, w.L, (float)(0.25 * C * sqrt(160.0 / (double)N)));
+        count_launch();
     }
     int64_t iters = 0;
     for (double eps = C / 10.0;; eps /= 8.0) {
@@ -367,10 +709,18 @@ mesh_status mesh_emd(const float *d_A, const float *d_B, int64_t n, float eps_re
         bool done = false;
         while (!done) {
             for (int k = 0; k < kEmdCheck; ++k) {
-                cudaMemsetAsync(w.active, 0, sizeof(unsigned), s);
-                k_emd_bid<<<bid_grid, kEmdBlock, 0, s>>>(N, w.A4, w.B4, w.price, w.assign, w.bids, (float)eps,
-                                                         w.active);
-                k_emd_resolve<<<grid_for(N, 256), 256, 0, s>>>(N, w.price, w.owner, w.assign, w.bids);
+                // the count wanted is the last round's
+                if (k == 0 || k == kEmdCheck - 1 || !lists) cudaMemsetAsync(w.active, 0, sizeof(unsigned), s);
+                if (lists) {
+                    const bool after_kernel = k != 0 && k != kEmdCheck - 1;
+                    launch_ex(after_kernel, k_emd_bid_lists, bid_grid, kEmdBlock, 0, s, N, (const float4 *)w.A4,
+                              (const float4 *)w.B4, (const int *)w.assign, w.bids, w.L, (float)eps, w.active);
+                    pdl_launch(k_emd_resolve_lists, grid_for(N, 256), 256, 0, s, N, w.B4, w.owner, w.assign, w.bids);
+                } else {
+                    k_emd_bid<<<bid_grid, kEmdBlock, 0, s>>>(N, w.A4, w.B4, w.price, w.assign, w.bids, (float)eps,
+                                                             w.active);
+                    k_emd_resolve<<<grid_for(N, 256), 256, 0, s>>>(N, w.price, w.owner, w.assign, w.bids);
+                }
                 count_launch(2);
                 ++iters;
             }
@@ -379,11 +729,11 @@ mesh_status mesh_emd(const float *d_A, const float *d_B, int64_t n, float eps_re
                 cudaStreamSynchronize(s) != cudaSuccess)
                 return MESH_ERR_CUDA;
             done = act == 0;
-            if (!done && act <= (unsigned)kTailQueue && n <= tail_max) {
+            if (!done && act <= (unsigned)kTailQueue && n <= kTailMaxN) {
                 int64_t left = max_iters > iters ? max_iters - iters : 1;
                 int cap = (int)(left < (int64_t)(1 << 24) ? left : (int64_t)(1 << 24));
-                k_emd_tail<<<1, kTailThreads, tail_smem(N), s>>>(N, w.A4, w.B4, w.price, w.owner, w.assign,
-                                                                 (float)eps, cap, w.active);
+                k_emd_tail<<<1, kTailThreads, 8 * (size_t)N, s>>>(N, w.A4, w.B4, lists ? nullptr : w.price, w.owner,
+                                                                  w.assign, w.L, (float)eps, cap, w.active);
                 count_launch();
                 if (cudaMemcpyAsync(&act, w.active, sizeof(unsigned), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
                     cudaStreamSynchronize(s) != cudaSuccess)

@@ -60,3 +60,38 @@ def test_emd_translation_at_10k_points():
     v = float(emd(dev(A), dev(B), eps_rel=1e-5).item())
     C = diag(A, B)
     assert abs(v - np.linalg.norm(t)) <= 1e-5 * C + 1e-6
+
+
+def _points_of(kind, n, rng):
+    if kind == "normal":
+        return rng.normal(size=(n, 3)).astype(np.float32)
+    if kind == "one":                               # every point the same
+        return np.full((n, 3), 0.25, np.float32)
+    if kind == "clusters":                          # a few points, each many times
+        return rng.normal(size=(5, 3)).astype(np.float32)[rng.integers(0, 5, n)]
+    i = np.arange(n)                                # a grid: many equal distances
+    return np.stack([i % 10, i // 10 % 10, i // 100], 1).astype(np.float32)
+
+
+@pytest.mark.parametrize("kind_a,kind_b", [("normal", "normal"), ("normal", "one"), ("clusters", "normal"),
+                                           ("normal", "clusters"), ("grid", "grid")])
+@pytest.mark.parametrize("n", [1, 2, 33, 256, 257, 1100])
+def test_emd_candidate_lists_leave_every_bid_unchanged(n, kind_a, kind_b):
+    """A workspace without room for the candidate lists runs every bid as a scan of all
+    objects: the mean, the assignment and the rounds are those with lists, bit for bit."""
+    import ctypes as C
+    from paper_2606_00444_gb300._abi import lib
+    rng = np.random.default_rng(n)
+    A, B = dev(_points_of(kind_a, n, rng)), dev(_points_of(kind_b, n, rng))
+    need = lib().mesh_emd_workspace_bytes(n)
+    got = []
+    for nbytes in (need, need - 1):
+        ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+        out = torch.empty(1, dtype=torch.float64, device="cuda")
+        sigma = torch.empty(n, dtype=torch.int32, device="cuda")
+        it = C.c_int64(0)
+        st = lib().mesh_emd(A.data_ptr(), B.data_ptr(), n, 1e-3, 200000, ws.data_ptr(), nbytes, out.data_ptr(),
+                            sigma.data_ptr(), C.byref(it), torch.cuda.current_stream().cuda_stream)
+        assert st == 0
+        got.append((host(out), host(sigma), it.value))
+    assert got[0][2] == got[1][2] and np.array_equal(got[0][1], got[1][1]) and np.array_equal(got[0][0], got[1][0])
