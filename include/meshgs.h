@@ -247,8 +247,9 @@ mesh_status mesh_closest_point(const mesh_bvh *bvh, const float *d_Q, int64_t nQ
  * the final tie window is still reached, so the answer is the one without the
  * hint, bit for bit; the hint changes only the work.  d_hint may be the same
  * array as d_face (each query reads its hint before writing its face).  Used by
- * the depth-first one-thread variants (0, 2-9, 13), the warp packets (12) and
- * the cooperative groups (lanes > 1); variants 1, 10 and 11 ignore it. */
+ * the pooled search (variant 0, and every call with several lanes per query),
+ * the depth-first one-thread variants (2-9, 13) and the warp packets (12);
+ * variants 1, 10 and 11 ignore it. */
 mesh_status mesh_closest_point_hinted(const mesh_bvh *bvh, const float *d_Q, int64_t nQ,
                                       float max_dist, const int32_t *d_hint, int32_t *d_face,
                                       float *d_bary, float *d_point, float *d_dist2, void *stream);
@@ -360,22 +361,22 @@ size_t mesh_contact_workspace_bytes(int64_t nQ);
 
 /* The contact query of a physics step: NearestSurface of the nQ particles
  * with cutoff max_dist, with d_face both the previous step's answers (read
- * first, as warm-start hints: -1 = none) and this step's (written).  The
- * queries run in the order of the previous step's work: each query's node
- * visits give it a class (48 or more, 24-47, 12-23, fewer), kept in d_ws,
- * and the next call runs the classes heaviest first, each in the given
- * order, so that a warp holds searches of similar depth.  d_ws therefore
- * carries state from one step to the next: pass the same workspace every
- * step for the same particles; its contents steer only the order (a fresh
- * or unrelated workspace gives a worse order, never a wrong answer).
- * Answers equal mesh_closest_point's bit for bit.  The one-thread searches
- * write face and distance; the weights and closest points (when asked for)
- * follow in a second launch with one thread per query (the distances are kept
- * in d_ws when d_dist2 is NULL).
- * Traversal variants 1, 10, 11 and cooperative groups run unordered without
- * classes (the warp packets of variant 12 take the classes, counting for each
- * query the nodes whose children it needed).  d_ws:
- * mesh_contact_workspace_bytes(nQ), 256-byte aligned. */
+ * first, as warm-start hints: -1 = none) and this step's (written).  Answers
+ * equal mesh_closest_point's bit for bit.  The default (the pooled search) needs
+ * nothing else.  The one-thread variants 2-9, 12 and 13 run the queries in the
+ * order of the previous step's work: each query's node visits give it a class
+ * (48 or more, 24-47, 12-23, fewer), kept in d_ws, and the next call runs the
+ * classes heaviest first, each in the given order, so that a warp holds searches
+ * of similar depth.  For them d_ws carries state from one step to the next: pass
+ * the same workspace every step for the same particles; its contents steer only
+ * the order (a fresh or unrelated workspace gives a worse order, never a wrong
+ * answer).  Their searches write face and distance; the weights and closest
+ * points (when asked for) follow in a second launch with one thread per query
+ * (the distances are kept in d_ws when d_dist2 is NULL; the warp packets of
+ * variant 12 write everything themselves and count for each query the nodes
+ * whose children it needed).  Variants 1, 10 and 11 and calls with several lanes
+ * per query run unordered.  d_ws: mesh_contact_workspace_bytes(nQ), 256-byte
+ * aligned. */
 mesh_status mesh_contact(const mesh_bvh *bvh, const float *d_Q, int64_t nQ, float max_dist,
                          int32_t *d_face, float *d_bary, float *d_point, float *d_dist2, void *d_ws,
                          size_t ws_bytes, void *stream);
@@ -389,20 +390,23 @@ mesh_status mesh_contact(const mesh_bvh *bvh, const float *d_Q, int64_t nQ, floa
 mesh_status mesh_closest_point_stats(const mesh_bvh *bvh, const float *d_Q, int64_t nQ,
                                      float max_dist, unsigned long long *d_counts, void *stream);
 
-/* Lanes that cooperate on one query in mesh_closest_point and mesh_chamfer.
- * 0 (default) picks from the query count: one thread per query when the
- * queries fill the GPU, else the smallest power of two up to 32 that does (a
- * group pops several stack entries per step and merges its candidates with
- * the same tie rule).  1, 2, 4, 8, 16 or 32 force a width.  Process-wide,
- * not thread-safe; for tuning and tests.  Results are the same for every
- * width, bit for bit. */
+/* Lanes per query in mesh_closest_point and mesh_chamfer: a warp of the pooled
+ * search holds 32 / lanes queries, whose nodes its lanes take from one stack.
+ * 0 (default) and 1 leave the number to the library (16 queries per warp when
+ * the queries fill the GPU, fewer queries per warp when they do not); 1 also
+ * asks mesh_closest_point for a one-thread variant where one is set
+ * (mesh_set_traversal), as 0 does when the queries fill the GPU.  2, 4, 8, 16
+ * or 32 force a width.  Process-wide, not thread-safe; for tuning and tests.
+ * Results are the same for every width, bit for bit. */
 mesh_status mesh_set_query_group(int lanes);
 
-/* One-thread-per-query traversal variant for mesh_closest_point (tuning):
- *   0 depth-first, 24-entry shared-memory stack per thread (default)
+/* Search of mesh_closest_point and mesh_contact (tuning); 1-13 are searches with
+ * one thread per query:
+ *   0 the pooled search: the queries of a warp share one stack of nodes, from
+ *     which each lane takes the next (default)
  *   1 while-while: leaf children queued while internal nodes are traversed
  *   2 depth-first, 8 shared entries    3 depth-first, stack in local memory only
- *   4 as 0 with one leaf-test site     5 as 3 with one leaf-test site
+ *   4 depth-first, 24 shared entries, one leaf-test site     5 as 3 with one leaf-test site
  *   6 as 2, 9 blocks per SM (<= 56 registers)    7 as 3, 9 blocks per SM
  *   8 as 3, 16 blocks per SM (<= 32 registers)   9 as 5, 12 blocks per SM
  *  10 persistent, dynamic fetch: lanes take new queries as they finish
@@ -443,7 +447,7 @@ mesh_status mesh_bvh_set_query_config(mesh_bvh *bvh, int lanes, int variant);
 mesh_status mesh_bvh_set_leaf_size(mesh_bvh *bvh, int leaf_size);
 
 /* Threads per block of this handle's one-thread traversals (mesh_closest_point
- * and mesh_contact with variants 0, 2 and 3): 128 (default; 0 = default), 64 or
+ * and mesh_contact with variants 2, 3 and 13): 128 (default; 0 = default), 64 or
  * 32.  Each form keeps the same register budget, so the same number of warps
  * fits an SM; smaller blocks free their slot as soon as their own searches end
  * (the searches of one block end at very different times).  Host-side setting,
@@ -501,21 +505,11 @@ size_t mesh_chamfer_step_workspace_bytes(int64_t nSA, int64_t nSB);
 /* The Chamfer distance of Sec. 4.2 for a sequence of frames (a physics step or
  * an optimisation step on the same samples): mesh_chamfer with d_faceA /
  * d_faceB both the previous call's faces (read first, as warm-start hints:
- * -1 = none) and this call's (written), and the samples of each side run in
- * the order of the previous call's costs, heaviest first: each sample's cost
- * (its node visits / 8 with one lane per sample, its group steps with
- * several, capped at 127) is kept in d_ws as an 8-bit key with the side in bit
- * 7, and the next call sorts the keys of both sides with one stable radix
- * pass, so that the samples sharing a block end together and the longest
- * searches start first.  d_ws therefore carries state from one call to the
- * next: pass the same workspace for the same samples; its contents steer only
- * the order (a fresh or unrelated workspace gives a worse order, never a
- * wrong answer).  The per-sample outputs equal mesh_chamfer's bit for bit;
- * d_out equals it up to the order of the float64 sums (each block sums its
- * samples, and the blocks hold other samples in another order).  d_faceA is
- * required when nSA > 0, d_faceB when nSB > 0; the other outputs may be NULL.
- * d_ws: mesh_chamfer_step_workspace_bytes(nSA, nSB), 256-byte aligned;
- * MESH_ERR_WORKSPACE otherwise. */
+ * -1 = none) and this call's (written).  The outputs equal mesh_chamfer's bit for
+ * bit.  d_faceA is required when nSA > 0, d_faceB when nSB > 0; the other outputs
+ * may be NULL.  d_ws: mesh_chamfer_step_workspace_bytes(nSA, nSB), 256-byte
+ * aligned; MESH_ERR_WORKSPACE otherwise.  Nothing in it is carried from call to
+ * call. */
 mesh_status mesh_chamfer_step(const mesh_bvh *A, const float *d_SA, int64_t nSA, const mesh_bvh *B,
                               const float *d_SB, int64_t nSB, void *d_ws, size_t ws_bytes, double *d_out,
                               int32_t *d_faceA, float *d_baryA, float *d_dist2A, int32_t *d_faceB,
@@ -604,8 +598,8 @@ mesh_status mesh_bind_gaussians_backward(const mesh_bvh *bvh, const int32_t *d_g
  * (int32, non-decreasing, off[0] = 0, off[B] = total; empty scenes allowed).
  * Each scene gets its own LBVH, identical to the one mesh_build_lbvh builds for
  * that scene alone, but every phase runs as one launch over all scenes, and
- * queries / Gaussians of all scenes go through one persistent launch (warps
- * pull work in chunks from a counter), so per-scene launch overhead vanishes
+ * queries / Gaussians of all scenes go through one launch, so per-scene launch
+ * overhead vanishes
  * and the whole frame can be captured in one CUDA graph. */
 typedef struct mesh_batch mesh_batch;
 
@@ -645,7 +639,7 @@ mesh_status mesh_batch_refit(mesh_batch *batch, const float *d_V, int64_t nV, vo
 
 /* Closest point for queries of every scene: query i belongs to scene s with
  * query_off[s] <= i < query_off[s+1] (device, int32 [B+1]).  Outputs as
- * mesh_closest_point, face ids SCENE-LOCAL.  One persistent launch. */
+ * mesh_closest_point, face ids SCENE-LOCAL.  One launch. */
 mesh_status mesh_batch_closest_point(mesh_batch *batch, const float *d_Q,
                                      const int32_t *d_query_off, int64_t nQ, float max_dist,
                                      int32_t *d_face, float *d_bary, float *d_point,

@@ -228,8 +228,8 @@ class MeshBVH:
         step's faces on entry (-1 = none) and this step's on return.  The arrays of
         `out` (face, and optionally bary, point, dist2) may be CUDA tensors or pinned
         host tensors; the kernel writes pinned ones directly (mesh_mapped_pointer).
-        `ws` carries the work classes that order the next step: pass the same one
-        every step."""
+        `ws` carries the work classes that order the next step with the one-thread
+        traversal variants: pass the same one every step."""
         Q = _f32(Q, 3, "Q")
         n = Q.shape[0]
         shapes = dict(face=(torch.int32, (n,)), bary=(torch.float32, (n, 3)),
@@ -547,10 +547,8 @@ def chamfer_step(A: MeshBVH, SA: torch.Tensor, B: MeshBVH, SB: torch.Tensor, ps:
     """chamfer() for a sequence of frames on the same samples (mesh_chamfer_step):
     ps["faceA"] / ps["faceB"] (int32, required) hold the previous call's faces on entry
     (-1 = none; warm start) and this call's on return, the other entries of ps
-    (baryA, dist2A, baryB, dist2B) are optional outputs, and each side's samples run
-    heaviest first by the costs the previous call left in `ws` (pass the same
-    Workspace every call).  Per-sample results equal chamfer()'s bit for bit; the two
-    means equal it up to the order of the float64 sums."""
+    (baryA, dist2A, baryB, dist2B) are optional outputs.  The results equal chamfer()'s
+    bit for bit."""
     SA = _f32(SA, 3, "SA")
     SB = _f32(SB, 3, "SB")
     nA, nB = SA.shape[0], SB.shape[0]

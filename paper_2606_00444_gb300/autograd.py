@@ -17,7 +17,7 @@ from .api import MeshBVH, Workspace, chamfer, chamfer_backward, chamfer_step
 def chamfer_state(nA: int, nB: int, device="cuda") -> dict:
     """State for Chamfer.apply over a sequence of steps on the same samples (an
     optimisation, a simulation): the per-sample faces (-1 = none yet) and the
-    workspace of mesh_chamfer_step that carries the samples' costs to the next step."""
+    workspace of mesh_chamfer_step."""
     dev = torch.device(device)
     ps = dict(faceA=torch.full((nA,), -1, dtype=torch.int32, device=dev), baryA=torch.empty(nA, 3, device=dev),
               faceB=torch.full((nB,), -1, dtype=torch.int32, device=dev), baryB=torch.empty(nB, 3, device=dev))
@@ -75,7 +75,7 @@ class Chamfer(torch.autograd.Function):
     """[mean_a d(a, B)^2, mean_b d(b, A)^2] for samples SA / SB and meshes (VA, bvhA),
     (VB, bvhB); differentiable in SA, VA, SB and VB.  With `state` (chamfer_state) the
     forward is the step of a sequence (mesh_chamfer_step: warm-started from the previous
-    step's faces, samples heaviest first): the same per-sample faces and weights, hence
+    step's faces): the same per-sample faces and weights, hence
     the same gradients (up to the order of the backward's float atomic sums)."""
 
     @staticmethod

@@ -47,7 +47,7 @@ struct mesh_bvh_impl {
 struct BatchStatus {
     unsigned int status;
     unsigned int n_degenerate;
-    unsigned int work;       // persistent-kernel work counter
+    unsigned int work;       // not used
     unsigned int pad;
 };
 

@@ -1,0 +1,575 @@
+// NearestSurface by warps that pool the work of several queries.
+//
+// A warp holds S queries (32 when there are many, fewer when the queries would
+// not fill the GPU) and one stack of (node, query) entries for all of them.
+// Each step its 32 lanes take the top 32 entries, whoever they belong to: a lane
+// reads one node record (two child boxes), tests both against its entry's query
+// and pruning radius, and the surviving children go back on the stack -- the
+// farther ones of all lanes below the nearer ones, so the pool advances about
+// depth first.  Surviving leaves wait in a second queue until 32 of them fill
+// the warp, and are then tested together.  What a query has found -- the least
+// distance, the pruning radius, the faces near the least distance -- lives in
+// shared memory, where any lane updates it.
+//
+// Why: one thread per query runs as long as its warp's deepest search, and
+// tests a face in nearly every step with three or four lanes on; 8 of 32 lanes
+// did useful work.  Here a lane is idle only while the pool holds fewer entries
+// than lanes, and the tail of one long search is shared by the whole warp: 26 of
+// 32 lanes on, 146 warp instructions per contact query.  Bound by the mix of
+// issue (57 % of slots) and the cached reads of scattered 64-byte records (L1
+// throughput 66 %) at 20 resident warps per SM.  1M contact queries of the
+// 200k-face torus: 549 -> 309 us cold, 380 -> 255 us warm-started (the one-thread
+// form with its work classes); unbounded 12.7 -> 4.5 ms; 20k queries 117 -> 44 us.
+//
+// The answer is the tie rule's (see nearest.cuh), as every search gives it: a
+// node is skipped only when its box is farther than a radius never smaller than
+// the final tie window's, and the nearest face is the lowest id among the
+// recorded faces inside the final window.
+#include <type_traits>
+
+#include "nearest.cuh"
+
+namespace meshgs {
+
+constexpr int kQueryWarps = 1;         // warps per block of the query kernels: a block ends with its own warp (the
+                                       // 64-scene batch 17.4 ms against 17.8 with four)
+constexpr int kChamferWarps = 4;       // and of the Chamfer kernel (its partial sums are per 128 / G samples)
+constexpr int kPoolLeaf = 96;         // waiting leaves: below 32 before a step, at most 64 more after it
+constexpr int kPoolRing = 8;          // faces recorded per query near its least distance
+
+// An entry is a node or first leaf (30 bits), its query's slot (5 bits), a
+// face count less one (3 bits, leaves) and the box distance, its low six bits
+// rounded off: an entry's distance only ever rounds down, so it is never
+// dropped too early.
+template <int S, bool kDeep> struct __align__(16) PoolWarp {
+    // Node entries.  A depth-first search deep inside a mesh defers about 20 siblings, one under a
+    // cutoff few; what the stacks leave of an SM's memory caches the tree.
+    static constexpr int kStack = S == 32 ? 448 : S == 16 ? (kDeep ? 512 : 320) : S == 8 ? (kDeep ? 384 : 256)
+                                  : S == 4 ? (kDeep ? 320 : 192) : kDeep ? 256 : 160;
+    float4 q[S];                      // position, float32 error bound of a distance
+    uint2 stack[kStack];
+    uint2 leaf[kPoolLeaf];
+    uint2 ring[S][kPoolRing];         // (distance bits, leaf) of faces within the window when tested
+    unsigned int dmin[S];             // least squared distance, as bits
+    float thr[S];                     // pruning radius, squared
+    int cnt[S];                       // faces in the ring; more than kPoolRing: some were not recorded
+};
+
+// What differs per query when the queries belong to several scenes.
+template <int S> struct PoolScene {
+    int base[S];                      // first node record and leaf
+    float tau[S];
+};
+
+__device__ __forceinline__ uint2 pool_entry(int id, int slot, int cnt1, float d2) {
+    return make_uint2((unsigned)id | ((unsigned)slot << 30),
+                      (__float_as_uint(d2) & ~63u) | ((unsigned)slot >> 2 << 3) | (unsigned)cnt1);
+}
+__device__ __forceinline__ int pool_id(uint2 e) { return (int)(e.x & 0x3fffffffu); }
+__device__ __forceinline__ int pool_slot(uint2 e) { return (int)((e.x >> 30) | (e.y >> 1 & 0x1cu)); }
+__device__ __forceinline__ int pool_count(uint2 e) { return (int)(e.y & 7u) + 1; }
+__device__ __forceinline__ float pool_dist(uint2 e) { return __uint_as_float(e.y & ~63u); }
+
+// The search of a warp's S queries; lane l < S brings query l (valid or not; T
+// holds its mesh's scale and size) and takes its hit.  hint: a leaf tested first, or -1.  descend: a query without a
+// hint first goes down the nearer children to one leaf, so that the pool
+// starts with a radius for each query (unbounded searches).
+// sc: per-query offsets into T's arrays (queries of several scenes), or NULL.
+template <int S, bool kDeep, bool kRange, bool kScenes>
+__device__ __forceinline__ Hit pool_search(const Traversal &T, PoolWarp<S, kDeep> &W, PoolScene<S> *sc, float3 q, bool valid,
+                                           float maxd2, int hint, bool descend, unsigned int *status) {
+    constexpr int kStack = PoolWarp<S, kDeep>::kStack;
+    const unsigned int kFull = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    const unsigned int lt = (1u << lane) - 1u;
+    // Traversal of slot's scene
+    auto scene_of = [&](int slot) {
+        Traversal t = T;
+        if constexpr (kScenes) {
+            t.nodes += 4 * (size_t)sc->base[slot];
+            t.tris += 3 * (size_t)sc->base[slot];
+            t.tau = sc->tau[slot];
+        }
+        return t;
+    };
+    const bool mine = lane < S && valid && T.n > 0;
+    if (lane < S) {
+        const float slack = query_slack(T, q);
+        W.q[lane] = make_float4(q.x, q.y, q.z, slack);
+        W.dmin[lane] = 0x7f800000u;
+        W.thr[lane] = cutoff_window2(maxd2, T.tau, slack);
+        W.cnt[lane] = 0;
+        if constexpr (kScenes) sc->tau[lane] = T.tau;        // base is set by the caller
+    }
+    __syncwarp();
+    int first = -1, first_cnt = 1;                           // the leaf this query tests first
+    if (mine) {
+        if (hint >= 0) {
+            first = hint;
+        } else if (T.n == 1) {
+            first = 0;
+        } else if (descend) {
+            const Traversal t = scene_of(lane);
+            int node = 0;
+            while (true) {
+                const float4 *r = t.nodes + 4 * (size_t)node;
+                const float4 l0 = ldg4(r), l1 = ldg4(r + 1), r0 = ldg4(r + 2), r1 = ldg4(r + 3);
+                const float dl = box_d2(q, l0, l1), dr = box_d2(q, r0, r1);
+                bool left = dl < dr;
+                if (dl == dr) left = box_minmax_d2(q, l0, l1) <= box_minmax_d2(q, r0, r1);
+                const int c = __float_as_int(left ? l0.w : r0.w);
+                if (c >= 0) { node = c; continue; }
+                first = -c - 1;
+                if constexpr (kRange) first_cnt = __float_as_int(left ? l1.w : r1.w);
+                break;
+            }
+        }
+    }
+    const unsigned int fm = __ballot_sync(kFull, first >= 0), rm = __ballot_sync(kFull, mine && T.n > 1);
+    if (first >= 0) W.leaf[__popc(fm & lt)] = pool_entry(first, lane, first_cnt - 1, 0.0f);
+    if (mine && T.n > 1) W.stack[__popc(rm & lt)] = pool_entry(0, lane, 0, 0.0f);
+    int nleaf = __popc(fm), nstack = __popc(rm);
+    bool start = nleaf > 0;                                  // the first leaves are tested before any node
+    __syncwarp();
+    while (true) {
+        if (nleaf >= 32 || start || (nstack == 0 && nleaf > 0)) {
+            // ---- test up to 32 waiting leaves, one per lane
+            const int take = min(32, nleaf);
+            start = start && nleaf > 32;
+            uint2 e = make_uint2(0u, 0u);
+            if (lane < take) e = W.leaf[nleaf - 1 - lane];
+            nleaf -= take;
+            const int slot = pool_slot(e);
+            const bool act = lane < take && pool_dist(e) <= W.thr[slot];
+            const float4 qs = W.q[slot];
+            const float3 p = xyz(qs);
+            const Traversal t = scene_of(slot);
+            int most = 1, cnt = act ? 1 : 0;
+            if constexpr (kRange) {
+                cnt = act ? pool_count(e) : 0;
+                most = (int)__reduce_max_sync(kFull, (unsigned)cnt);
+            }
+            for (int k = 0; k < most; ++k) {
+                const int leaf = pool_id(e) + k;
+                float d2 = INFINITY;
+                bool test = k < cnt;
+                if (test) {
+                    const float4 *tr = t.tris + 3 * (size_t)leaf;
+                    const float4 a = ldg4(tr), b = ldg4(tr + 1), c = ldg4(tr + 2);
+                    d2 = tri_distance2(p, xyz(a), xyz(b), xyz(c), b.w != 0.0f);
+                    atomicMin(&W.dmin[slot], __float_as_uint(d2));
+                }
+                __syncwarp();
+                if (test) {
+                    float w2, p2;
+                    windows(__uint_as_float(W.dmin[slot]), t.tau, qs.w, w2, p2);
+                    W.thr[slot] = fminf(W.thr[slot], p2);    // the same value from every lane of the slot
+                    if (d2 <= w2) {
+                        const int pos = atomicAdd(&W.cnt[slot], 1);
+                        if (pos < kPoolRing) W.ring[slot][pos] = make_uint2(__float_as_uint(d2), (unsigned)leaf);
+                    }
+                }
+                __syncwarp();
+                // a ring filling up drops the faces the window has left behind
+                if (lane < S) {
+                    const int m = W.cnt[lane];
+                    if (m > kPoolRing / 2 && m <= kPoolRing) {
+                        const Traversal tl = scene_of(lane);
+                        float w2, p2;
+                        windows(__uint_as_float(W.dmin[lane]), tl.tau, W.q[lane].w, w2, p2);
+                        int keep = 0;
+                        for (int j = 0; j < m; ++j) {
+                            const uint2 c = W.ring[lane][j];
+                            if (__uint_as_float(c.x) <= w2) W.ring[lane][keep++] = c;
+                        }
+                        W.cnt[lane] = keep;
+                    }
+                }
+                __syncwarp();
+            }
+            continue;
+        }
+        if (nstack == 0) break;
+        // ---- visit up to 32 nodes, one per lane; fewer when the stack is nearly full (its last
+        // kMaxTreeDepth entries are room for one entry's subtree taken depth first)
+        const int take = min(min(32, nstack), max(1, kStack - kMaxTreeDepth - nstack));
+        uint2 e = make_uint2(0u, 0u);
+        if (lane < take) e = W.stack[nstack - 1 - lane];
+        nstack -= take;
+        __syncwarp();
+        const int slot = pool_slot(e);
+        const float thr = W.thr[slot];
+        const bool act = lane < take && pool_dist(e) <= thr;
+        const float3 p = xyz(W.q[slot]);
+        int cn = 0, cf = 0, leaves = 0;                      // nearer and farther child; 1: left leaf, 2: right leaf
+        float dn = 0.0f, df = 0.0f, dl = 0.0f, dr = 0.0f;
+        int ll = 0, lr = 0, nl = 0, nr = 0;
+        bool pn = false, pf = false;
+        if (act) {
+            const Traversal t = scene_of(slot);
+            const float4 *r = t.nodes + 4 * (size_t)pool_id(e);
+            const float4 l0 = ldg4(r), l1 = ldg4(r + 1), r0 = ldg4(r + 2), r1 = ldg4(r + 3);
+            dl = box_d2(p, l0, l1);
+            dr = box_d2(p, r0, r1);
+            const int cl = __float_as_int(l0.w), cr = __float_as_int(r0.w);
+            const bool il = dl <= thr, ir = dr <= thr;
+            const bool gl = il && cl >= 0, gr = ir && cr >= 0;
+            leaves = (il && cl < 0 ? 1 : 0) | (ir && cr < 0 ? 2 : 0);
+            ll = -cl - 1;
+            lr = -cr - 1;
+            if constexpr (kRange) { nl = __float_as_int(l1.w) - 1; nr = __float_as_int(r1.w) - 1; }
+            const bool left = gl && (!gr || dl <= dr);
+            pn = gl || gr;
+            pf = gl && gr;
+            cn = left ? cl : cr;
+            dn = left ? dl : dr;
+            cf = left ? cr : cl;
+            df = left ? dr : dl;
+        }
+        const unsigned int bf = __ballot_sync(kFull, pf), bn = __ballot_sync(kFull, pn);
+        const unsigned int bl = __ballot_sync(kFull, leaves & 1), br = __ballot_sync(kFull, leaves & 2);
+        const int nf = __popc(bf), lf = __popc(bl);
+        if (pf) W.stack[nstack + __popc(bf & lt)] = pool_entry(cf, slot, 0, df);
+        if (pn) W.stack[nstack + nf + __popc(bn & lt)] = pool_entry(cn, slot, 0, dn);
+        if (leaves & 1) W.leaf[nleaf + __popc(bl & lt)] = pool_entry(ll, slot, nl, dl);
+        if (leaves & 2) W.leaf[nleaf + lf + __popc(br & lt)] = pool_entry(lr, slot, nr, dr);
+        nstack += nf + __popc(bn);
+        nleaf += lf + __popc(br);
+        __syncwarp();
+    }
+    // ---- each query's answer: the lowest id inside the final window
+    Hit h{-1, 0x7fffffff, INFINITY};
+    if (mine) {
+        const float m = __uint_as_float(W.dmin[lane]);
+        if (m <= maxd2) {
+            const Traversal t = scene_of(lane);
+            const int cnt = W.cnt[lane];
+            if (cnt > kPoolRing) {
+                Best B{-1, INFINITY, m, 0.0f, -1.0f};
+                resolve_ties(t, B, q, status);
+                h.leaf = B.leaf;
+                h.d2 = B.d2;
+            } else {
+                float w2, p2;
+                windows(m, t.tau, W.q[lane].w, w2, p2);
+                for (int j = 0; j < cnt; ++j) {
+                    const uint2 c = W.ring[lane][j];
+                    if (!(__uint_as_float(c.x) <= w2)) continue;
+                    const int f = face_of(t, (int)c.y);
+                    if (f < h.face) { h.face = f; h.leaf = (int)c.y; h.d2 = __uint_as_float(c.x); }
+                }
+            }
+            if (h.leaf >= 0 && cnt > kPoolRing) h.face = face_of(t, h.leaf);
+        }
+    }
+    return h;
+}
+
+// The queries of a warp: S consecutive ones.
+template <int S, bool kDeep, bool kRange>
+__global__ void __launch_bounds__(32 * kQueryWarps, 32 / kQueryWarps)
+k_pool_closest_point(Traversal T, const Header *__restrict__ hdr, unsigned int *status, const float *__restrict__ Q,
+                     int64_t nQ, float maxd2, int *face, float *bary, float *point, float *dist2, const int *hint,
+                     const int *__restrict__ iperm) {
+    __shared__ PoolWarp<S, kDeep> s_pool[kQueryWarps];
+    pdl_wait();
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t i0 = ((int64_t)blockIdx.x * kQueryWarps + wid) * S, i = i0 + lane;
+    if (i0 >= nQ) return;                                    // whole warp past the end
+    const bool valid = lane < S && i < nQ;
+    set_scale(T, hdr);
+    const float3 q = valid ? make_float3(Q[3 * i], Q[3 * i + 1], Q[3 * i + 2]) : make_float3(0.0f, 0.0f, 0.0f);
+    int hl = -1;
+    if (valid && hint) {                                     // may alias face: read before the write below
+        const int hf = hint[i];
+        if (hf >= 0 && hf < T.n) hl = __ldg(iperm + hf);
+    }
+    const Hit h = pool_search<S, kDeep, kRange, false>(T, s_pool[wid], nullptr, q, valid, maxd2, hl, T.mmd, status);
+    if (valid) write_hit(T, h, q, i, face, bary, point, dist2);
+}
+
+// Queries of many scenes (mesh_batch_closest_point): each lane finds its query's
+// scene, and the pool's entries carry scene-local nodes.
+template <int S, bool kDeep>
+__global__ void __launch_bounds__(32 * kQueryWarps, 32 / kQueryWarps)
+k_pool_batch(const float4 *__restrict__ nodes, const float4 *__restrict__ tris, const float4 *__restrict__ scene_box,
+             const int *__restrict__ face_off, const int *__restrict__ query_off, int nscenes,
+             const float *__restrict__ Q, int64_t nQ, float maxd2, bool mmd, int *face, float *bary, float *point,
+             float *dist2, unsigned int *status) {
+    __shared__ PoolWarp<S, kDeep> s_pool[kQueryWarps];
+    __shared__ PoolScene<S> s_scene[kQueryWarps];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t i0 = ((int64_t)blockIdx.x * kQueryWarps + wid) * S, i = i0 + lane;
+    if (i0 >= nQ) return;
+    const bool valid = lane < S && i < nQ;
+    Traversal T{nodes, tris, 0, 0.0f, 0.0f, mmd, nullptr};
+    float3 q = make_float3(0.0f, 0.0f, 0.0f);
+    int fb = 0;
+    if (valid) {
+        const int sc = segment_of(query_off, nscenes, i);
+        fb = __ldg(face_off + sc);
+        T.n = __ldg(face_off + sc + 1) - fb;
+        set_scale(T, scene_box[2 * sc], scene_box[2 * sc + 1]);
+        q = make_float3(Q[3 * i], Q[3 * i + 1], Q[3 * i + 2]);
+    }
+    if (lane < S) s_scene[wid].base[lane] = fb;
+    Hit h = pool_search<S, kDeep, false, true>(T, s_pool[wid], &s_scene[wid], q, valid, maxd2, -1, mmd, status);
+    if (!valid) return;
+    if (h.leaf >= 0) h.face -= fb;
+    T.tris += 3 * (size_t)fb;
+    write_hit(T, h, q, i, face, bary, point, dist2);
+}
+
+// ---------------------------------------------------------------------------
+// Chamfer (Sec. 4.2): both directions in one launch (blocks [0, nbA) query SA
+// against B, the rest SB against A).  Each block sums its squared distances in
+// float64 with a fixed reduction tree and stores the partial; the last block
+// to finish (ticket counter) adds the partials in a fixed order, writes the
+// two means and resets the counter, so the result is bit-reproducible.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ double block_sum_d(double x, double *s) {
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    if (lane == 0) s[w] = x;
+    __syncthreads();
+    double t = 0.0;
+    if (threadIdx.x == 0)
+        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += s[k];
+    __syncthreads();
+    return t;
+}
+
+template <int S, bool kRange>
+__global__ void __launch_bounds__(32 * kChamferWarps, 32 / kChamferWarps)
+k_pool_chamfer(ChamferSide A2B, ChamferSide B2A, unsigned int nbA, unsigned int *status, double *partial,
+               unsigned int *ticket, double *out) {
+    __shared__ PoolWarp<S, true> s_pool[kChamferWarps];
+    __shared__ double s_red[kChamferWarps];
+    __shared__ bool s_last;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const bool first = blockIdx.x < nbA;
+    const ChamferSide &C = first ? A2B : B2A;
+    const int64_t i0 = ((int64_t)(first ? blockIdx.x : blockIdx.x - nbA) * kChamferWarps + wid) * S, i = i0 + lane;
+    const bool valid = lane < S && i < C.n;
+    double d2 = 0.0;
+    if (i0 < C.n) {                                          // uniform in the warp
+        Traversal T = C.T;
+        set_scale(T, C.hdr);
+        const float3 q = valid ? make_float3(C.S[3 * i], C.S[3 * i + 1], C.S[3 * i + 2]) : make_float3(0.0f, 0.0f, 0.0f);
+        int hl = -1;
+        if (valid && C.hint) {
+            const int hf = C.hint[i];
+            if (hf >= 0 && hf < T.n) hl = __ldg(C.iperm + hf);
+        }
+        const Hit h = pool_search<S, true, kRange, false>(T, s_pool[wid], nullptr, q, valid, INFINITY, hl, true, status);
+        if (valid) {
+            write_hit(T, h, q, i, C.face, C.bary, nullptr, C.dist2);
+            d2 = h.leaf >= 0 ? (double)h.d2 : 0.0;
+        }
+    }
+    const double s = block_sum_d(d2, s_red);
+    if (threadIdx.x == 0) {
+        partial[blockIdx.x] = s;
+        __threadfence();
+        unsigned int t = atomicAdd(ticket, 1u);
+        s_last = (t == gridDim.x - 1);
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // fixed-order final sums: thread k adds partials k, k + blockDim, ... of each side
+    double a = 0.0, b = 0.0;
+    for (unsigned int k = threadIdx.x; k < nbA; k += blockDim.x) a += __ldcg(partial + k);
+    for (unsigned int k = nbA + threadIdx.x; k < gridDim.x; k += blockDim.x) b += __ldcg(partial + k);
+    a = block_sum_d(a, s_red);
+    b = block_sum_d(b, s_red);
+    if (threadIdx.x == 0) {
+        out[0] = A2B.n > 0 ? a / (double)A2B.n : 0.0;
+        out[1] = B2A.n > 0 ? b / (double)B2A.n : 0.0;
+        *ticket = 0u;
+    }
+}
+
+// Angle-weighted pseudo-normal of vertex vid (Baerentzen & Aanaes 2005): the
+// sum over the faces around it of the unit face normal times the face's angle
+// at the vertex.  The ring is found from face f through the face adjacency
+// (for a consistently oriented mesh, crossing the edge that follows the vertex
+// in each face turns one way round it; an open ring is also walked the other
+// way from f), up to kMaxRing faces, and summed in ascending face id, so the
+// result is the same whichever face the walk starts from and run to run.  A
+// ring larger than kMaxRing (or one the adjacency cannot close) sets
+// MESH_DEV_NONMANIFOLD and sums the faces found.
+constexpr int kMaxRing = 32;
+
+__device__ __forceinline__ int slot_of(int4 fv, int vid) {
+    return fv.x == vid ? 0 : (fv.y == vid ? 1 : (fv.z == vid ? 2 : -1));
+}
+
+__device__ __forceinline__ float4 vertex_pseudo_normal(const int4 *__restrict__ faces, const int *__restrict__ adj,
+                                                    const float4 *__restrict__ verts,
+                                                    const float4 *__restrict__ fnorm, int f, int vid,
+                                                    unsigned int *status) {
+    int ring[kMaxRing];
+    int nr = 0;
+    bool full = false;
+    int g = f;
+    while (true) {                                   // one way round
+        ring[nr++] = g;
+        int k = slot_of(faces[g], vid);
+        int h = k < 0 ? -1 : adj[3 * g + (k + 2) % 3];
+        if (h == f) break;
+        if (h < 0) break;
+        if (nr == kMaxRing) { full = true; break; }
+        g = h;
+    }
+    if (!full && nr < kMaxRing) {                     // open ring: the other way from f
+        int k0 = slot_of(faces[f], vid);
+        int h = k0 < 0 ? -1 : adj[3 * f + (k0 + 1) % 3];
+        bool closed = false;
+        for (int i = 0; i < nr; ++i) closed |= ring[i] == h;
+        while (h >= 0 && !closed) {
+            if (nr == kMaxRing) { full = true; break; }
+            ring[nr++] = h;
+            int k = slot_of(faces[h], vid);
+            int nh = k < 0 ? -1 : adj[3 * h + (k + 1) % 3];
+            for (int i = 0; i < nr; ++i) closed |= ring[i] == nh;
+            h = nh;
+        }
+    }
+    if (full) atomicOr(status, (unsigned)MESH_DEV_NONMANIFOLD);
+    float nx = 0.0f, ny = 0.0f, nz = 0.0f;
+    int last = -1;
+    for (int done = 0; done < nr; ++done) {          // ascending face id (distinct ids)
+        int pick = 0x7fffffff;
+        for (int i = 0; i < nr; ++i)
+            if (ring[i] > last && ring[i] < pick) pick = ring[i];
+        if (pick == 0x7fffffff) break;
+        last = pick;
+        int4 fv = faces[pick];
+        int k = slot_of(fv, vid);
+        if (k < 0) continue;
+        int id[3] = {fv.x, fv.y, fv.z};
+        float4 p = verts[id[k]], a = verts[id[(k + 1) % 3]], b = verts[id[(k + 2) % 3]];
+        float ax = a.x - p.x, ay = a.y - p.y, az = a.z - p.z;
+        float bx = b.x - p.x, by = b.y - p.y, bz = b.z - p.z;
+        float la = sqrtf(ax * ax + ay * ay + az * az), lb = sqrtf(bx * bx + by * by + bz * bz);
+        if (la == 0.0f || lb == 0.0f) continue;
+        float cs = fminf(1.0f, fmaxf(-1.0f, (ax * bx + ay * by + az * bz) / (la * lb)));
+        float ang = acosf(cs);
+        float4 n = fnorm[pick];
+        nx += ang * n.x; ny += ang * n.y; nz += ang * n.z;
+    }
+    return make_float4(nx, ny, nz, 0.0f);
+}
+
+// NearestSurface plus the sign of (q - c) . N, N the pseudo-normal of the
+// feature the nearest point lies on: face interior (no zero weight), edge
+// opposite vertex k (weight k zero), vertex (two zero weights).
+static __device__ __noinline__ float signed_of_hit(const Traversal &T, Hit h, float3 q, const int4 *__restrict__ faces,
+                                                   const int *__restrict__ adj, const float4 *__restrict__ fnorm,
+                                                   const float4 *__restrict__ verts, unsigned int *status) {
+    const float4 *t = T.tris + 3 * (size_t)h.leaf;
+    float4 a = ldg4(t), b = ldg4(t + 1), c = ldg4(t + 2);
+    float u, v, w;
+    tri_closest(q, xyz(a), xyz(b), xyz(c), b.w != 0.0f, u, v, w);
+    if (weights_need_f64(xyz(a), xyz(b), xyz(c), h.d2))
+        tri_weights_f64(q, xyz(a), xyz(b), xyz(c), b.w != 0.0f, u, v, w);
+    int f = h.face;
+    int zeros = (u == 0.0f) + (v == 0.0f) + (w == 0.0f);
+    float4 N;
+    if (zeros == 0) {
+        N = fnorm[f];
+    } else if (zeros == 1) {
+        int k = u == 0.0f ? 0 : (v == 0.0f ? 1 : 2);
+        N = fnorm[f];
+        int g = adj[3 * f + k];
+        if (g >= 0) { float4 m = fnorm[g]; N.x += m.x; N.y += m.y; N.z += m.z; }
+    } else {
+        int4 fv = faces[f];
+        int vid = u != 0.0f ? fv.x : (v != 0.0f ? fv.y : fv.z);
+        N = vertex_pseudo_normal(faces, adj, verts, fnorm, f, vid, status);
+    }
+    float cx = u * a.x + v * b.x + w * c.x, cy = u * a.y + v * b.y + w * c.y, cz = u * a.z + v * b.z + w * c.z;
+    float dn = (q.x - cx) * N.x + (q.y - cy) * N.y + (q.z - cz) * N.z;
+    return (dn >= 0.0f ? 1.0f : -1.0f) * sqrtf(h.d2);
+}
+
+template <int S, bool kDeep, bool kRange>
+__global__ void __launch_bounds__(32 * kQueryWarps, 32 / kQueryWarps)
+k_pool_signed(Traversal T, const Header *__restrict__ hdr, unsigned int *status, const float *__restrict__ Q,
+              int64_t nQ, float maxd2, const int4 *__restrict__ faces, const int *__restrict__ adj,
+              const float4 *__restrict__ fnorm, const float4 *__restrict__ verts, int *face, float *bary,
+              float *point, float *sdist) {
+    __shared__ PoolWarp<S, kDeep> s_pool[kQueryWarps];
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int64_t i0 = ((int64_t)blockIdx.x * kQueryWarps + wid) * S, i = i0 + lane;
+    if (i0 >= nQ) return;
+    const bool valid = lane < S && i < nQ;
+    set_scale(T, hdr);
+    const float3 q = valid ? make_float3(Q[3 * i], Q[3 * i + 1], Q[3 * i + 2]) : make_float3(0.0f, 0.0f, 0.0f);
+    const Hit h = pool_search<S, kDeep, kRange, false>(T, s_pool[wid], nullptr, q, valid, maxd2, -1, T.mmd, status);
+    if (!valid) return;
+    write_hit(T, h, q, i, face, bary, point, nullptr);
+    sdist[i] = h.leaf < 0 ? INFINITY : signed_of_hit(T, h, q, faces, adj, fnorm, verts, status);
+}
+
+// Calls f with S = 32 / G as a compile-time constant.
+template <typename F> static void pool_dispatch(int G, F f) {
+    switch (G) {
+        case 1: f(std::integral_constant<int, 32>()); break;
+        case 2: f(std::integral_constant<int, 16>()); break;
+        case 4: f(std::integral_constant<int, 8>()); break;
+        case 8: f(std::integral_constant<int, 4>()); break;
+        case 16: f(std::integral_constant<int, 2>()); break;
+        default: f(std::integral_constant<int, 1>()); break;
+    }
+}
+
+void pool_closest_point(const mesh_bvh *b, Traversal T, const float *Q, int64_t nQ, float maxd2, int G, int *face,
+                        float *bary, float *point, float *dist2, const int *hint, cudaStream_t s) {
+    Header *h = b->hdr();
+    pool_dispatch(G, [&](auto S) {
+        auto kern = b->leaf_size > 1 ? (T.mmd ? k_pool_closest_point<S.value, true, true>
+                                              : k_pool_closest_point<S.value, false, true>)
+                                     : (T.mmd ? k_pool_closest_point<S.value, true, false>
+                                              : k_pool_closest_point<S.value, false, false>);
+        kern<<<grid_for(nQ, kQueryWarps * S.value), 32 * kQueryWarps, 0, s>>>(T, h, &h->status, Q, nQ, maxd2, face, bary,
+                                                                       point, dist2, hint, b->iperm());
+    });
+    count_launch();
+}
+
+void pool_signed(const mesh_bvh *b, Traversal T, const float *Q, int64_t nQ, float maxd2, int G, int *face, float *bary,
+                 float *point, float *sdist, cudaStream_t s) {
+    Header *h = b->hdr();
+    pool_dispatch(G, [&](auto S) {
+        auto kern = b->leaf_size > 1 ? (T.mmd ? k_pool_signed<S.value, true, true> : k_pool_signed<S.value, false, true>)
+                                     : (T.mmd ? k_pool_signed<S.value, true, false> : k_pool_signed<S.value, false, false>);
+        kern<<<grid_for(nQ, kQueryWarps * S.value), 32 * kQueryWarps, 0, s>>>(T, h, &h->status, Q, nQ, maxd2, b->faces(),
+                                                                       b->adj(), b->fnorm(), b->verts(), face, bary,
+                                                                       point, sdist);
+    });
+    count_launch();
+}
+
+void pool_chamfer(int G, bool range, const ChamferSide &a2b, const ChamferSide &b2a, unsigned nbA, unsigned grid,
+                  unsigned *status, double *partial, unsigned *ticket, double *out, cudaStream_t s) {
+    pool_dispatch(G, [&](auto S) {
+        auto kern = range ? k_pool_chamfer<S.value, true> : k_pool_chamfer<S.value, false>;
+        kern<<<grid, 32 * kChamferWarps, 0, s>>>(a2b, b2a, nbA, status, partial, ticket, out);
+    });
+    count_launch();
+}
+
+void pool_batch(const mesh_batch *b, const float *Q, const int *query_off, int64_t nQ, float maxd2, bool mmd, int G,
+                int *face, float *bary, float *point, float *dist2, cudaStream_t s) {
+    pool_dispatch(G, [&](auto S) {
+        auto kern = mmd ? k_pool_batch<S.value, true> : k_pool_batch<S.value, false>;
+        kern<<<grid_for(nQ, kQueryWarps * S.value), 32 * kQueryWarps, 0, s>>>(
+            b->nodes(), b->tris(), b->scene_box(), b->face_off(), query_off, (int)b->L.n_scenes, Q, nQ, maxd2, mmd,
+            face, bary, point, dist2, &b->st()->status);
+    });
+    count_launch();
+}
+
+}  // namespace meshgs

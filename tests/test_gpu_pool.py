@@ -1,0 +1,102 @@
+"""The pooled search (traversal variant 0, and every width of several lanes per query)
+against the one-thread search of the same queries: bit for bit, at the edges of its
+warps, with its stack nearly full and with more tied faces than a query records."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2606_00444_gb300 import MeshBatch, MeshBVH
+from parity import assert_identical, dev
+from workloads.meshes import displaced_icosphere, icosphere
+from workloads.sampling import uniform_box
+
+pytestmark = pytest.mark.gpu
+
+LANES = [1, 2, 4, 8, 16, 32]
+
+
+def one_thread(bvh, Q, md, hint=None):
+    bvh.set_query_config(1, 2)
+    out = bvh.closest_point(Q, md, hint=hint)
+    bvh.set_query_config(-1, -1)
+    return out
+
+
+def pooled(bvh, Q, md, lanes, hint=None):
+    bvh.set_query_config(lanes, 0)
+    out = bvh.closest_point(Q, md, hint=hint)
+    bvh.set_query_config(-1, -1)
+    return out
+
+
+@pytest.mark.parametrize("lanes", LANES)
+@pytest.mark.parametrize("faces", [1, 2, 3, 1280])
+def test_ragged_query_counts(lanes, faces):
+    V, F = displaced_icosphere(3, 0.1, 0.4)
+    F = np.ascontiguousarray(F[:faces])
+    bvh = MeshBVH.from_mesh(dev(V), dev(F))
+    S = 32 // lanes
+    for n in sorted({1, S - 1, S, S + 1, 3 * S + 1, 67}):
+        if n < 1:
+            continue
+        Q = dev(uniform_box(n, [-1.5] * 3, [1.5] * 3, seed=n))
+        for md in (float("inf"), 0.3, 0.0):
+            ref = one_thread(bvh, Q, md)
+            assert_identical(pooled(bvh, Q, md, lanes), ref)
+            assert_identical(pooled(bvh, Q, md, lanes, hint=ref["face"]), ref)
+    assert bvh.status()[0] == 0
+
+
+@pytest.mark.parametrize("method", ["lbvh", "ploc"])
+@pytest.mark.parametrize("lanes", LANES)
+def test_deep_searches_with_the_stack_nearly_full(lanes, method):
+    """Queries about the centre of a sphere: every face is nearly equally near, so each
+    search defers a sibling at almost every level of the tree."""
+    V, F = icosphere(5)
+    bvh = MeshBVH.from_mesh(dev(V), dev(F), method=method)
+    rng = np.random.default_rng(5)
+    Q = dev((rng.normal(size=(64, 3)) * 1e-3).astype(np.float32))
+    ref = one_thread(bvh, Q, float("inf"))
+    assert_identical(pooled(bvh, Q, float("inf"), lanes), ref)
+    ref = one_thread(bvh, Q, 1.5)                         # a cutoff that prunes nothing: the shallow stacks
+    assert_identical(pooled(bvh, Q, 1.5, lanes), ref)
+    assert bvh.status()[0] == 0
+
+
+@pytest.mark.parametrize("lanes", LANES)
+@pytest.mark.parametrize("leaf", [1, 4])
+def test_more_tied_faces_than_a_query_records(lanes, leaf):
+    """A fan of 40 faces around one vertex, queried at and above it, and a stack of 40
+    copies of one face: all are at the same distance, the lowest id wins."""
+    t = np.linspace(0, 2 * np.pi, 40, endpoint=False)
+    V = np.concatenate([[[0, 0, 1]], np.stack([np.cos(t), np.sin(t), 0 * t], 1)]).astype(np.float32)
+    i = np.arange(40)
+    fan = np.stack([0 * i, 1 + i, 1 + (i + 1) % 40], 1).astype(np.int32)
+    rng = np.random.default_rng(1)
+    for F in (fan[rng.permutation(40)], np.repeat(fan[:1], 40, 0)):
+        bvh = MeshBVH.from_mesh(dev(V), dev(np.ascontiguousarray(F)))
+        bvh.set_leaf_size(leaf)
+        Q = dev(np.array([[0, 0, 1], [0, 0, 2], [0, 0, 1.001], [0.1, 0.2, 3]], np.float32))
+        for md in (float("inf"), 2.5):
+            assert_identical(pooled(bvh, Q, md, lanes), one_thread(bvh, Q, md))
+        assert int(pooled(bvh, Q, float("inf"), lanes)["face"][1]) == 0
+        assert bvh.status()[0] == 0
+
+
+def test_batch_warps_that_span_scenes():
+    """Scenes of a few queries each, some with no faces: one warp holds queries of many."""
+    rng = np.random.default_rng(9)
+    meshes, qs = [], []
+    for k in range(23):
+        V, F = displaced_icosphere(int(rng.integers(0, 4)), 0.1, 0.1 * k)
+        V = (V * rng.uniform(0.1, 50.0)).astype(np.float32)
+        F = F[:[0, 1, 2, len(F)][k % 4]]
+        meshes.append((V, np.ascontiguousarray(F)))
+        qs.append(uniform_box(int(rng.integers(0, 9)), V.min(0) * 1.2, V.max(0) * 1.2, seed=k))
+    batch = MeshBatch.from_meshes(meshes)
+    off = dev(np.concatenate([[0], np.cumsum([len(q) for q in qs])]).astype(np.int32))
+    for md in (float("inf"), 0.5):
+        got = batch.closest_point(dev(np.concatenate(qs)), off, md)
+        ref = [one_thread(MeshBVH.from_mesh(dev(v), dev(f)), dev(q), md) for (v, f), q in zip(meshes, qs) if len(q)]
+        assert_identical(got, {k: torch.cat([r[k] for r in ref]) for k in ref[0]})
+    assert batch.status()[0] == 0
