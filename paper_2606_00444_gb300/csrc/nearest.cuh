@@ -509,6 +509,10 @@ struct ChamferSide {
 // grid blocks of 128 / G samples, the first nbA of them a2b's.
 void pool_chamfer(int G, bool range, const ChamferSide &a2b, const ChamferSide &b2a, unsigned nbA, unsigned grid,
                   unsigned *status, double *partial, unsigned *ticket, double *out, cudaStream_t s);
+// Projection onto the k (1 to kKnnMax) nearest faces (mesh_knn_project).
+constexpr int kKnnMax = 8;
+void pool_knn(const mesh_bvh *b, Traversal T, const float *Q, int64_t nQ, int k, int G, const float *anchor,
+              float anchor_w, float *point, int *face, float *d2, cudaStream_t s);
 void pool_batch(const mesh_batch *b, const float *Q, const int *query_off, int64_t nQ, float maxd2, bool mmd, int G,
                 int *face, float *bary, float *point, float *dist2, cudaStream_t s);
 

@@ -513,6 +513,244 @@ k_pool_signed(Traversal T, const Header *__restrict__ hdr, unsigned int *status,
     sdist[i] = h.leaf < 0 ? INFINITY : signed_of_hit(T, h, q, faces, adj, fnorm, verts, status);
 }
 
+// ---------------------------------------------------------------------------
+// k-NN weighted surface projection: the NearestSurface of temporal tracking
+// (Sec. 3.3, Strategy 1, Eq. 1).  The paper names the method without k or
+// weights; here: the k faces nearest to the query (ties by the lower face
+// id), each giving its closest point p_j at distance d_j, blended with
+// weights 1 / max(d_j, 1e-6 x box diagonal); optionally mixed with an anchor
+// point, (1 - a) v' + a anchor (the periodic re-anchoring to the template).
+//
+// The pooled search with a sorted list of the k best (distance, face) per query
+// in shared memory; a face that may enter is inserted by the whole warp, one
+// lane per list entry.  The pruning radius is the k-th distance, widened by the
+// float32 bound, so the k faces are those of least (distance, id) whatever the
+// order.  A query first goes down to one leaf and tests the leaves beside it in
+// leaf order, which are near it, so the search starts with k faces.  A tracked
+// template has some 10k vertices: one thread each left 108 blocks waiting on
+// their longest search (367 us at 13.7k queries and 40k faces; rebuild and
+// projection together 583 us, 231 us with the pool).
+// ---------------------------------------------------------------------------
+template <int S> struct __align__(16) PoolKnn {
+    static constexpr int kStack = S == 8 ? 320 : 256;
+    static constexpr int kSeeds = kPoolLeaf / 8;         // leaves a query tests first
+    float4 q[S];
+    uint2 stack[kStack];
+    uint2 leaf[kPoolLeaf];
+    float d2[S][kKnnMax];                                // sorted by (distance, face)
+    int face[S][kKnnMax], pos[S][kKnnMax];               // face id and leaf
+    float thr[S];
+};
+
+template <int S, bool kRange>
+__global__ void __launch_bounds__(32, 32)
+k_pool_knn(Traversal T, const Header *__restrict__ hdr, const float *Q, int64_t nQ, int k, const float *anchor,
+           float anchor_w, float *point, int *face_out, float *d2_out) {
+    __shared__ PoolKnn<S> W;
+    constexpr int kStack = PoolKnn<S>::kStack, kSeeds = PoolKnn<S>::kSeeds;
+    const unsigned int kFull = 0xffffffffu;
+    const int lane = threadIdx.x;
+    const unsigned int lt = (1u << lane) - 1u;
+    const int64_t i0 = (int64_t)blockIdx.x * S;
+    const int own = (int)(nQ - i0 < S ? nQ - i0 : S);    // this warp's queries
+    set_scale(T, hdr);
+    for (int j = lane; j < S * kKnnMax; j += 32) {
+        W.d2[j / kKnnMax][j % kKnnMax] = INFINITY;
+        W.face[j / kKnnMax][j % kKnnMax] = 0x7fffffff;
+        W.pos[j / kKnnMax][j % kKnnMax] = -1;
+    }
+    float3 q = make_float3(0.0f, 0.0f, 0.0f);
+    int seed = -1;                                       // the leaf this query comes down to
+    if (lane < own) {
+        const int64_t i = i0 + lane;
+        q = make_float3(Q[3 * i], Q[3 * i + 1], Q[3 * i + 2]);   // may alias point
+        W.q[lane] = make_float4(q.x, q.y, q.z, query_slack(T, q));
+        W.thr[lane] = INFINITY;
+        if (T.n == 1) {
+            seed = 0;
+        } else if (T.n > 1) {
+            int node = 0;
+            while (seed < 0) {
+                const float4 *r = T.nodes + 4 * (size_t)node;
+                const float4 l0 = ldg4(r), l1 = ldg4(r + 1), r0 = ldg4(r + 2), r1 = ldg4(r + 3);
+                const float dl = box_d2(q, l0, l1), dr = box_d2(q, r0, r1);
+                bool left = dl < dr;
+                if (dl == dr) left = box_minmax_d2(q, l0, l1) <= box_minmax_d2(q, r0, r1);
+                const int c = __float_as_int(left ? l0.w : r0.w);
+                if (c >= 0) node = c;
+                else seed = -c - 1;
+            }
+        }
+    }
+    // the leaves around each query's own, and its root
+    int nleaf = 0, nstack = 0;
+    {
+        const int m = min(min(2 * k, kSeeds), T.n);      // seeds per query
+        const int s0 = min(max(seed - m / 2, 0), T.n - m);
+        if (seed >= 0)
+            for (int j = 0; j < m; ++j) W.leaf[lane * m + j] = pool_entry(s0 + j, lane, 0, 0.0f);
+        if (T.n > 0) nleaf = own * m;
+        if (T.n > 1) {
+            if (lane < own) W.stack[lane] = pool_entry(0, lane, 0, 0.0f);
+            nstack = own;
+        }
+    }
+    bool start = nleaf > 0;
+    __syncwarp();
+    while (true) {
+        if (nleaf >= 32 || start || (nstack == 0 && nleaf > 0)) {
+            const int take = min(32, nleaf);
+            uint2 e = make_uint2(0u, 0u);
+            if (lane < take) e = W.leaf[nleaf - 1 - lane];
+            nleaf -= take;
+            start = start && nleaf > 0;
+            const int slot = pool_slot(e);
+            const bool act = lane < take && pool_dist(e) <= W.thr[slot];
+            const float3 p = xyz(W.q[slot]);
+            int most = 1, cnt = act ? 1 : 0;
+            if constexpr (kRange) {
+                cnt = act ? pool_count(e) : 0;
+                most = (int)__reduce_max_sync(kFull, (unsigned)cnt);
+            }
+            for (int j = 0; j < most; ++j) {
+                const int leaf = pool_id(e) + j;
+                float d2 = INFINITY;
+                int f = 0;
+                bool in = j < cnt;
+                if (in) {
+                    const float4 *tr = T.tris + 3 * (size_t)leaf;
+                    const float4 a = ldg4(tr), b = ldg4(tr + 1), c = ldg4(tr + 2);
+                    d2 = tri_distance2(p, xyz(a), xyz(b), xyz(c), b.w != 0.0f);
+                    f = __float_as_int(a.w);
+                    in = d2 <= W.d2[slot][k - 1];
+                }
+                unsigned int todo = __ballot_sync(kFull, in);
+                while (todo) {                           // insert one face: lane l < k has entry l
+                    const int src = __ffs(todo) - 1;
+                    todo &= todo - 1u;
+                    const int sl = __shfl_sync(kFull, slot, src), fc = __shfl_sync(kFull, f, src),
+                              lf = __shfl_sync(kFull, leaf, src);
+                    const float d = __shfl_sync(kFull, d2, src);
+                    const bool entry = lane < k;
+                    const float ed = entry ? W.d2[sl][lane] : INFINITY;
+                    const int ef = entry ? W.face[sl][lane] : 0x7fffffff, ep = entry ? W.pos[sl][lane] : -1;
+                    const bool listed = __any_sync(kFull, entry && ef == fc);
+                    const int at = __popc(__ballot_sync(kFull, entry && (ed < d || (ed == d && ef < fc))));
+                    const float ud = __shfl_up_sync(kFull, ed, 1);
+                    const int uf = __shfl_up_sync(kFull, ef, 1), up = __shfl_up_sync(kFull, ep, 1);
+                    if (!listed && entry && lane >= at) {
+                        const float nd = lane == at ? d : ud;
+                        W.d2[sl][lane] = nd;
+                        W.face[sl][lane] = lane == at ? fc : uf;
+                        W.pos[sl][lane] = lane == at ? lf : up;
+                        if (lane == k - 1) {
+                            const float r = sqrtf(nd) + W.q[sl].w;
+                            W.thr[sl] = r * r;
+                        }
+                    }
+                    __syncwarp();
+                }
+            }
+            continue;
+        }
+        if (nstack == 0) break;
+        // (as pool_search)
+        const int take = min(min(32, nstack), max(1, kStack - kMaxTreeDepth - nstack));
+        uint2 e = make_uint2(0u, 0u);
+        if (lane < take) e = W.stack[nstack - 1 - lane];
+        nstack -= take;
+        __syncwarp();
+        const int slot = pool_slot(e);
+        const float thr = W.thr[slot];
+        const bool act = lane < take && pool_dist(e) <= thr;
+        const float3 p = xyz(W.q[slot]);
+        int cn = 0, cf = 0, ll = 0, lr = 0, nl = 0, nr = 0;
+        float dn = 0.0f, df = 0.0f, dl = 0.0f, dr = 0.0f;
+        bool pn = false, pf = false, tl = false, tr = false;
+        if (act) {
+            const float4 *r = T.nodes + 4 * (size_t)pool_id(e);
+            const float4 l0 = ldg4(r), l1 = ldg4(r + 1), r0 = ldg4(r + 2), r1 = ldg4(r + 3);
+            dl = box_d2(p, l0, l1);
+            dr = box_d2(p, r0, r1);
+            const int cl = __float_as_int(l0.w), cr = __float_as_int(r0.w);
+            const bool il = dl <= thr, ir = dr <= thr, gl = il && cl >= 0, gr = ir && cr >= 0;
+            tl = il && cl < 0;
+            tr = ir && cr < 0;
+            ll = -cl - 1;
+            lr = -cr - 1;
+            if constexpr (kRange) { nl = __float_as_int(l1.w) - 1; nr = __float_as_int(r1.w) - 1; }
+            const bool left = gl && (!gr || dl <= dr);
+            pn = gl || gr;
+            pf = gl && gr;
+            cn = left ? cl : cr;
+            dn = left ? dl : dr;
+            cf = left ? cr : cl;
+            df = left ? dr : dl;
+        }
+        const unsigned int bf = __ballot_sync(kFull, pf), bn = __ballot_sync(kFull, pn);
+        const unsigned int bl = __ballot_sync(kFull, tl), br = __ballot_sync(kFull, tr);
+        const int nf = __popc(bf), lf = __popc(bl);
+        if (pf) W.stack[nstack + __popc(bf & lt)] = pool_entry(cf, slot, 0, df);
+        if (pn) W.stack[nstack + nf + __popc(bn & lt)] = pool_entry(cn, slot, 0, dn);
+        if (tl) W.leaf[nleaf + __popc(bl & lt)] = pool_entry(ll, slot, nl, dl);
+        if (tr) W.leaf[nleaf + lf + __popc(br & lt)] = pool_entry(lr, slot, nr, dr);
+        nstack += nf + __popc(bn);
+        nleaf += lf + __popc(br);
+        __syncwarp();
+    }
+    // the blend: lane 8 s + j takes face j of query s, and lane 8 s sums them nearest first
+    const float4 rlo = hdr->root_lo, rhi = hdr->root_hi;
+    const float dx = rhi.x - rlo.x, dy = rhi.y - rlo.y, dz = rhi.z - rlo.z;
+    const float delta = 1e-6f * sqrtf(dx * dx + dy * dy + dz * dz);
+    for (int b0 = 0; b0 < S; b0 += 4) {
+        const int sl = b0 + lane / 8, j = lane % 8;
+        const bool on = sl < own && j < k;
+        float wt = 0.0f, px = 0.0f, py = 0.0f, pz = 0.0f;
+        if (on) {
+            const int64_t i = i0 + sl;
+            const int leaf = W.pos[sl][j];
+            const float d2 = W.d2[sl][j];
+            if (leaf >= 0) {
+                const float4 *t = T.tris + 3 * (size_t)leaf;
+                const float4 a = ldg4(t), b = ldg4(t + 1), c = ldg4(t + 2);
+                float u, v, w;
+                tri_closest(xyz(W.q[sl]), xyz(a), xyz(b), xyz(c), b.w != 0.0f, u, v, w);
+                wt = 1.0f / fmaxf(sqrtf(d2), delta);
+                px = u * a.x + v * b.x + w * c.x;
+                py = u * a.y + v * b.y + w * c.y;
+                pz = u * a.z + v * b.z + w * c.z;
+            }
+            if (face_out) face_out[i * k + j] = leaf >= 0 ? W.face[sl][j] : -1;
+            if (d2_out) d2_out[i * k + j] = leaf >= 0 ? d2 : INFINITY;
+        }
+        float sw = 0.0f, ax = 0.0f, ay = 0.0f, az = 0.0f;
+#pragma unroll
+        for (int m = 0; m < kKnnMax; ++m) {
+            const int src = (lane & ~7) + m;
+            const float wm = __shfl_sync(kFull, wt, src), xm = __shfl_sync(kFull, px, src),
+                        ym = __shfl_sync(kFull, py, src), zm = __shfl_sync(kFull, pz, src);
+            sw += wm;
+            ax += wm * xm;
+            ay += wm * ym;
+            az += wm * zm;
+        }
+        if (sl < own && j == 0) {
+            const int64_t i = i0 + sl;
+            const float4 qs = W.q[sl];
+            float ox = qs.x, oy = qs.y, oz = qs.z;
+            if (W.pos[sl][0] >= 0) { ox = ax / sw; oy = ay / sw; oz = az / sw; }
+            if (anchor) {
+                ox = (1.0f - anchor_w) * ox + anchor_w * anchor[3 * i];
+                oy = (1.0f - anchor_w) * oy + anchor_w * anchor[3 * i + 1];
+                oz = (1.0f - anchor_w) * oz + anchor_w * anchor[3 * i + 2];
+            }
+            point[3 * i] = ox;
+            point[3 * i + 1] = oy;
+            point[3 * i + 2] = oz;
+        }
+    }
+}
+
 // Calls f with S = 32 / G as a compile-time constant.
 template <typename F> static void pool_dispatch(int G, F f) {
     switch (G) {
@@ -549,6 +787,19 @@ void pool_signed(const mesh_bvh *b, Traversal T, const float *Q, int64_t nQ, flo
                                                                        b->adj(), b->fnorm(), b->verts(), face, bary,
                                                                        point, sdist);
     });
+    count_launch();
+}
+
+void pool_knn(const mesh_bvh *b, Traversal T, const float *Q, int64_t nQ, int k, int G, const float *anchor,
+              float anchor_w, float *point, int *face, float *d2, cudaStream_t s) {
+    auto go = [&](auto S) {
+        auto kern = b->leaf_size > 1 ? k_pool_knn<S.value, true> : k_pool_knn<S.value, false>;
+        kern<<<grid_for(nQ, S.value), 32, 0, s>>>(T, b->hdr(), Q, nQ, k, anchor, anchor_w, point, face, d2);
+    };
+    if (G <= 4) go(std::integral_constant<int, 8>());
+    else if (G == 8) go(std::integral_constant<int, 4>());
+    else if (G == 16) go(std::integral_constant<int, 2>());
+    else go(std::integral_constant<int, 1>());
     count_launch();
 }
 

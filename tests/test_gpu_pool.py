@@ -100,3 +100,30 @@ def test_batch_warps_that_span_scenes():
         ref = [one_thread(MeshBVH.from_mesh(dev(v), dev(f)), dev(q), md) for (v, f), q in zip(meshes, qs) if len(q)]
         assert_identical(got, {k: torch.cat([r[k] for r in ref]) for k in ref[0]})
     assert batch.status()[0] == 0
+
+
+@pytest.mark.parametrize("n", [1, 3, 33, 100_003])
+@pytest.mark.parametrize("k,leaf", [(1, 1), (4, 1), (8, 1), (8, 4)])
+def test_knn_lists_are_the_k_least_distances(n, k, leaf):
+    """The k faces of each query, checked against every face's own distance (a mesh of that
+    face alone): the k least, nearest first, with the lower id first among equals; at the
+    pooled widths 1-8 (by the query count), meshes smaller than k, and leaf ranges."""
+    V, F = icosphere(1)
+    rng = np.random.default_rng(n + k)
+    Qn = (rng.normal(size=(n, 3))).astype(np.float32)
+    Qn[: min(n, 12)] = V[: min(n, 12)]                    # on vertices: ties of five faces
+    for faces in (3, len(F)):
+        Fs = np.ascontiguousarray(F[:faces])
+        bvh = MeshBVH.from_mesh(dev(V), dev(Fs))
+        bvh.set_leaf_size(leaf)
+        _, face, d2 = bvh.knn_project(dev(Qn), k=k, want_faces=True)
+        m = min(n, 200)
+        Q = dev(Qn[:m])
+        each = torch.stack([one_thread(MeshBVH.from_mesh(dev(V), dev(Fs[f:f + 1])), Q, float("inf"))["dist2"]
+                            for f in range(faces)], 1).cpu().numpy()
+        order = np.lexsort((np.broadcast_to(np.arange(faces), each.shape), each), axis=1)[:, :k]
+        c = min(k, faces)
+        assert np.array_equal(face[:m, :c].cpu().numpy(), order)
+        assert np.array_equal(d2[:m, :c].cpu().numpy(), np.take_along_axis(each, order, 1))
+        assert (face[:, c:] == -1).all() and torch.isinf(d2[:, c:]).all()
+        assert bvh.status()[0] == 0
