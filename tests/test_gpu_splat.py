@@ -166,3 +166,29 @@ def test_fixed_capacity_render_is_the_render_and_replays_in_a_graph():
     gs_render_capacity(mu, q, sc, op, col, R, t, f, f, W / 2, H / 2, W, H, small, counts=counts)
     torch.cuda.synchronize()
     assert counts[0].item() == 1 and counts[1].item() > small
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 64, 65, 97, 129])
+def test_instance_counts_at_the_edges_of_a_warps_fetches(n):
+    """n Gaussians over one tile: the compositing takes them 32 at a time and fetches two
+    steps ahead."""
+    rng = np.random.default_rng(n)
+    mu = np.stack([rng.uniform(-0.3, 0.3, n), rng.uniform(-0.3, 0.3, n), 2 + 0.02 * np.arange(n)], 1)
+    quat = np.tile([1.0, 0, 0, 0], (n, 1))
+    scale = rng.uniform(0.05, 0.3, (n, 3))
+    args = (mu[rng.permutation(n)], quat, scale, np.full(n, 0.03), rng.uniform(0, 1, (n, 3)))
+    compare(args, (np.eye(3), np.zeros(3), 20.0), 16, 16)
+
+
+@pytest.mark.parametrize("w,h", [(1, 1), (7, 3), (8, 4), (9, 5), (16, 16), (17, 33), (33, 17)])
+def test_small_images_are_crops_of_larger_ones(w, h):
+    """A pixel's value does not depend on the image's size: every warp's pixels, inside the
+    image or partly past its edge."""
+    rng = np.random.default_rng(7)
+    n = 400
+    a = [dev(np.asarray(x, np.float32)) for x in
+         (rng.uniform(-1, 1, (n, 3)) + [0, 0, 3], rng.normal(size=(n, 4)), rng.uniform(0.02, 0.2, (n, 3)),
+          rng.uniform(0.2, 0.9, n), rng.uniform(0, 1, (n, 3)))]
+    big = gs_render(*a, np.eye(3), np.zeros(3), 30.0, 30.0, 12.0, 10.0, 48, 48)
+    img = gs_render(*a, np.eye(3), np.zeros(3), 30.0, 30.0, 12.0, 10.0, w, h)
+    assert torch.equal(img[0], big[0][:h, :w]) and torch.equal(img[1], big[1][:h, :w])
