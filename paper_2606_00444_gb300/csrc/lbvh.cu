@@ -28,13 +28,10 @@ mesh_status check_launch() {
 }
 
 constexpr int kBlock = 256;
-constexpr int kSortThreads = 256;
-constexpr int kSortItems = 4;
-constexpr int kSortTile = kSortThreads * kSortItems;   // keys per sort tile
-constexpr int kSortWarps = kSortThreads / 32;
 constexpr int kRadix = 256;
+constexpr int kSortTileMin = 1024;    // keys per sort tile: 1024, 2048, 4096 or 8192 (sort_shape)
+constexpr int kSortTilesMax = 512;    // tiles whose counts a pass sums itself
 constexpr int kScanThreads = 256;     // one block per digit; also scans the 256 digit totals
-static_assert(kSortThreads == kRadix, "one thread per digit in the sort kernels");
 
 // ---------------------------------------------------------------------------
 // Float <-> order-preserving unsigned encoding, so box extremes can be reduced
@@ -50,11 +47,13 @@ __device__ __forceinline__ float ord2f(unsigned int u) {
 
 // ---------------------------------------------------------------------------
 // a1: vertex-buffer update, [nV][3] -> float4 [nV] (w = 0).
-// Optionally (re)initialises the 6-word centroid box used by the Morton step.
+// Optionally (re)initialises the 6-word centroid box used by the Morton step and
+// the header (a build).
 // ---------------------------------------------------------------------------
 __global__ void k_copy_verts(const float *__restrict__ V3, int nV, float4 *__restrict__ V4,
-                             unsigned int *__restrict__ cbox) {
+                             unsigned int *__restrict__ cbox, Header *__restrict__ hdr = nullptr) {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (hdr && i < (int)(sizeof(Header) / 4)) reinterpret_cast<unsigned int *>(hdr)[i] = 0u;
     if (cbox && i < 6) cbox[i] = (i < 3) ? 0xffffffffu : 0u;
     if (i >= nV) return;
     const float *p = V3 + 3 * (size_t)i;
@@ -177,66 +176,106 @@ __device__ __forceinline__ unsigned int spread3(unsigned int v) {
 }
 
 // ---------------------------------------------------------------------------
+// a3: stable LSD radix sort of (key, face id), 8 bits per pass, one kernel per
+// pass and no inter-block waiting of any kind.  hist[t * 256 + d] counts digit d
+// in tile t of the pass's input.
+//   k_sort_hist:  the first pass's counts (the build's k_morton counts them as it
+//                 makes the keys); also clears the later passes' counts
+//   k_sort_pass:  a block per tile sums the tiles' counts of every digit -- all of
+//                 them for the digit's base, those of earlier tiles for its own
+//                 offset -- ranks its keys (warp match_any + per-warp counters),
+//                 scatters them through shared memory, writes them out
+//                 coalesced, and adds each to the next pass's counts, whose tile
+//                 its output position gives.
+// A pass was three kernels (counts, a scan of 256 x tiles counts, scatter): at 200k
+// keys 13.6 us and three launch gaps each against 9 us and one (the rebuild 137 ->
+// 98 us); tiles grow with n so that their counts
+// stay few enough to sum in every block.  Past kSortTilesMax tiles k_sort_scan
+// turns them into offsets first (a block's sum of the counts would read more
+// than its keys).
+// ---------------------------------------------------------------------------
+// Adds a key's digit to its block's 256 counters h (one block per tile).
+__device__ __forceinline__ void sort_count(unsigned int *h, bool valid, unsigned int digit) {
+    const unsigned int d = valid ? digit : 0x100u;
+    const unsigned int peers = __match_any_sync(0xffffffffu, d);
+    if (valid && (__ffs(peers) - 1) == (int)(threadIdx.x & 31)) atomicAdd(&h[d], (unsigned)__popc(peers));
+}
+
+struct SortHist {
+    unsigned int *first, *rest;        // counts of the first pass; of the later ones, T * 256 apart
+    int T;                             // tiles; with one, no counts are kept
+    int passes;
+};
+
+__device__ __forceinline__ void sort_put_counts(const SortHist &H, const unsigned int *h, int threads) {
+    if (H.T == 1) return;
+    for (int d = threadIdx.x; d < kRadix; d += threads) {
+        H.first[(size_t)blockIdx.x * kRadix + d] = h[d];
+        for (int p = 0; p + 1 < H.passes; ++p) H.rest[((size_t)p * H.T + blockIdx.x) * kRadix + d] = 0u;
+    }
+}
+
+// ---------------------------------------------------------------------------
 // a2: 30-bit Morton key per face.  t = (s - lo) * (1 / (hi - lo)) per axis,
 // q = clamp(floor(t * 1024), 0, 1023), bits interleaved x-major.  Every
 // float operation is an explicit round-to-nearest intrinsic so no FMA
-// contraction can change a key.
+// contraction can change a key.  A block makes the keys of one sort tile and
+// counts their first digit.
 // ---------------------------------------------------------------------------
-__global__ void k_morton(const float4 *__restrict__ cent, int nF,
-                         const unsigned int *__restrict__ cbox, unsigned int *__restrict__ keys,
-                         int *__restrict__ vals) {
-    int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= nF) return;
+template <int kThreads, int kItems>
+__global__ void __launch_bounds__(kThreads)
+k_morton(const float4 *__restrict__ cent, int nF, const unsigned int *__restrict__ cbox,
+         unsigned int *__restrict__ keys, unsigned int *__restrict__ counts, int T) {
+    __shared__ unsigned int h[kRadix];
+    pdl_wait();
+    for (int d = threadIdx.x; d < kRadix; d += kThreads) h[d] = 0u;
+    __syncthreads();
     float lo[3], inv[3];
     for (int k = 0; k < 3; ++k) {
         lo[k] = ord2f(cbox[k]);
         float ext = __fsub_rn(ord2f(cbox[3 + k]), lo[k]);
         inv[k] = ext > 0.0f ? __fdiv_rn(1.0f, ext) : 0.0f;
     }
-    float4 s = cent[f];
-    float sv[3] = {s.x, s.y, s.z};
-    unsigned int q[3];
-    for (int k = 0; k < 3; ++k) {
-        float t = __fmul_rn(__fsub_rn(sv[k], lo[k]), inv[k]);
-        float x = floorf(__fmul_rn(t, 1024.0f));
-        int qi = (int)x;
-        qi = qi < 0 ? 0 : (qi > 1023 ? 1023 : qi);
-        q[k] = (unsigned int)qi;
+#pragma unroll
+    for (int r = 0; r < kItems; ++r) {
+        const int f = blockIdx.x * (kThreads * kItems) + r * kThreads + threadIdx.x;
+        unsigned int key = 0u;
+        if (f < nF) {
+            float4 s = cent[f];
+            float sv[3] = {s.x, s.y, s.z};
+            unsigned int q[3];
+            for (int k = 0; k < 3; ++k) {
+                float t = __fmul_rn(__fsub_rn(sv[k], lo[k]), inv[k]);
+                float x = floorf(__fmul_rn(t, 1024.0f));
+                int qi = (int)x;
+                qi = qi < 0 ? 0 : (qi > 1023 ? 1023 : qi);
+                q[k] = (unsigned int)qi;
+            }
+            key = (spread3(q[0]) << 2) | (spread3(q[1]) << 1) | spread3(q[2]);
+            keys[f] = key;
+        }
+        sort_count(h, f < nF, key & 0xffu);
     }
-    keys[f] = (spread3(q[0]) << 2) | (spread3(q[1]) << 1) | spread3(q[2]);
-    vals[f] = f;
+    __syncthreads();
+    if (T > 1)
+        for (int d = threadIdx.x; d < kRadix; d += kThreads) counts[(size_t)blockIdx.x * kRadix + d] = h[d];
 }
 
-// ---------------------------------------------------------------------------
-// a3: stable LSD radix sort of (key, face id), 8 bits per pass, reduce-then-
-// scan (three kernels per pass, no inter-block waiting of any kind).
-//   upsweep:   per-tile digit histogram, stored digit-major hist[d * T + t]
-//   scan:      one block, exclusive scan of hist in that order, which makes
-//              hist[d * T + t] the global output offset of digit d in tile t
-//   downsweep: stable in-tile ranking (warp match_any + per-warp counters),
-//              scatter through shared memory, coalesced write-out.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(kSortThreads)
-k_sort_upsweep(const unsigned int *__restrict__ keys, int n, int shift,
-               unsigned int *__restrict__ hist, int T, unsigned int *__restrict__ ticket) {
+template <int kThreads, int kItems>
+__global__ void __launch_bounds__(kThreads)
+k_sort_hist(const unsigned int *__restrict__ keys, int n, int shift, SortHist H) {
     __shared__ unsigned int h[kRadix];
     pdl_wait();
-    pdl_trigger();
-    h[threadIdx.x] = 0;
-    if (blockIdx.x == 0 && threadIdx.x == 0) *ticket = 0u;   // the scan's ticket (it runs after this kernel)
+    for (int d = threadIdx.x; d < kRadix; d += kThreads) h[d] = 0u;
     __syncthreads();
-    int base = blockIdx.x * kSortTile;
-    int lane = threadIdx.x & 31;
+    const int base = blockIdx.x * (kThreads * kItems);
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
-        int idx = base + r * kSortThreads + threadIdx.x;
-        bool valid = idx < n;
-        unsigned int d = valid ? (keys[idx] >> shift) & 0xffu : 0x100u;
-        unsigned int peers = __match_any_sync(0xffffffffu, d);
-        if (valid && (__ffs(peers) - 1) == lane) atomicAdd(&h[d], (unsigned)__popc(peers));
+    for (int r = 0; r < kItems; ++r) {
+        const int idx = base + r * kThreads + threadIdx.x;
+        sort_count(h, idx < n, idx < n ? (keys[idx] >> shift) & 0xffu : 0u);
     }
     __syncthreads();
-    hist[(size_t)threadIdx.x * T + blockIdx.x] = h[threadIdx.x];
+    sort_put_counts(H, h, kThreads);
 }
 
 __device__ __forceinline__ unsigned int warp_incl_scan(unsigned int x, int lane) {
@@ -268,31 +307,29 @@ __device__ unsigned int block_excl_scan(unsigned int x, unsigned int *s_warp, un
     return r;
 }
 
-// Offsets for one pass, by one block per digit d: an exclusive scan of the
-// digit's per-tile counts hist[d * T + t] (in place, tile offsets within the
-// digit), and the digit's total.  The last block to finish (ticket counter;
-// nobody waits) turns the 256 totals into exclusive digit bases and resets the
-// ticket.  The output position of digit d in tile t is base[d] + hist[d*T+t].
+// Offsets for one pass with many tiles, by one block per digit d: an exclusive
+// scan over the tiles of the digit's counts hist[t * 256 + d] (in place), and the
+// digit's total.  The last block to finish (ticket counter; nobody waits) turns
+// the 256 totals into exclusive digit bases and resets the ticket.
 __global__ void __launch_bounds__(kScanThreads)
 k_sort_scan(unsigned int *__restrict__ hist, int T, unsigned int *__restrict__ dsum,
             unsigned int *__restrict__ base, unsigned int *__restrict__ ticket) {
     __shared__ unsigned int s_warp[33];
     __shared__ bool s_last;
     pdl_wait();
-    pdl_trigger();
-    unsigned int *h = hist + (size_t)blockIdx.x * T;
+    unsigned int *h = hist + blockIdx.x;
     unsigned int carry = 0;
     const int chunk = kScanThreads * 4;
     for (int b0 = 0; b0 < T; b0 += chunk) {
         int i0 = b0 + 4 * threadIdx.x;
         unsigned int v[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = (i0 + k < T) ? h[i0 + k] : 0u;
+        for (int k = 0; k < 4; ++k) v[k] = (i0 + k < T) ? h[(size_t)(i0 + k) * kRadix] : 0u;
         unsigned int tot;
         unsigned int run = carry + block_excl_scan(v[0] + v[1] + v[2] + v[3], s_warp, &tot);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            if (i0 + k < T) h[i0 + k] = run;
+            if (i0 + k < T) h[(size_t)(i0 + k) * kRadix] = run;
             run += v[k];
         }
         carry += tot;
@@ -311,69 +348,126 @@ k_sort_scan(unsigned int *__restrict__ hist, int T, unsigned int *__restrict__ d
     if (threadIdx.x == 0) *ticket = 0u;
 }
 
-__global__ void __launch_bounds__(kSortThreads)
-k_sort_downsweep(const unsigned int *__restrict__ kin, const int *__restrict__ vin,
-                 unsigned int *__restrict__ kout, int *__restrict__ vout, int n, int shift,
-                 const unsigned int *__restrict__ hist, int T,
-                 const unsigned int *__restrict__ dbase) {
-    __shared__ unsigned int s_keys[kSortTile];
-    __shared__ int s_vals[kSortTile];
-    __shared__ unsigned int s_wcnt[kSortWarps][kRadix];
-    __shared__ unsigned int s_dstart[kRadix];
-    __shared__ unsigned int s_goff[kRadix];
-    __shared__ unsigned int s_warp[33];
+// One pass (see above).  dbase: the digit bases when hist holds scanned offsets
+// (k_sort_scan ran), else NULL.  next: the next pass's counts (NULL: the last
+// pass, or one tile).  vin NULL: the values are the indices.  kGrouped: a warp adds
+// its equal counters first, for keys whose neighbours share digits (tile ids,
+// depths: 58 against 73 us for the render's two passes over 1.8M tile ids;
+// Morton keys share few, and take 36 us instead of 44 without it at 200k).
+template <int kThreads, int kItems> struct SortSmem {
+    unsigned int keys[kThreads * kItems];
+    int vals[kThreads * kItems];
+    unsigned int wcnt[kThreads / 32][kRadix];
+    unsigned int below[kThreads / kRadix][kRadix], total[kThreads / kRadix][kRadix];
+    unsigned int dstart[kRadix], goff[kRadix], warp[33];
+};
+
+template <int kThreads, int kItems, bool kGrouped>
+__global__ void __launch_bounds__(kThreads)
+k_sort_pass(const unsigned int *__restrict__ kin, const int *__restrict__ vin, unsigned int *__restrict__ kout,
+            int *__restrict__ vout, int n, int shift, const unsigned int *__restrict__ hist, int T,
+            const unsigned int *__restrict__ dbase, unsigned int *__restrict__ next) {
+    extern __shared__ char dsm_sort[];
+    SortSmem<kThreads, kItems> &sm = *reinterpret_cast<SortSmem<kThreads, kItems> *>(dsm_sort);
+    constexpr int kTile = kThreads * kItems, kWarps = kThreads / 32, kGroups = kThreads / kRadix;
     pdl_wait();
-    pdl_trigger();
-    int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-    for (int i = tid; i < kSortWarps * kRadix; i += kSortThreads) (&s_wcnt[0][0])[i] = 0;
-    __syncthreads();
-    int base = blockIdx.x * kSortTile;
-    unsigned int key[kSortItems], rank[kSortItems];
-    int val[kSortItems];
-    unsigned int lt_mask = (1u << lane) - 1u;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+    for (int i = tid; i < kWarps * kRadix; i += kThreads) (&sm.wcnt[0][0])[i] = 0;
+    const int base = blockIdx.x * kTile;
+    unsigned int key[kItems], rank[kItems];
+    int val[kItems];
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
-        int idx = base + w * (32 * kSortItems) + r * 32 + lane;
-        bool valid = idx < n;
-        key[r] = valid ? kin[idx] : 0u;
-        val[r] = valid ? (vin ? vin[idx] : idx) : 0;      // vin NULL: the values are the indices
-        unsigned int d = valid ? (key[r] >> shift) & 0xffu : 0x100u;
-        unsigned int peers = __match_any_sync(0xffffffffu, d);
-        unsigned int before = valid ? s_wcnt[w][d] : 0u;
+    for (int r = 0; r < kItems; ++r) {
+        const int idx = base + w * (32 * kItems) + r * 32 + lane;
+        key[r] = idx < n ? kin[idx] : 0u;
+        val[r] = idx < n ? (vin ? vin[idx] : idx) : 0;
+    }
+    // the digit's keys in all tiles and in the tiles before this one
+    const int d = tid % kRadix, grp = tid / kRadix;
+    if (T > 1 && !dbase) {
+        const int per = (T + kGroups - 1) / kGroups, t0 = grp * per, t1 = min(T, t0 + per);
+        unsigned int tot = 0u, low = 0u;
+        for (int t = t0; t < t1; t += 16) {
+            unsigned int c[16];
+#pragma unroll
+            for (int k = 0; k < 16; ++k) c[k] = t + k < t1 ? hist[(size_t)(t + k) * kRadix + d] : 0u;
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                tot += c[k];
+                if (t + k < (int)blockIdx.x) low += c[k];
+            }
+        }
+        sm.total[grp][d] = tot;
+        sm.below[grp][d] = low;
+    }
+    __syncthreads();
+    const unsigned int lt_mask = (1u << lane) - 1u;
+#pragma unroll
+    for (int r = 0; r < kItems; ++r) {
+        const bool valid = base + w * (32 * kItems) + r * 32 + lane < n;
+        const unsigned int dg = valid ? (key[r] >> shift) & 0xffu : 0x100u;
+        const unsigned int peers = __match_any_sync(0xffffffffu, dg);
+        const unsigned int before = valid ? sm.wcnt[w][dg] : 0u;
         __syncwarp();
-        if (valid && (peers & lt_mask) == 0u) s_wcnt[w][d] = before + __popc(peers);
+        if (valid && (peers & lt_mask) == 0u) sm.wcnt[w][dg] = before + __popc(peers);
         __syncwarp();
         rank[r] = valid ? before + __popc(peers & lt_mask) : 0xffffffffu;
     }
     __syncthreads();
     // per digit: exclusive prefix over warps, then exclusive scan over digits
-    unsigned int run = 0;
-    for (int ww = 0; ww < kSortWarps; ++ww) {
-        unsigned int c = s_wcnt[ww][tid];
-        s_wcnt[ww][tid] = run;
-        run += c;
+    unsigned int run = 0u, total = 0u, below = 0u;
+    if (tid < kRadix) {
+        for (int ww = 0; ww < kWarps; ++ww) {
+            const unsigned int c = sm.wcnt[ww][tid];
+            sm.wcnt[ww][tid] = run;
+            run += c;
+        }
+        if (T == 1) {
+            total = run;
+        } else if (!dbase) {
+            for (int g = 0; g < kGroups; ++g) { total += sm.total[g][tid]; below += sm.below[g][tid]; }
+        } else {
+            below = hist[(size_t)blockIdx.x * kRadix + tid];
+        }
     }
-    unsigned int start = block_excl_scan(run, s_warp, nullptr);
-    s_dstart[tid] = start;
-    s_goff[tid] = dbase[tid] + hist[(size_t)tid * T + blockIdx.x];
+    const unsigned int start = block_excl_scan(run, sm.warp, nullptr);
+    const unsigned int first = dbase ? (tid < kRadix ? dbase[tid] : 0u) : block_excl_scan(total, sm.warp, nullptr);
+    if (tid < kRadix) {
+        sm.dstart[tid] = start;
+        sm.goff[tid] = first + below;
+    }
     __syncthreads();
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
+    for (int r = 0; r < kItems; ++r) {
         if (rank[r] != 0xffffffffu) {
-            unsigned int d = (key[r] >> shift) & 0xffu;
-            unsigned int pos = s_dstart[d] + s_wcnt[w][d] + rank[r];
-            s_keys[pos] = key[r];
-            s_vals[pos] = val[r];
+            const unsigned int dg = (key[r] >> shift) & 0xffu;
+            const unsigned int pos = sm.dstart[dg] + sm.wcnt[w][dg] + rank[r];
+            sm.keys[pos] = key[r];
+            sm.vals[pos] = val[r];
         }
     }
     __syncthreads();
-    int nvalid = min(kSortTile, n - base);
-    for (int i = tid; i < nvalid; i += kSortThreads) {
-        unsigned int k = s_keys[i];
-        unsigned int d = (k >> shift) & 0xffu;
-        unsigned int g = s_goff[d] + (unsigned)i - s_dstart[d];
+    const int nvalid = min(kTile, n - base);
+    auto put = [&](int i) {                              // returns the next pass's counter of the key
+        const unsigned int k = sm.keys[i];
+        const unsigned int dg = (k >> shift) & 0xffu;
+        const unsigned int g = sm.goff[dg] + (unsigned)i - sm.dstart[dg];
         kout[g] = k;
-        vout[g] = s_vals[i];
+        vout[g] = sm.vals[i];
+        return (g / kTile) * kRadix + ((k >> (shift + 8)) & 0xffu);
+    };
+    if constexpr (kGrouped) {
+        for (int i0 = 0; i0 < nvalid; i0 += kThreads) {
+            const unsigned int row = i0 + tid < nvalid ? put(i0 + tid) : 0xffffffffu;
+            if (!next) continue;
+            const unsigned int peers = __match_any_sync(0xffffffffu, row);
+            if (row != 0xffffffffu && (peers & lt_mask) == 0u) atomicAdd(&next[row], (unsigned)__popc(peers));
+        }
+    } else {
+        for (int i = tid; i < nvalid; i += kThreads) {
+            const unsigned int row = put(i);
+            if (next) atomicAdd(&next[row], 1u);
+        }
     }
 }
 
@@ -847,7 +941,7 @@ __global__ void k_batch_faces(const int *__restrict__ F3, int nF, const int *__r
 __global__ void k_batch_morton(const float4 *__restrict__ cent, int nF, const int4 *__restrict__ F4,
                                const unsigned int *__restrict__ cbox,
                                unsigned int *__restrict__ key_of_face,
-                               unsigned int *__restrict__ keys, int *__restrict__ vals) {
+                               unsigned int *__restrict__ keys) {
     int f = blockIdx.x * blockDim.x + threadIdx.x;
     if (f >= nF) return;
     const unsigned int *bx = cbox + 6 * F4[f].w;
@@ -866,7 +960,6 @@ __global__ void k_batch_morton(const float4 *__restrict__ cent, int nF, const in
     unsigned int key = (spread3(q[0]) << 2) | (spread3(q[1]) << 1) | spread3(q[2]);
     key_of_face[f] = key;
     keys[f] = key;
-    vals[f] = f;
 }
 
 // Scene id of each (Morton-sorted) face, as the key of the last, stable pass.
@@ -957,15 +1050,14 @@ __global__ void k_batch_leaves_up(int nF, const int *__restrict__ face_off, int 
 struct BuildWs {
     unsigned int *keysA, *keysB, *hist, *cbox, *dsum, *dbase, *ticket;
     int *valsA, *valsB;
-    float4 *cent;
-    int tiles;
+    float4 *cent;                      // face centroids; once the keys exist, the later passes' counts
     size_t bytes;
 };
 
 static BuildWs build_ws_layout(char *base, int64_t nF) {
     BuildWs w{};
     int64_t n = nF > 0 ? nF : 1;
-    w.tiles = (int)((n + kSortTile - 1) / kSortTile);
+    const int64_t rows = (n + kSortTileMin - 1) / kSortTileMin;
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes, 256); return base + o; };
     w.keysA = (unsigned int *)take(4 * n);
@@ -973,7 +1065,7 @@ static BuildWs build_ws_layout(char *base, int64_t nF) {
     w.valsA = (int *)take(4 * n);
     w.valsB = (int *)take(4 * n);
     w.cent = (float4 *)take(16 * n);
-    w.hist = (unsigned int *)take((size_t)4 * kRadix * w.tiles);
+    w.hist = (unsigned int *)take((size_t)4 * kRadix * rows);
     w.cbox = (unsigned int *)take(32);
     w.dsum = (unsigned int *)take(4 * kRadix);
     w.dbase = (unsigned int *)take(4 * kRadix);
@@ -982,39 +1074,107 @@ static BuildWs build_ws_layout(char *base, int64_t nF) {
     return w;
 }
 
-// Four 8-bit passes over (w.keysA, w.valsA): A -> B -> A -> B -> (out_keys,
-// out_vals).  out_keys may be w.keysA (the last pass reads B).
-static void radix_sort_pairs(const BuildWs &w, int n, unsigned int *out_keys, int *out_vals,
-                             cudaStream_t s) {
-    unsigned int *kin = w.keysA, *kout = w.keysB;
-    int *vin = w.valsA, *vout = w.valsB;
-    for (int pass = 0; pass < 4; ++pass) {
-        if (pass == 3) { kout = out_keys; vout = out_vals; }
-        int shift = 8 * pass;
-        k_sort_upsweep<<<w.tiles, kSortThreads, 0, s>>>(kin, n, shift, w.hist, w.tiles, w.ticket);
-        k_sort_scan<<<kRadix, kScanThreads, 0, s>>>(w.hist, w.tiles, w.dsum, w.dbase, w.ticket);
-        k_sort_downsweep<<<w.tiles, kSortThreads, 0, s>>>(kin, vin, kout, vout, n, shift, w.hist,
-                                                          w.tiles, w.dbase);
-        count_launch(3);
-        unsigned int *tk = kin; kin = kout; kout = tk;
-        int *tv = vin; vin = vout; vout = tv;
-    }
+// Threads and keys per thread of a sort of n keys: f gets them as compile-time
+// constants.  Tiles grow with n: a pass reads every tile's 256 counts in every
+// block, 1 KB x tiles^2 in all, against 8 B x n of keys -- at most about 250 tiles
+// up to 2M keys.  Smaller tiles than these spread the ranking over more SMs.
+template <typename F> static void sort_shape(int n, F f) {
+    using std::integral_constant;
+    if (n <= 160 * 1024) f(integral_constant<int, 256>(), integral_constant<int, 4>());
+    else if (n <= 480 * 1024) f(integral_constant<int, 256>(), integral_constant<int, 8>());
+    else if (n <= 1024 * 1024) f(integral_constant<int, 512>(), integral_constant<int, 8>());
+    else f(integral_constant<int, 512>(), integral_constant<int, 16>());
 }
 
-// One pass for the other kernels of the library, its three kernels launched as
-// programmatic dependents (the contact and Chamfer steps' orders run on a
-// frame's critical path, where the launch latency counts).  The build's passes
-// above use plain launches: there the early-launched grids measured slower.
+static int sort_tiles(int n) {
+    int T = 0;
+    sort_shape(n, [&](auto th, auto it) { T = (n + th.value * it.value - 1) / (th.value * it.value); });
+    return T;
+}
+
+// The later passes' counts lie over the centroids (16 B per key; three more
+// passes take 3 KB per tile of at least 1024 keys; one tile keeps no counts).
+static SortHist sort_hist(const BuildWs &w, int n, int passes) {
+    return SortHist{w.hist, reinterpret_cast<unsigned int *>(w.cent), sort_tiles(n), passes};
+}
+
+static void morton_keys(const BuildWs &w, int n, cudaStream_t s) {
+    const SortHist H = sort_hist(w, n, 4);
+    sort_shape(n, [&](auto th, auto it) {
+        pdl_launch(k_morton<th.value, it.value>, (unsigned)H.T, th.value, 0, s, (const float4 *)w.cent, n,
+                   (const unsigned int *)w.cbox, w.keysA, H.first, H.T);
+    });
+    count_launch();
+    // the centroids are read: the later passes' counts take their place
+    if (H.T > 1) cudaMemsetAsync(H.rest, 0, (size_t)(H.passes - 1) * H.T * kRadix * sizeof(unsigned int), s);
+}
+
+// Passes p = 0 .. H.passes - 1 on bits 8 p .. 8 p + 7 (plus shift0), the first
+// from (kin, vin) with its counts in H.first, the last into (kout, vout); those
+// between alternate over the workspace's B and A arrays (kin may be A when
+// H.passes > 1, and kout too when it is even).  after_kernel: the call's last
+// launch is a kernel (the first pass is its programmatic dependent).
+template <bool kGrouped>
+static void sort_passes(const BuildWs &w, int n, int shift0, const unsigned int *kin, const int *vin,
+                        unsigned int *kout, int *vout, const SortHist &H, bool after_kernel, cudaStream_t s) {
+    sort_shape(n, [&](auto th, auto it) {
+        constexpr int TH = th.value, IT = it.value;
+        using Smem = SortSmem<TH, IT>;
+        auto kern = k_sort_pass<TH, IT, kGrouped>;
+        static const cudaError_t set =
+            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
+        (void)set;                                       // a failure shows as the launch's
+        const unsigned int *ki = kin;
+        const int *vi = vin;
+        for (int p = 0; p < H.passes; ++p) {
+            const bool last = p == H.passes - 1;
+            unsigned int *ko = last ? kout : (p & 1) ? w.keysA : w.keysB;
+            int *vo = last ? vout : (p & 1) ? w.valsA : w.valsB;
+            unsigned int *h = p == 0 ? H.first : H.rest + (size_t)(p - 1) * H.T * kRadix;
+            unsigned int *next = last || H.T == 1 ? nullptr : H.rest + (size_t)p * H.T * kRadix;
+            const bool scanned = H.T > kSortTilesMax;
+            if (scanned) {
+                if (p == 0) cudaMemsetAsync(w.ticket, 0, sizeof(unsigned int), s);
+                launch_ex(p != 0, k_sort_scan, kRadix, kScanThreads, 0, s, h, H.T, w.dsum, w.dbase, w.ticket);
+                count_launch();
+            }
+            launch_ex(p != 0 || after_kernel || scanned, kern, (unsigned)H.T, TH, sizeof(Smem), s, ki, vi, ko, vo, n,
+                      shift0 + 8 * p, (const unsigned int *)h, H.T,
+                      scanned ? (const unsigned int *)w.dbase : (const unsigned int *)nullptr, next);
+            count_launch();
+            ki = ko;
+            vi = vo;
+        }
+    });
+}
+
+// The counts of the first pass over `keys`.
+static void sort_count_keys(int n, int shift, const unsigned int *keys, const SortHist &H, cudaStream_t s) {
+    if (H.T == 1) return;
+    sort_shape(n, [&](auto th, auto it) {
+        pdl_launch(k_sort_hist<th.value, it.value>, (unsigned)H.T, th.value, 0, s, keys, n, shift, H);
+    });
+    count_launch();
+}
+
+// The sorting permutation of keysA (30-bit keys) and the keys in order.  counted:
+// morton_keys made the keys; else the call's last launch is the kernel that did.
+static void radix_sort_keys(const BuildWs &w, int n, unsigned int *out_keys, int *out_vals, bool counted,
+                            cudaStream_t s) {
+    const SortHist H = sort_hist(w, n, 4);
+    if (!counted) sort_count_keys(n, 0, w.keysA, H, s);
+    sort_passes<false>(w, n, 0, w.keysA, nullptr, out_keys, out_vals, H, !counted || H.T == 1, s);
+}
+
+// One stable pass on bits shift .. shift + 7, after a kernel of the same call.
 static void radix_pass(const BuildWs &w, int n, int shift, const unsigned int *kin, const int *vin,
                        unsigned int *kout, int *vout, cudaStream_t s) {
-    pdl_launch(k_sort_upsweep, w.tiles, kSortThreads, 0, s, kin, n, shift, w.hist, w.tiles, w.ticket);
-    pdl_launch(k_sort_scan, kRadix, kScanThreads, 0, s, w.hist, w.tiles, w.dsum, w.dbase, w.ticket);
-    pdl_launch(k_sort_downsweep, w.tiles, kSortThreads, 0, s, kin, vin, kout, vout, n, shift, w.hist, w.tiles,
-               w.dbase);
-    count_launch(3);
+    const SortHist H = sort_hist(w, n, 1);
+    sort_count_keys(n, shift, kin, H, s);
+    sort_passes<true>(w, n, shift, kin, vin, kout, vout, H, true, s);
 }
 
-// Stable sort of (key, value) pairs on the low `bits` key bits (8 per pass),
+// Stable sort of (key, value) pairs on the low `bits` key bits (8 per pass), after a kernel of the same call,
 // for other kernels of the library; ws holds sort_pairs_ws_bytes(n) bytes.
 // vin NULL: the values are the indices 0 .. n-1 (the sorting permutation).
 size_t sort_pairs_ws_bytes(int64_t n) { return build_ws_layout(nullptr, n).bytes + 256; }
@@ -1022,16 +1182,9 @@ size_t sort_pairs_ws_bytes(int64_t n) { return build_ws_layout(nullptr, n).bytes
 void sort_pairs_u32(void *ws, int n, int bits, const unsigned int *kin, const int *vin, unsigned int *kout,
                     int *vout, cudaStream_t s) {
     BuildWs w = build_ws_layout((char *)ws, n);
-    const int passes = bits <= 0 ? 1 : (bits + 7) / 8;
-    unsigned int *kb[2] = {w.keysA, w.keysB};
-    int *vb[2] = {w.valsA, w.valsB};
-    for (int p = 0; p < passes; ++p) {
-        const unsigned int *ki = p == 0 ? kin : kb[(p - 1) & 1];
-        const int *vi = p == 0 ? vin : vb[(p - 1) & 1];
-        unsigned int *ko = p == passes - 1 ? kout : kb[p & 1];
-        int *vo = p == passes - 1 ? vout : vb[p & 1];
-        radix_pass(w, n, 8 * p, ki, vi, ko, vo, s);
-    }
+    const SortHist H = sort_hist(w, n, bits <= 0 ? 1 : (bits + 7) / 8);
+    sort_count_keys(n, 0, kin, H, s);
+    sort_passes<true>(w, n, 0, kin, vin, kout, vout, H, true, s);
 }
 
 struct BatchWs {
@@ -1391,7 +1544,7 @@ mesh_status mesh_update_vertices(mesh_bvh *bvh, const float *d_V, int64_t nV, vo
     bvh->L.n_verts = nV;
     if (nV == 0) return MESH_OK;
     cudaStream_t s = (cudaStream_t)stream;
-    k_copy_verts<<<grid_for(nV, kBlock), kBlock, 0, s>>>(d_V, (int)nV, bvh->verts(), nullptr);
+    k_copy_verts<<<grid_for(nV, kBlock), kBlock, 0, s>>>(d_V, (int)nV, bvh->verts(), nullptr, nullptr);
     count_launch();
     return check_launch();
 }
@@ -1461,17 +1614,18 @@ static void build_keys(mesh_bvh *bvh, const float *d_V, int64_t nV, const int32_
     bvh->adj_ready = false;
     bvh->wide_valid = false;
     int n = (int)nF;
-    cudaMemsetAsync(bvh->hdr(), 0, sizeof(Header), s);
     if (nV > 0) {
-        k_copy_verts<<<grid_for(nV > 6 ? nV : 6, kBlock), kBlock, 0, s>>>(
-            d_V, (int)nV, bvh->verts(), n > 0 ? w.cbox : nullptr);
+        k_copy_verts<<<grid_for(nV, kBlock), kBlock, 0, s>>>(d_V, (int)nV, bvh->verts(), n > 0 ? w.cbox : nullptr,
+                                                             bvh->hdr());
         count_launch();
+    } else {
+        cudaMemsetAsync(bvh->hdr(), 0, sizeof(Header), s);
     }
     if (n == 0) return;
     k_faces_centroids<<<grid_for(n, kBlock), kBlock, 0, s>>>(d_F, n, (int)nV, bvh->verts(),
                                                              bvh->faces(), w.cent, w.cbox, bvh->hdr());
-    k_morton<<<grid_for(n, kBlock), kBlock, 0, s>>>(w.cent, n, w.cbox, w.keysA, w.valsA);
-    count_launch(2);
+    count_launch();
+    morton_keys(w, n, s);
 }
 
 mesh_status mesh_build_lbvh(mesh_bvh *bvh, const float *d_V, int64_t nV, const int32_t *d_F,
@@ -1485,7 +1639,7 @@ mesh_status mesh_build_lbvh(mesh_bvh *bvh, const float *d_V, int64_t nV, const i
     int n = (int)nF;
     build_keys(bvh, d_V, nV, d_F, nF, w, s);
     if (n == 0) return check_launch();
-    radix_sort_pairs(w, n, bvh->keys(), bvh->perm(), s);
+    radix_sort_keys(w, n, bvh->keys(), bvh->perm(), true, s);
     if (n > 1) {
         k_karras<<<grid_for(n - 1, kBlock), kBlock, 0, s>>>(bvh->keys(), n, bvh->nodes(),
                                                            bvh->parent(), bvh->rend());
@@ -1513,11 +1667,11 @@ mesh_status mesh_build_ploc(mesh_bvh *bvh, const float *d_V, int64_t nV, const i
     build_keys(bvh, d_V, nV, d_F, nF, w.sort, s);
     if (n == 0) return check_launch();
     if (n == 1) {                                     // a lone leaf, as mesh_build_lbvh leaves it
-        radix_sort_pairs(w.sort, n, bvh->keys(), bvh->perm(), s);
+        radix_sort_keys(w.sort, n, bvh->keys(), bvh->perm(), true, s);
         cudaMemsetAsync(bvh->parent(), 0xff, sizeof(int), s);
         return bottom_up(bvh, nullptr, s);
     }
-    radix_sort_pairs(w.sort, n, w.sk, w.perm0, s);
+    radix_sort_keys(w.sort, n, w.sk, w.perm0, true, s);
     k_ploc_leaves<<<grid_for(n, kBlock), kBlock, 0, s>>>(n, w.perm0, bvh->faces(), bvh->verts(), w.clA, w.cbA);
     count_launch();
     std::vector<int2> batches;                        // (first node, count) made per iteration
@@ -1599,9 +1753,9 @@ mesh_status mesh_morton_order(const float *d_P, int64_t n, int32_t *d_order, voi
     int m = (int)n;
     k_init_box<<<1, 32, 0, s>>>(w.cbox);
     k_points_centroids<<<grid_for(m, kBlock), kBlock, 0, s>>>(d_P, m, w.cent, w.cbox);
-    k_morton<<<grid_for(m, kBlock), kBlock, 0, s>>>(w.cent, m, w.cbox, w.keysA, w.valsA);
-    count_launch(3);
-    radix_sort_pairs(w, m, w.keysA, d_order, s);
+    count_launch(2);
+    morton_keys(w, m, s);
+    radix_sort_keys(w, m, w.keysA, d_order, true, s);
     return check_launch();
 }
 
@@ -1659,7 +1813,7 @@ mesh_status mesh_batch_build(mesh_batch *batch, int64_t n_scenes, const float *d
     cudaMemcpyAsync(batch->vert_off(), d_vert_off, 4 * (size_t)(B + 1), cudaMemcpyDeviceToDevice, s);
     cudaMemcpyAsync(batch->face_off(), d_face_off, 4 * (size_t)(B + 1), cudaMemcpyDeviceToDevice, s);
     if (nV > 0) {
-        k_copy_verts<<<grid_for(nV, kBlock), kBlock, 0, s>>>(d_V, (int)nV, batch->verts(), nullptr);
+        k_copy_verts<<<grid_for(nV, kBlock), kBlock, 0, s>>>(d_V, (int)nV, batch->verts(), nullptr, nullptr);
         count_launch();
     }
     if (n == 0) return check_launch();
@@ -1669,12 +1823,12 @@ mesh_status mesh_batch_build(mesh_batch *batch, int64_t n_scenes, const float *d
                                                          B, batch->verts(), batch->faces(), w.sort.cent,
                                                          w.cbox, status);
     k_batch_morton<<<grid_for(n, kBlock), kBlock, 0, s>>>(w.sort.cent, n, batch->faces(), w.cbox,
-                                                          w.key_of_face, w.sort.keysA, w.sort.valsA);
+                                                          w.key_of_face, w.sort.keysA);
     count_launch(3);
     // Morton order over all faces, then a stable pass (two past 256 scenes) on
     // the scene id: faces end up grouped by scene in the order a per-scene
     // build would give them.
-    radix_sort_pairs(w.sort, n, w.sort.keysA, w.sort.valsA, s);
+    radix_sort_keys(w.sort, n, w.sort.keysA, w.sort.valsA, false, s);
     k_batch_scene_keys<<<grid_for(n, kBlock), kBlock, 0, s>>>(w.sort.valsA, n, batch->faces(),
                                                               w.sort.keysA);
     count_launch();
@@ -1702,7 +1856,7 @@ mesh_status mesh_batch_refit(mesh_batch *batch, const float *d_V, int64_t nV, vo
     if (!batch || (d_V && nV != batch->L.n_verts)) return MESH_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     if (d_V && nV > 0) {
-        k_copy_verts<<<grid_for(nV, kBlock), kBlock, 0, s>>>(d_V, (int)nV, batch->verts(), nullptr);
+        k_copy_verts<<<grid_for(nV, kBlock), kBlock, 0, s>>>(d_V, (int)nV, batch->verts(), nullptr, nullptr);
         count_launch();
     }
     int n = (int)batch->L.n_faces;

@@ -185,3 +185,16 @@ def test_point_morton_order_bit_exact(n):
     _, perm = oracle.sort_pairs(keys)
     got = host(morton_order(dev(P)))
     assert np.array_equal(got, perm)
+
+
+@pytest.mark.parametrize("n", [1023, 1024, 1025, 2049, 160 * 1024, 160 * 1024 + 1, 480 * 1024 + 1,
+                               1024 * 1024 + 1, 512 * 8192 + 1])
+def test_sort_at_the_edges_of_its_tiles(n):
+    """One tile and two, the first size of every tile length, and the first whose tile
+    counts are scanned in a launch of their own."""
+    from paper_2606_00444_gb300 import morton_order
+    rng = np.random.default_rng(n)
+    P = rng.integers(-40, 40, (n, 3)).astype(np.float32)     # many equal keys
+    idx = np.arange(n, dtype=np.int32)
+    keys = oracle.morton(P, np.stack([idx, idx, idx], 1))
+    assert np.array_equal(host(morton_order(dev(P))), np.argsort(keys, kind="stable"))
