@@ -231,7 +231,9 @@ __device__ __forceinline__ void list_close(const EmdLists &L, int i, int cnt, in
 // Value of an object to within about 1e-6 of its distance, for choosing a
 // threshold: one reciprocal-root instruction instead of a rounded square root.
 __device__ __forceinline__ float value_approx(float d2, float price) {
-    return -(d2 * rsqrtf(fmaxf(d2, 1e-30f))) - price;
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(fmaxf(d2, 1e-30f)));
+    return -(d2 * r) - price;
 }
 
 __global__ void k_emd_lists_init(int n, EmdLists L, float margin) {
@@ -364,27 +366,52 @@ __global__ void k_emd_resolve_lists(int n, float4 *__restrict__ B4, int *owner, 
 // an evicted owner joins the back of the queue.  At most max_bids bids;
 // *active gets the points still queued.
 //
-// Warp 0 commits bids: prices and owners in shared memory, the bidder's list
-// (read through L1: the points of a price war take turns, and 91 KB of shared
-// memory leave the SM room to keep theirs), the next bidder's list fetched
-// ahead while the queue holds one.  When a list does not decide, the other 31
-// warps, which hold the objects' coordinates in registers, make it again.
-// A call is a chain of ~270k dependent bids at 10k points, so the latency of
-// one bid is the time: a block-wide scan of all objects for each took 2.0 us
-// (531 of the call's 545 ms; 259 ms with lists, of which a bid from its list
-// takes about 1600 cycles, most of them the list's trip from L2, and a new
-// list about 10000).
-constexpr int kTailThreads = 1024;
+// A call is a chain of ~270k dependent bids at 10k points, so the latency of one
+// bid is the time.  A list's trip from L2 is most of a bid's (a block-wide scan
+// of all objects for each bid took 2.0 us, a bid from its list 0.8), so the
+// lists of the next kTailAhead queued points are read together, each by a warp,
+// which leaves the lane-wise best 32 entries in shared memory with the value
+// that everything left out stays below.  Warp 0 then commits those bids in
+// queue order, each from its 32 entries at the prices of that moment (in shared
+// memory, as are the owners), as long as they decide it: prices only rise, so
+// what was left out stays below.  The head of the queue, with no bid since its
+// list was read, bids from the whole list.  A point whose list no longer decides
+// gets a new one from a scan by all other warps, which hold the objects'
+// coordinates in registers, two points at a time.
+// 10k points, eps 1e-4: 259 ms with one list at a time, 191 ms so (531 with scans).
+constexpr int kTailThreads = 768;                    // 80 registers each: 48 of coordinates
 constexpr int kTailQueue = 256;
-constexpr int kScanThreads = kTailThreads - 32;      // warps 1-31
-constexpr int kScanPer = 12;                         // objects a scanning thread holds
+constexpr int kTailAhead = 16;
+constexpr int kScanThreads = kTailThreads - 32;      // all but warp 0
+constexpr int kScanPer = 16;                         // objects a scanning thread holds
 constexpr int kTailMaxN = 11417;                     // largest n taken (16 + 4 B of shared memory each would fit)
 static_assert(kScanThreads * kScanPer >= kTailMaxN, "every object is held by a thread");
+static_assert(kTailAhead < kTailThreads / 32, "a warp per list, beside warp 0");
 
-enum { kTailDone = 0, kTailList = 1, kTailExact = 2 };
+enum { kTailDone = 0, kTailRead = 1, kTailList = 2, kTailExact = 3 };
 
 __device__ __forceinline__ void bar_sync(int id, int threads) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+
+// What a warp leaves of a queued point's list: per lane its least cost (distance
+// plus price; the value negated) entry, and the least cost not among them.
+struct TailAhead {
+    float d[kTailAhead][32];
+    int j[kTailAhead][32];
+    float rest[kTailAhead];            // -inf: the list does not decide
+    float b1, b2;                      // the head's bid from its whole list
+    int j1;
+};
+
+// Least and second-least cost of a warp's lanes (one entry each) and the lowest
+// object at the least.  Costs are not negative, so their bits order like them.
+__device__ __forceinline__ void least2(float c, int j, float &c1, int &j1, float &c2) {
+    const unsigned full = 0xffffffffu, u = __float_as_uint(c);
+    const unsigned m = __reduce_min_sync(full, u);
+    j1 = (int)__reduce_min_sync(full, u == m ? (unsigned)j : 0x7fffffffu);
+    c2 = __uint_as_float(__reduce_min_sync(full, u == m && j == j1 ? 0x7f800000u : u));
+    c1 = __uint_as_float(m);
 }
 
 __global__ void __launch_bounds__(kTailThreads, 1)
@@ -392,10 +419,11 @@ k_emd_tail(int n, const float4 *__restrict__ A4, float4 *B4, float *price, int *
            float eps, int max_bids, unsigned *active) {
     extern __shared__ float sp[];                    // prices, then owners
     int *s_own = reinterpret_cast<int *>(sp + n);
+    __shared__ TailAhead s_ahead;
     __shared__ int queue[kTailQueue];
-    __shared__ float r1[32], r2[32];
+    __shared__ float r1[2][32], r2[2][32];
     __shared__ int rj[32], s_wcnt[32];
-    __shared__ int s_len, s_mode, s_point, s_cnt;
+    __shared__ int s_len, s_mode, s_head, s_point[2], s_cnt[2];
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const bool lists = L.entry != nullptr;
     for (int j = tid; j < n; j += kTailThreads) { sp[j] = price ? price[j] : B4[j].w; s_own[j] = owner[j]; }
@@ -421,12 +449,12 @@ k_emd_tail(int n, const float4 *__restrict__ A4, float4 *B4, float *price, int *
         __syncthreads();
     }
     if (wid == 0) {
-        int head = 0, len = s_len, bids = 0, mode = kTailDone;
-        auto commit = [&](int i, float b1, int j1, float b2) {
+        int head = 0, len = s_len, bids = 0;
+        auto commit = [&](int i, float gap, int j1) {    // gap: best less second-best value
             const int old = s_own[j1];
             __syncwarp();
             if (lane == 0) {
-                sp[j1] += (b2 == -INFINITY ? 0.0f : b1 - b2) + eps;
+                sp[j1] += gap + eps;
                 s_own[j1] = i;
                 assign[i] = j1;
                 if (old >= 0) {
@@ -439,66 +467,62 @@ k_emd_tail(int n, const float4 *__restrict__ A4, float4 *B4, float *price, int *
             if (old < 0) --len;
             __syncwarp();
         };
-        auto price_of = [&](int j) { return sp[j]; };
-        bool fresh = false;                          // the head's list was just made
-        while (true) {
-            mode = kTailDone;
-            int i = -1;
-            if (lists) {
-                int4 e[4];
-                float T = 0.0f;
-                int have = -1;                       // the point whose list e and T hold
-                while (bids < max_bids && len > 0) {
-                    i = queue[head % kTailQueue];
-                    if (have != i) {
-                        T = L.hdr[i].x;
-                        list_load(L, i, lane, e);
-                    }
-                    int4 f[4];
-                    float Tn = 0.0f;
-                    int next = -1;
-                    if (len > 1) {
-                        next = queue[(head + 1) % kTailQueue];
-                        Tn = L.hdr[next].x;
-                        list_load(L, next, lane, f);
-                    }
-                    mode = kTailList;
-                    if (T == INFINITY) break;
-                    float b1, b2;
-                    int j1;
-                    list_best2(e, price_of, b1, j1, b2);
-                    if (!(b1 > T && b2 >= T)) break;
-                    commit(i, b1, j1, b2);
-                    mode = kTailDone;
-                    fresh = false;
-                    have = next;
-                    T = Tn;
-                    if (next >= 0) {
-#pragma unroll
-                        for (int m = 0; m < 4; ++m) e[m] = f[m];
-                    }
-                }
-                if (mode == kTailList && fresh) mode = kTailExact;
-            } else if (bids < max_bids && len > 0) {
-                i = queue[head % kTailQueue];
-                mode = kTailExact;
-            }
-            if (lane == 0) { s_mode = mode; s_point = i; }
+        // hand a step to the other warps and wait for it
+        auto step = [&](int mode) {
+            if (lane == 0) { s_mode = mode; s_head = head; s_len = len; }
             bar_sync(1, kTailThreads);
-            if (mode == kTailDone) break;
-            bar_sync(1, kTailThreads);               // the scan is done
-            fresh = mode == kTailList;
-            if (mode == kTailExact) {
-                float b1 = lane > 0 ? r1[lane] : -INFINITY, b2 = lane > 0 ? r2[lane] : -INFINITY;
-                int j1 = lane > 0 ? rj[lane] : 0x7fffffff;
-                warp_best2(b1, j1, b2);
-                if ((unsigned)j1 >= (unsigned)n) {   // no comparable value (NaN input): leave the point queued
-                    max_bids = bids;
-                    continue;
+            if (mode != kTailDone) bar_sync(1, kTailThreads);
+        };
+        bool fresh = false;                          // the head's list was just made
+        while (bids < max_bids && len > 0) {
+            if (lists) {
+                step(kTailRead);
+                const int ahead = min(len, kTailAhead);
+                int done = 0;
+                if (s_ahead.rest[0] >= 0.0f) {       // the head, from its whole list
+                    const float b1 = s_ahead.b1, b2 = s_ahead.b2;
+                    commit(queue[head % kTailQueue], b2 == -INFINITY ? 0.0f : b1 - b2, s_ahead.j1);
+                    done = 1;
                 }
-                commit(i, b1, j1, b2);
+                float d = s_ahead.d[1][lane];        // the next entries, one bid ahead of their use
+                int j = s_ahead.j[1][lane];
+                while (done > 0 && done < ahead && bids < max_bids) {
+                    const float rest = s_ahead.rest[done];
+                    if (!(rest >= 0.0f)) break;      // (its entries need not be written)
+                    const float nd = d + sp[j];
+                    const int i = queue[head % kTailQueue], nj = j;
+                    if (done + 1 < ahead) { d = s_ahead.d[done + 1][lane]; j = s_ahead.j[done + 1][lane]; }
+                    float c1, c2;
+                    int j1;
+                    least2(nd, nj, c1, j1, c2);
+                    if (!(c1 < rest && c2 <= rest)) break;
+                    commit(i, c2 == INFINITY ? 0.0f : c2 - c1, j1);
+                    ++done;
+                }
+                if (done > 0) { fresh = false; continue; }
             }
+            if (lists && !fresh) {                   // new lists for the head and the next that needs one
+                const int ahead = min(len, kTailAhead);
+                const unsigned need = __ballot_sync(0xffffffffu, lane > 0 && lane < ahead && s_ahead.rest[lane < kTailAhead ? lane : 0] < 0.0f);
+                if (lane == 0) {
+                    s_point[0] = queue[head % kTailQueue];
+                    s_point[1] = need ? queue[(head + __ffs(need) - 1) % kTailQueue] : -1;
+                }
+                step(kTailList);
+                fresh = true;
+                continue;
+            }
+            if (lane == 0) s_point[0] = queue[head % kTailQueue];
+            step(kTailExact);
+            float b1 = lane > 0 && lane < kTailThreads / 32 ? r1[0][lane] : -INFINITY;
+            float b2 = lane > 0 && lane < kTailThreads / 32 ? r2[0][lane] : -INFINITY;
+            int j1 = lane > 0 && lane < kTailThreads / 32 ? rj[lane] : 0x7fffffff;
+            warp_best2(b1, j1, b2);
+            if ((unsigned)j1 >= (unsigned)n) break;  // no comparable value (NaN input): leave the point queued
+            commit(s_point[0], b2 == -INFINITY ? 0.0f : b1 - b2, j1);
+            fresh = false;
         }
+        step(kTailDone);
         if (lane == 0) *active = (unsigned)len;
     } else {
         const int t = tid - 32;
@@ -511,11 +535,54 @@ k_emd_tail(int n, const float4 *__restrict__ A4, float4 *B4, float *price, int *
         }
         while (true) {
             bar_sync(1, kTailThreads);
-            const int mode = s_mode, i = s_point;
+            const int mode = s_mode;
             if (mode == kTailDone) break;
-            const float4 a = A4[i];
-            float b1 = -INFINITY, b2 = -INFINITY;
+            if (mode == kTailRead) {
+                const int q = wid - 1;
+                if (q < min(s_len, kTailAhead)) {
+                    const int i = queue[(s_head + q) % kTailQueue];
+                    const float T = L.hdr[i].x;
+                    int4 e[4];
+                    list_load(L, i, lane, e);
+                    if (T == INFINITY) {             // no list (its entries are not read)
+                        s_ahead.d[q][lane] = INFINITY;
+                        s_ahead.j[q][lane] = 0;
+                        if (lane == 0) s_ahead.rest[q] = -INFINITY;
+                    } else {
+                        // this lane's least cost, its object, and its second-least
+                        float c1 = INFINITY, c2 = INFINITY, d1 = INFINITY;
+                        int j1 = 0;
+                        auto take = [&](int j, int dbits) {
+                            const float d = __int_as_float(dbits), c = d + sp[j];
+                            const bool better = c < c1 || (c == c1 && j < j1);
+                            c2 = fminf(c2, better ? c1 : c);
+                            if (better) { c1 = c; d1 = d; j1 = j; }
+                        };
+#pragma unroll
+                        for (int m = 0; m < 4; ++m) {
+                            take(e[m].x, e[m].y);
+                            take(e[m].z, e[m].w);
+                        }
+                        s_ahead.d[q][lane] = d1;
+                        s_ahead.j[q][lane] = j1;
+                        const float second = __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(c2)));
+                        float l1, l2;
+                        int lj;
+                        least2(c1, j1, l1, lj, l2);
+                        l2 = fminf(l2, second);      // the list's second-least: another lane's best or some lane's second
+                        if (lane == 0) {
+                            const bool decides = l1 < -T && l2 <= -T;
+                            s_ahead.rest[q] = decides ? fminf(second, -T) : -INFINITY;
+                            if (q == 0) { s_ahead.b1 = -l1; s_ahead.b2 = -l2; s_ahead.j1 = lj; }
+                        }
+                    }
+                }
+                bar_sync(1, kTailThreads);
+                continue;
+            }
             if (mode == kTailExact) {
+                const float4 a = A4[s_point[0]];
+                float b1 = -INFINITY, b2 = -INFINITY;
                 int j1 = 0x7fffffff;
 #pragma unroll
                 for (int k = 0; k < kScanPer; ++k) {
@@ -523,40 +590,61 @@ k_emd_tail(int n, const float4 *__restrict__ A4, float4 *B4, float *price, int *
                     if (j < n) merge2(b1, j1, b2, -sqrtf(emd_d2(a, bx[k], by[k], bz[k])) - sp[j], j, -INFINITY);
                 }
                 warp_best2(b1, j1, b2);
-                if (lane == 0) { r1[wid] = b1; r2[wid] = b2; rj[wid] = j1; }
+                if (lane == 0) { r1[0][wid] = b1; r2[0][wid] = b2; rj[wid] = j1; }
                 bar_sync(1, kTailThreads);
                 continue;
             }
-            const float margin = L.hdr[i].y;
-            if (t == 0) s_cnt = 0;
+            // new lists of one or two points
+            const int i0 = s_point[0], i1 = s_point[1];
+            const float4 a0 = A4[i0], a1 = A4[i1 >= 0 ? i1 : i0];
+            const float margin0 = L.hdr[i0].y, margin1 = L.hdr[i1 >= 0 ? i1 : i0].y;
+            if (t < 2) s_cnt[t] = 0;
+            float b1 = -INFINITY, b2 = -INFINITY, e1 = -INFINITY, e2 = -INFINITY;
 #pragma unroll
             for (int k = 0; k < kScanPer; ++k) {
                 const int j = t + k * kScanThreads;
                 if (j < n) {
-                    const float v = value_approx(emd_d2(a, bx[k], by[k], bz[k]), sp[j]);
+                    const float p = sp[j];
+                    float v = value_approx(emd_d2(a0, bx[k], by[k], bz[k]), p);
                     b2 = fmaxf(b2, fminf(b1, v));
                     b1 = fmaxf(b1, v);
+                    v = value_approx(emd_d2(a1, bx[k], by[k], bz[k]), p);
+                    e2 = fmaxf(e2, fminf(e1, v));
+                    e1 = fmaxf(e1, v);
                 }
             }
             int dummy = lane;
             warp_best2(b1, dummy, b2);
-            if (lane == 0) { r1[wid] = b1; r2[wid] = b2; }
+            dummy = lane;
+            warp_best2(e1, dummy, e2);
+            if (lane == 0) { r1[0][wid] = b1; r2[0][wid] = b2; r1[1][wid] = e1; r2[1][wid] = e2; }
             bar_sync(2, kScanThreads);
-            b1 = lane > 0 ? r1[lane] : -INFINITY;
-            b2 = lane > 0 ? r2[lane] : -INFINITY;
+            const bool in = lane > 0 && lane < kTailThreads / 32;
+            b1 = in ? r1[0][lane] : -INFINITY;
+            b2 = in ? r2[0][lane] : -INFINITY;
+            e1 = in ? r1[1][lane] : -INFINITY;
+            e2 = in ? r2[1][lane] : -INFINITY;
             dummy = lane;
             warp_best2(b1, dummy, b2);
-            const float T = b2 - margin;
+            dummy = lane;
+            warp_best2(e1, dummy, e2);
+            const float T0 = b2 - margin0, T1 = e2 - margin1;
 #pragma unroll
             for (int k = 0; k < kScanPer; ++k) {
                 const int j = t + k * kScanThreads;
                 if (j < n) {
-                    const float d2 = emd_d2(a, bx[k], by[k], bz[k]);
-                    if (list_qualifies(d2, sp[j], T)) list_append(L, i, &s_cnt, j, d2);
+                    const float p = sp[j];
+                    const float d0 = emd_d2(a0, bx[k], by[k], bz[k]);
+                    if (list_qualifies(d0, p, T0)) list_append(L, i0, &s_cnt[0], j, d0);
+                    if (i1 >= 0) {
+                        const float d1 = emd_d2(a1, bx[k], by[k], bz[k]);
+                        if (list_qualifies(d1, p, T1)) list_append(L, i1, &s_cnt[1], j, d1);
+                    }
                 }
             }
             bar_sync(2, kScanThreads);
-            list_close(L, i, s_cnt, n, T, margin, t, kScanThreads);
+            list_close(L, i0, s_cnt[0], n, T0, margin0, t, kScanThreads);
+            if (i1 >= 0) list_close(L, i1, s_cnt[1], n, T1, margin1, t, kScanThreads);
             bar_sync(1, kTailThreads);
         }
     }
