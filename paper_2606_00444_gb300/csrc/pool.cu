@@ -35,7 +35,11 @@ constexpr int kQueryWarps = 1;         // warps per block of the query kernels: 
                                        // 64-scene batch 17.4 ms against 17.8 with four)
 constexpr int kChamferWarps = 4;       // and of the Chamfer kernel (its partial sums are per 128 / G samples)
 constexpr int kPoolLeaf = 96;         // waiting leaves: below 32 before a step, at most 64 more after it
-constexpr int kPoolRing = 8;          // faces recorded per query near its least distance
+// Faces recorded per query near its least distance.  A query that meets more at
+// once is decided by resolve_ties, one thread's search: with 8 for every S, one
+// such query of 20k made the Chamfer metric 219 us long instead of 150.  Few
+// queries per warp leave room for more.
+template <int S> constexpr int kPoolRing = S == 32 ? 8 : S == 16 ? 12 : S == 8 ? 16 : 32;
 
 // An entry is a node or first leaf (30 bits), its query's slot (5 bits), a
 // face count less one (3 bits, leaves) and the box distance, its low six bits
@@ -49,10 +53,10 @@ template <int S, bool kDeep> struct __align__(16) PoolWarp {
     float4 q[S];                      // position, float32 error bound of a distance
     uint2 stack[kStack];
     uint2 leaf[kPoolLeaf];
-    uint2 ring[S][kPoolRing];         // (distance bits, leaf) of faces within the window when tested
+    uint2 ring[S][kPoolRing<S>];         // (distance bits, leaf) of faces within the window when tested
     unsigned int dmin[S];             // least squared distance, as bits
     float thr[S];                     // pruning radius, squared
-    int cnt[S];                       // faces in the ring; more than kPoolRing: some were not recorded
+    int cnt[S];                       // faces in the ring; more than kPoolRing<S>: some were not recorded
 };
 
 // What differs per query when the queries belong to several scenes.
@@ -166,14 +170,14 @@ __device__ __forceinline__ Hit pool_search(const Traversal &T, PoolWarp<S, kDeep
                     W.thr[slot] = fminf(W.thr[slot], p2);    // the same value from every lane of the slot
                     if (d2 <= w2) {
                         const int pos = atomicAdd(&W.cnt[slot], 1);
-                        if (pos < kPoolRing) W.ring[slot][pos] = make_uint2(__float_as_uint(d2), (unsigned)leaf);
+                        if (pos < kPoolRing<S>) W.ring[slot][pos] = make_uint2(__float_as_uint(d2), (unsigned)leaf);
                     }
                 }
                 __syncwarp();
                 // a ring filling up drops the faces the window has left behind
                 if (lane < S) {
                     const int m = W.cnt[lane];
-                    if (m > kPoolRing / 2 && m <= kPoolRing) {
+                    if (m > kPoolRing<S> / 2 && m <= kPoolRing<S>) {
                         const Traversal tl = scene_of(lane);
                         float w2, p2;
                         windows(__uint_as_float(W.dmin[lane]), tl.tau, W.q[lane].w, w2, p2);
@@ -244,7 +248,7 @@ __device__ __forceinline__ Hit pool_search(const Traversal &T, PoolWarp<S, kDeep
         if (m <= maxd2) {
             const Traversal t = scene_of(lane);
             const int cnt = W.cnt[lane];
-            if (cnt > kPoolRing) {
+            if (cnt > kPoolRing<S>) {
                 Best B{-1, INFINITY, m, 0.0f, -1.0f};
                 resolve_ties(t, B, q, status);
                 h.leaf = B.leaf;
@@ -259,7 +263,7 @@ __device__ __forceinline__ Hit pool_search(const Traversal &T, PoolWarp<S, kDeep
                     if (f < h.face) { h.face = f; h.leaf = (int)c.y; h.d2 = __uint_as_float(c.x); }
                 }
             }
-            if (h.leaf >= 0 && cnt > kPoolRing) h.face = face_of(t, h.leaf);
+            if (h.leaf >= 0 && cnt > kPoolRing<S>) h.face = face_of(t, h.leaf);
         }
     }
     return h;
