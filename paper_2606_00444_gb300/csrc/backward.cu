@@ -38,10 +38,7 @@ __device__ __forceinline__ void point_backward(const int4 *__restrict__ faces,
         float bb[3] = {u, v, w};
         for (int j = 0; j < 3; ++j) {
             if (bb[j] == 0.0f) continue;
-            float *p = gV + 3 * (size_t)vv[j];
-            atomicAdd(p, -bb[j] * rx);
-            atomicAdd(p + 1, -bb[j] * ry);
-            atomicAdd(p + 2, -bb[j] * rz);
+            atomic_add3(gV + 3 * (size_t)vv[j], -bb[j] * rx, -bb[j] * ry, -bb[j] * rz);
         }
     }
 }
@@ -103,10 +100,7 @@ __global__ void k_interpolate_backward(const int4 *__restrict__ faces, int nF,
     for (int j = 0; j < 3; ++j) {
         float bj = bary[3 * i + j];
         if (bj == 0.0f) continue;
-        float *p = gV + 3 * (size_t)vv[j];
-        atomicAdd(p, bj * gx);
-        atomicAdd(p + 1, bj * gy);
-        atomicAdd(p + 2, bj * gz);
+        atomic_add3(gV + 3 * (size_t)vv[j], bj * gx, bj * gy, bj * gz);
     }
 }
 

@@ -79,9 +79,7 @@ __global__ void k_batch_bind_gaussians(const int4 *__restrict__ faces, const flo
 }
 
 __device__ __forceinline__ void add_grad(float *gV, int v, V3 g) {
-    atomicAdd(gV + 3 * (size_t)v, g.x);
-    atomicAdd(gV + 3 * (size_t)v + 1, g.y);
-    atomicAdd(gV + 3 * (size_t)v + 2, g.z);
+    atomic_add3(gV + 3 * (size_t)v, g.x, g.y, g.z);
 }
 
 // VJP of the normalisation y = x / |x|: (g - y (y . g)) / |x|.

@@ -443,3 +443,20 @@ def test_chamfer_backward_entry_point_matches_oracle(pair):
     assert torch.equal(gVA2, gVA) or torch.allclose(gVA2, gVA, rtol=1e-6, atol=1e-9)
     assert not gVB2.any()
     assert A.status()[0] == 0 and B.status()[0] == 0
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2, 3])
+def test_gradient_rows_at_any_float_alignment(shift):
+    """The gradients are added in pairs where a row's floats allow it: the same sums for a
+    gradient array that starts on any 4-byte boundary, and nothing beside it."""
+    V, F = icosphere(2)
+    bvh = MeshBVH.from_mesh(dev(V), dev(F))
+    face = torch.arange(len(F), dtype=torch.int32, device="cuda")
+    bary = torch.full((len(F), 3), 0.25, device="cuda")
+    gP = torch.ones(len(F), 3, device="cuda") * torch.tensor([1.0, 2.0, 4.0], device="cuda")
+    buf = torch.zeros(3 * len(V) + 8, device="cuda")
+    gV = buf[shift:shift + 3 * len(V)].view(-1, 3)
+    bvh.interpolate_backward(face, bary, gP, gV)
+    valence = np.bincount(F.reshape(-1), minlength=len(V))
+    assert np.array_equal(gV.cpu().numpy(), 0.25 * valence[:, None] * np.array([1.0, 2.0, 4.0], np.float32))
+    assert float(buf[:shift].abs().sum() + buf[shift + 3 * len(V):].abs().sum()) == 0.0
