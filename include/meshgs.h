@@ -97,8 +97,9 @@ typedef struct {
     size_t off_iperm;    /* int32 [max_faces]   leaf of face f (inverse of perm)               */
     size_t off_adj;      /* int32 [max_faces][3] face across the edge opposite vertex k, or -1  */
     size_t off_fnorm;    /* float4 [max_faces]  unit face normals (signed distance)            */
-    size_t off_xlist;    /* bottom-up scratch: per leaf the prefix and suffix box unions
-                            inside its block of 512 leaves (2 x 32 B), the nodes whose leaf
+    size_t off_xlist;    /* bottom-up scratch: per 32 leaves the box unions of the leaves before
+                            and after them in their block of 512 leaves (2 x 32 B, in arrays
+                            sized for as much per leaf), the nodes whose leaf
                             ranges cross blocks int32x4 [max_faces] (node, range start, range
                             end, parent link), per block its box (32 B) and its count of
                             crossing nodes (int32)                                           */
@@ -196,9 +197,10 @@ mesh_status mesh_update_vertices(mesh_bvh *bvh, const float *d_V, int64_t nV, vo
  * mesh_refit(bvh, NULL, 0).  Two kernels, the same the build ends with: one
  * block per 512 consecutive leaves answers every node whose leaf range lies
  * inside the block from a sparse table of its leaf boxes in shared memory
- * (and writes each leaf's prefix and suffix union in the block), then one
- * warp per node whose range crosses blocks unions the suffix, the prefix and
- * the boxes of the blocks between.  No atomics and no waits; nothing is
+ * (and writes, per 32 leaves, the unions of the block's leaves before and
+ * after them), then one warp per node whose range crosses blocks unions the
+ * leaves of its first and last 32, those unions and the boxes of the blocks
+ * between.  No atomics and no waits; nothing is
  * derived once per topology: a refit after any build is valid. */
 mesh_status mesh_refit(mesh_bvh *bvh, const float *d_V, int64_t nV, void *stream);
 

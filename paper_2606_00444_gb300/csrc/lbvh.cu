@@ -571,12 +571,14 @@ __device__ __forceinline__ bool exactly_degenerate(float4 a, float4 b, float4 c)
 //     node's index is one end of its range, so it is in the block's index
 //     range) from two entries of level floor(log2(b - a + 1)) as soon as that
 //     level exists;
-//   * writes the prefix and suffix unions of its leaves and its own box.
+//   * writes the prefix and suffix unions of its groups of 32 leaves and its own box.
 // Every leaf and node writes its box into its parent's record half, so the
 // records need no second pass.  The nodes whose ranges cross a block boundary
 // -- a few per boundary -- are listed per block; the second kernel answers
-// each of them with one warp: suffix union in the first block, prefix union
-// in the last, and the boxes of the blocks between.  No atomics, no fences,
+// each of them with one warp: the leaves left of its first group of 32 and that
+// block's groups after it, the boxes of the blocks between, and the groups and
+// leaves of its last block.  (Unions per leaf were a third of the kernel's
+// writes, 64 of 176 bytes a leaf, for a few nodes per block.)  No atomics, no fences,
 // no spin, and the result does not depend on thread timing.  When the caller
 // passes new vertices, the first kernel also repacks them (a1) and gathers
 // the triangles from the caller's buffer.
@@ -662,10 +664,13 @@ struct Rebind {
 // degenerate flag.
 constexpr int kBindFloats = 20;
 
-constexpr size_t kRefitLocalSmem = 12 * kRefitBlock * sizeof(float)      // two table levels
-                                   + 64 * sizeof(int);                    // crossing-list scan
-constexpr size_t kRefitBindSmem = kBindFloats * kRefitBlock * sizeof(float)   // rebind records
-                                  + 64 * sizeof(int)                          // scans
+// Rows of kRefitBlock floats: two table levels (12), then each leaf's corners and
+// face id, kept from the first phase for the last; the rebind records take the
+// rows from 0 once the table is done and their thread has read its corners.
+constexpr int kRefitRows = 22, kCornerRow = 12;
+static_assert(kBindFloats <= kRefitRows, "the rebind records fit the rows");
+constexpr size_t kRefitLocalSmem = kRefitRows * kRefitBlock * sizeof(float) + 64 * sizeof(int);   // crossing-list scan
+constexpr size_t kRefitBindSmem = kRefitLocalSmem                             // (scans)
                                   + 2 * kRefitBlock * sizeof(int);            // Gaussian offsets, starts
 
 // The Gaussians of a refit block's leaves, one per thread: leaf l (this
@@ -734,7 +739,7 @@ k_refit_local(int n, const float *__restrict__ V3, int nV, float4 *__restrict__ 
     pdl_wait();
     pdl_trigger();
     float *tab = reinterpret_cast<float *>(dsm);
-    int *s_warp = reinterpret_cast<int *>(tab + (kBind ? kBindFloats : 12) * kRefitBlock);
+    int *s_warp = reinterpret_cast<int *>(tab + kRefitRows * kRefitBlock);
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int base = blockIdx.x * kRefitBlock, j = base + tid;
     // leaf j: box into level 0 and into its parent's record
@@ -743,11 +748,15 @@ k_refit_local(int n, const float *__restrict__ V3, int nV, float4 *__restrict__ 
         float4 hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.0f);
         if (j < n) {
             int pe_leaf = parent[(n - 1) + j];
+            const int f = perm[j];
             float4 a, b, c;
-            load_tri(V3, V4, faces[perm[j]], a, b, c);
+            load_tri(V3, V4, faces[f], a, b, c);
             lo = box_min(box_min(a, b), c);
             hi = box_max(box_max(a, b), c);
             put_box(nodes, hdr, pe_leaf, -(j + 1), 1, lo, hi);
+            const float r[10] = {a.x, a.y, a.z, b.x, b.y, b.z, c.x, c.y, c.z, __int_as_float(f)};
+#pragma unroll
+            for (int k = 0; k < 10; ++k) tab[(kCornerRow + k) * kRefitBlock + tid] = r[k];
         }
         SBox{tab}.put(tid, lo, hi);
     }
@@ -776,10 +785,14 @@ k_refit_local(int n, const float *__restrict__ V3, int nV, float4 *__restrict__ 
     }
     // Range queries, level by level: the union over [i0, i0 + L) with
     // 2^k <= L < 2^(k+1) is level k at i0 and at i0 + L - 2^k.  Asked here:
-    // the owned node j (its range), and leaf j's prefix [0, tid] and suffix
-    // [tid, kRefitBlock) inside the block (the block's box is the suffix of 0).
+    // the owned node j (its range), and, by the first thread of each 32 leaves, the
+    // union of the block's leaves before them and of those after them.
     const int node_level = (j < n - 1 && !cross) ? 31 - __clz(rb - ra + 1) : -1;
-    const int pre_level = 31 - __clz(tid + 1), suf_level = 31 - __clz(kRefitBlock - tid);
+    // (not for a tree of one block, whose scratch need not hold a block's groups)
+    const bool asks = lane == 0 && j < n && gridDim.x > 1;
+    const int before = asks ? tid : 0, after = asks ? kRefitBlock - 32 - tid : 0;
+    const int pre_level = before > 0 ? 31 - __clz(before) : -1, suf_level = after > 0 ? 31 - __clz(after) : -1;
+    const size_t group = (size_t)blockIdx.x * (kRefitBlock / 32) + wid;
     for (int k = 0; k <= kRefitLevels; ++k) {
         const SBox cur{tab + (k & 1) * 6 * kRefitBlock}, nxt{tab + ((k + 1) & 1) * 6 * kRefitBlock};
         const int h = 1 << k;
@@ -789,22 +802,19 @@ k_refit_local(int n, const float *__restrict__ V3, int nV, float4 *__restrict__ 
             node_link(j, ra, rb, leaf_size, link, cnt);
             put_box(nodes, hdr, pe_node, link, cnt, box_min(cur.lo(i0), cur.lo(i1)), box_max(cur.hi(i0), cur.hi(i1)));
         }
-        if (pre_level == k && j < n) {
-            int i1 = tid - h + 1;
-            pre[2 * (size_t)j] = box_min(cur.lo(0), cur.lo(i1));
-            pre[2 * (size_t)j + 1] = box_max(cur.hi(0), cur.hi(i1));
+        if (pre_level == k) {
+            const int i1 = before - h;
+            pre[2 * group] = box_min(cur.lo(0), cur.lo(i1));
+            pre[2 * group + 1] = box_max(cur.hi(0), cur.hi(i1));
         }
         if (suf_level == k) {
-            int i1 = kRefitBlock - h;
-            float4 lo = box_min(cur.lo(tid), cur.lo(i1)), hi = box_max(cur.hi(tid), cur.hi(i1));
-            if (j < n) {
-                suf[2 * (size_t)j] = lo;
-                suf[2 * (size_t)j + 1] = hi;
-            }
-            if (tid == 0) {
-                bbox[2 * blockIdx.x] = lo;
-                bbox[2 * blockIdx.x + 1] = hi;
-            }
+            const int i0 = tid + 32, i1 = kRefitBlock - h;
+            suf[2 * group] = box_min(cur.lo(i0), cur.lo(i1));
+            suf[2 * group + 1] = box_max(cur.hi(i0), cur.hi(i1));
+        }
+        if (k == kRefitLevels && tid == 0) {
+            bbox[2 * blockIdx.x] = cur.lo(0);
+            bbox[2 * blockIdx.x + 1] = cur.hi(0);
         }
         if (k == 1 && cross)                             // offsets written by warp 0 in round 0
             xlist[base + s_warp[32 + wid] + __popc(ball & ((1u << lane) - 1u))] = make_int4(j, ra, rb, pe_node);
@@ -817,10 +827,13 @@ k_refit_local(int n, const float *__restrict__ V3, int nV, float4 *__restrict__ 
     int gs = 0, gcnt = 0;                                // kBind: this leaf's Gaussians
     if constexpr (kBind) __syncthreads();                // the table is read no more: records go there
     if (j < n) {
-        int f = perm[j];                                 // reloaded: cheaper than keeping it live
+        float r0[10];                                    // kept in shared memory: cheaper than live registers
+#pragma unroll
+        for (int k = 0; k < 10; ++k) r0[k] = tab[(kCornerRow + k) * kRefitBlock + tid];
+        const int f = __float_as_int(r0[9]);
         iperm[f] = j;
-        float4 a, b, c;
-        load_tri(V3, V4, faces[f], a, b, c);
+        const float4 a = make_float4(r0[0], r0[1], r0[2], 0.0f), b = make_float4(r0[3], r0[4], r0[5], 0.0f),
+                     c = make_float4(r0[6], r0[7], r0[8], 0.0f);
         float deg = exactly_degenerate(a, b, c) ? 1.0f : 0.0f;
         tris[3 * (size_t)j + 0] = make_float4(a.x, a.y, a.z, __int_as_float(f));
         tris[3 * (size_t)j + 1] = make_float4(b.x, b.y, b.z, deg);
@@ -849,14 +862,15 @@ k_refit_local(int n, const float *__restrict__ V3, int nV, float4 *__restrict__ 
     }
 }
 
-// One warp per crossing node: the suffix union in its first block, the prefix
-// union in its last, and the boxes of the blocks between.
+// One warp per crossing node: a lane per leaf of its first and of its last 32, the
+// unions of the other groups of those two blocks, and the boxes of the blocks
+// between.
 constexpr int kTopThreads = 256;
 
 __global__ void __launch_bounds__(kTopThreads)
 k_refit_top(const int4 *__restrict__ xlist, const int *__restrict__ xcnt, const float4 *__restrict__ pre,
-            const float4 *__restrict__ suf, const float4 *__restrict__ bbox, float4 *__restrict__ nodes,
-            Header *__restrict__ hdr, int leaf_size) {
+            const float4 *__restrict__ suf, const float4 *__restrict__ bbox, const float4 *__restrict__ tris,
+            float4 *__restrict__ nodes, Header *__restrict__ hdr, int leaf_size) {
     pdl_wait();
     pdl_trigger();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = kTopThreads >> 5;
@@ -865,9 +879,23 @@ k_refit_top(const int4 *__restrict__ xlist, const int *__restrict__ xcnt, const 
         int4 e = xlist[(size_t)blockIdx.x * kRefitBlock + r];   // node, range start, range end, parent
         float4 lo = make_float4(INFINITY, INFINITY, INFINITY, 0.0f);
         float4 hi = make_float4(-INFINITY, -INFINITY, -INFINITY, 0.0f);
-        if (lane == 0) {
-            lo = box_min(__ldcg(suf + 2 * (size_t)e.y), __ldcg(pre + 2 * (size_t)e.z));
-            hi = box_max(__ldcg(suf + 2 * (size_t)e.y + 1), __ldcg(pre + 2 * (size_t)e.z + 1));
+        // e.y and e.z lie in different blocks, so both groups of 32 are whole up to the range's end
+        const int jy = (e.y & ~31) + lane, jz = (e.z & ~31) + lane;
+        auto leaf = [&](int j) {
+            const float4 *t = tris + 3 * (size_t)j;
+            const float4 a = __ldcg(t), b = __ldcg(t + 1), c = __ldcg(t + 2);
+            lo = box_min(lo, box_min(box_min(a, b), c));
+            hi = box_max(hi, box_max(box_max(a, b), c));
+        };
+        if (jy >= e.y) leaf(jy);
+        if (jz <= e.z) leaf(jz);
+        if (lane == 0 && (e.y % kRefitBlock) / 32 + 1 < kRefitBlock / 32) {
+            lo = box_min(lo, __ldcg(suf + 2 * (size_t)(e.y / 32)));
+            hi = box_max(hi, __ldcg(suf + 2 * (size_t)(e.y / 32) + 1));
+        }
+        if (lane == 1 && (e.z % kRefitBlock) / 32 > 0) {
+            lo = box_min(lo, __ldcg(pre + 2 * (size_t)(e.z / 32)));
+            hi = box_max(hi, __ldcg(pre + 2 * (size_t)(e.z / 32) + 1));
         }
         for (int b = e.y / kRefitBlock + 1 + lane; b < e.z / kRefitBlock; b += 32) {
             lo = box_min(lo, __ldcg(bbox + 2 * b));
@@ -1231,9 +1259,10 @@ static mesh_batch_layout batch_layout(int64_t maxB, int64_t maxV, int64_t maxF) 
     return L;
 }
 
-// Scratch of the bottom-up kernels: prefix and suffix unions of the leaf
-// boxes inside each block (2 float4 per leaf each), the crossing nodes (int4
-// per face), the blocks' boxes (2 float4 each) and the per-block counts.
+// Scratch of the bottom-up kernels: per 32 leaves the unions of their block's
+// leaves before and after them (2 float4 each, at the start of two arrays with
+// room for that much per leaf), the crossing nodes (int4 per face), the blocks'
+// boxes (2 float4 each) and the per-block counts.
 static int64_t refit_blocks(int64_t f) { return (f + kRefitBlock - 1) / kRefitBlock; }
 static size_t xlist_bytes(int64_t f) {
     int64_t nb = refit_blocks(f);
@@ -1576,7 +1605,7 @@ static mesh_status bottom_up(mesh_bvh *bvh, const float *V3, cudaStream_t s,
         bvh->leaf_size);
     count_launch();
     if (nb > 1) {
-        pdl_launch(k_refit_top, nb, kTopThreads, 0, s, xlist, xcnt, pre, suf, bbox, bvh->nodes(), bvh->hdr(),
+        pdl_launch(k_refit_top, nb, kTopThreads, 0, s, xlist, xcnt, pre, suf, bbox, bvh->tris(), bvh->nodes(), bvh->hdr(),
                    bvh->leaf_size);
         count_launch();
     }
