@@ -460,3 +460,23 @@ def test_gradient_rows_at_any_float_alignment(shift):
     valence = np.bincount(F.reshape(-1), minlength=len(V))
     assert np.array_equal(gV.cpu().numpy(), 0.25 * valence[:, None] * np.array([1.0, 2.0, 4.0], np.float32))
     assert float(buf[:shift].abs().sum() + buf[shift + 3 * len(V):].abs().sum()) == 0.0
+
+
+@pytest.mark.parametrize("shift", [0, 1, 2])
+def test_gaussians_into_arrays_at_any_float_alignment(shift):
+    """The rotations are stored whole where their array is 16-byte aligned: the same
+    Gaussians, and nothing beside them, from either form and either entry point."""
+    V, F = icosphere(3)
+    bvh = MeshBVH.from_mesh(dev(V), dev(F))
+    n = len(F)
+    gface = torch.arange(n, dtype=torch.int32, device="cuda")
+    gbary = torch.full((n, 3), 1 / 3, device="cuda")
+    ref = bvh.bind_gaussians(gface, gbary)
+    for call in (lambda out: bvh.bind_gaussians(gface, gbary, out=out),
+                 lambda out: bvh.refit_bind(dev(V), torch.arange(n + 1, dtype=torch.int32, device="cuda"), gbary, out=out)):
+        bufs = [torch.zeros(c * n + 8, device="cuda") for c in (3, 4, 3)]
+        out = tuple(b[shift:shift + c * n].view(n, c) for b, c in zip(bufs, (3, 4, 3)))
+        call(out)
+        for got, want, b in zip(out, ref, bufs):
+            assert torch.equal(got, want)
+            assert float(b[:shift].abs().sum() + b[shift + want.numel():].abs().sum()) == 0.0
