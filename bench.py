@@ -1280,7 +1280,8 @@ def main():
     rec = contact_traffic(res["tuned"]) if res["tuned"]["lanes"] == 1 else None
     rec = rec or {}
     dram, lts = rec.get("dram_bytes"), rec.get("lts_bytes")
-    roof = {"kernel": f"k_closest_point {traversal_label(res['tuned'])} (contact, 1M queries, "
+    roof = {"kernel": f"{'k_pool_closest_point' if res['tuned']['variant'] == 0 else 'k_closest_point'} "
+                      f"{traversal_label(res['tuned'])} (contact, 1M queries, "
                       f"no warm start, frame {ROOF_FRAME})",
             "ms": res["roof_ms"],
             "bound": "l2", "achieved": achieved, "peak": l2, "unit": "GB/s", "frac": achieved / l2,

@@ -113,6 +113,7 @@ k_emd_bid(int n, const float4 *__restrict__ A4, const float4 *__restrict__ B4, c
     }
     if (lane == 0) {
         atomicAdd(active, 1u);
+        if ((unsigned)j1 >= (unsigned)n) return;     // no comparable value (NaN input): no bid
         float inc = (b2 == -INFINITY ? 0.0f : b1 - b2) + eps;
         float bid = price[j1] + inc;
         atomicMax(&bids[j1], ((unsigned long long)__float_as_uint(bid) << 32) | (unsigned)i);
