@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <utility>
 
 #include "meshgs.h"
@@ -129,6 +130,20 @@ template <typename... KArgs, typename... Args>
 inline void pdl_launch(void (*kernel)(KArgs...), unsigned int grid, unsigned int block, size_t smem, cudaStream_t s,
                        Args &&...args) {
     launch_ex(true, kernel, grid, block, smem, s, std::forward<Args>(args)...);
+}
+
+// Lets `kernel` take `bytes` of dynamic shared memory on the current device; done:
+// the devices where it may already, one bit each (the setting is per device).
+template <typename... KArgs>
+inline bool allow_smem(void (*kernel)(KArgs...), size_t bytes, std::atomic<unsigned long long> &done) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return false;
+    const unsigned long long bit = dev < 64 ? 1ull << dev : 0ull;
+    if (bit && (done.load() & bit)) return true;
+    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes) != cudaSuccess)
+        return false;
+    done.fetch_or(bit);
+    return true;
 }
 
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }

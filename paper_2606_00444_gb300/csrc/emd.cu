@@ -782,9 +782,8 @@ mesh_status mesh_emd(const float *d_A, const float *d_B, int64_t n, float eps_re
     if (!(C > 0.0)) C = 1.0;
     const double eps_final = eps_rel * C;
     const unsigned bid_grid = grid_for(N, kEmdWarps);
-    static const bool tail_ok =                       // the dynamic shared memory the tail takes
-        cudaFuncSetAttribute(k_emd_tail, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * kTailMaxN) == cudaSuccess;
-    if (!tail_ok) return MESH_ERR_CUDA;
+    static std::atomic<unsigned long long> tail_smem{0};
+    if (!allow_smem(k_emd_tail, 8 * (size_t)kTailMaxN, tail_smem)) return MESH_ERR_CUDA;
     if (lists) {
         // a first guess of the margin: about 1 % of the box diagonal's objects at 10k points
         k_emd_lists_init<<<grid_for(N, 256), 256, 0, s>>>(N, w.L, (float)(0.25 * C * sqrt(160.0 / (double)N)));

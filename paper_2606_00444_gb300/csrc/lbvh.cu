@@ -1149,9 +1149,8 @@ static void sort_passes(const BuildWs &w, int n, int shift0, const unsigned int 
         constexpr int TH = th.value, IT = it.value;
         using Smem = SortSmem<TH, IT>;
         auto kern = k_sort_pass<TH, IT, kGrouped>;
-        static const cudaError_t set =
-            cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
-        (void)set;                                       // a failure shows as the launch's
+        static std::atomic<unsigned long long> smem{0};
+        allow_smem(kern, sizeof(Smem), smem);            // a failure shows as the launch's
         const unsigned int *ki = kin;
         const int *vi = vin;
         for (int p = 0; p < H.passes; ++p) {
@@ -1581,15 +1580,10 @@ mesh_status mesh_update_vertices(mesh_bvh *bvh, const float *d_V, int64_t nV, vo
 // Launches the two bottom-up kernels (build and refit); V3 = new vertices or NULL.
 static mesh_status bottom_up(mesh_bvh *bvh, const float *V3, cudaStream_t s,
                              Rebind rb = Rebind{nullptr, nullptr, nullptr, 0, nullptr, nullptr, nullptr}) {
-    static bool smem_set = false;                    // the dynamic shared memory the kernels take
-    if (!smem_set) {
-        if (cudaFuncSetAttribute(k_refit_local<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kRefitLocalSmem) != cudaSuccess ||
-            cudaFuncSetAttribute(k_refit_local<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)kRefitBindSmem) != cudaSuccess)
-            return MESH_ERR_CUDA;
-        smem_set = true;
-    }
+    static std::atomic<unsigned long long> smem{0}, smem_bind{0};
+    if (!allow_smem(k_refit_local<false>, kRefitLocalSmem, smem) ||
+        !allow_smem(k_refit_local<true>, kRefitBindSmem, smem_bind))
+        return MESH_ERR_CUDA;
     int n = (int)bvh->L.n_faces;
     bvh->wide_valid = false;
     unsigned int nb = grid_for(n, kRefitBlock);
