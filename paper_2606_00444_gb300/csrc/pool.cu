@@ -35,11 +35,10 @@ constexpr int kQueryWarps = 1;         // warps per block of the query kernels: 
                                        // 64-scene batch 17.4 ms against 17.8 with four)
 constexpr int kChamferWarps = 4;       // and of the Chamfer kernel (its partial sums are per 128 / G samples)
 constexpr int kPoolLeaf = 96;         // waiting leaves: below 32 before a step, at most 64 more after it
-// Faces recorded per query near its least distance.  A query that meets more at
-// once is decided by resolve_ties, one thread's search: with 8 for every S, one
-// such query of 20k made the Chamfer metric 219 us long instead of 150.  Few
-// queries per warp leave room for more.
+// Faces recorded per query near its least distance; a query that meets more keeps
+// those that can still be its answer (pool_absorb).
 template <int S> constexpr int kPoolRing = S == 32 ? 8 : S == 16 ? 12 : S == 8 ? 16 : 32;
+constexpr int kPoolLost = 1 << 20;    // a count from which on faces were not recorded
 
 // An entry is a node or first leaf (30 bits), its query's slot (5 bits), a
 // face count less one (3 bits, leaves) and the box distance, its low six bits
@@ -56,7 +55,7 @@ template <int S, bool kDeep> struct __align__(16) PoolWarp {
     uint2 ring[S][kPoolRing<S>];         // (distance bits, leaf) of faces within the window when tested
     unsigned int dmin[S];             // least squared distance, as bits
     float thr[S];                     // pruning radius, squared
-    int cnt[S];                       // faces in the ring; more than kPoolRing<S>: some were not recorded
+    int cnt[S];                       // faces in the ring; kPoolLost or more: some were not recorded
 };
 
 // What differs per query when the queries belong to several scenes.
@@ -73,6 +72,59 @@ __device__ __forceinline__ int pool_id(uint2 e) { return (int)(e.x & 0x3fffffffu
 __device__ __forceinline__ int pool_slot(uint2 e) { return (int)((e.x >> 30) | (e.y >> 1 & 0x1cu)); }
 __device__ __forceinline__ int pool_count(uint2 e) { return (int)(e.y & 7u) + 1; }
 __device__ __forceinline__ float pool_dist(uint2 e) { return __uint_as_float(e.y & ~63u); }
+
+// Makes room in the rings of the queries that have just met more faces than their
+// rings hold; each such face waits in the lane that tested it (over: slot, d2, leaf,
+// face).  Of two recorded faces the farther one with the higher id is never the
+// answer, whatever the final window: what remains is a front of falling ids over
+// rising distances, one face where many are exactly as far (the faces around a
+// vertex).  A window is 2e-6 of a squared distance wide, some 17 to 34 float32
+// values, and a front of ids in no order is the logarithm of that; one longer than
+// the ring is left to resolve_ties.
+//
+// The search itself may not be left to resolve_ties: it is one lane's depth-first
+// search while the warp waits.  On the axis through a vertex of 512 faces 100 queries
+// took 181 us so and 20k 1211, now 46 and 279; 100 queries 1000 radii from a sphere
+// of 82k faces (hundreds of faces tie in float32) 443 us, now 54.
+template <int S, bool kDeep, bool kScenes>
+static __device__ __noinline__ void pool_absorb(const float4 *tris, float tau, PoolWarp<S, kDeep> &W,
+                                                const PoolScene<S> *sc, bool over, int slot, float d2, int leaf,
+                                                int face) {
+    const unsigned int kFull = 0xffffffffu, kNone = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    unsigned int todo = __ballot_sync(kFull, over);
+    while (todo) {
+        const int sl = __shfl_sync(kFull, slot, __ffs(todo) - 1);
+        const bool mine = over && slot == sl;
+        todo &= ~__ballot_sync(kFull, mine);
+        if (W.cnt[sl] >= kPoolLost) continue;                // decided by resolve_ties already
+        const float4 *t = kScenes ? tris + 3 * (size_t)sc->base[sl] : tris;
+        float w2, p2;
+        windows(__uint_as_float(W.dmin[sl]), kScenes ? sc->tau[sl] : tau, W.q[sl].w, w2, p2);
+        // the candidates: a ring entry and a waiting face per lane (a full ring: every entry is set)
+        const uint2 e = W.ring[sl][lane < kPoolRing<S> ? lane : 0];
+        unsigned int ed = lane < kPoolRing<S> && __uint_as_float(e.x) <= w2 ? e.x : kNone;
+        unsigned int nd = mine && d2 <= w2 ? __float_as_uint(d2) : kNone;
+        const unsigned int ef = ed != kNone ? __float_as_uint(ldg4(t + 3 * (size_t)e.y).w) : kNone;
+        const unsigned int nf = (unsigned)face;
+        __syncwarp();                                        // read before the entries are written again
+        int n = 0;
+        while (true) {                                       // the nearest left, and of those the lowest id
+            const unsigned int m = __reduce_min_sync(kFull, min(ed, nd));
+            if (m == kNone) break;
+            const unsigned int f = __reduce_min_sync(kFull, min(ed == m ? ef : kNone, nd == m ? nf : kNone));
+            if (n < kPoolRing<S>) {
+                if (ed == m && ef == f) W.ring[sl][n] = e;
+                if (nd == m && nf == f) W.ring[sl][n] = make_uint2(m, (unsigned)leaf);
+            }
+            ++n;
+            if (ef >= f) ed = kNone;
+            if (nf >= f) nd = kNone;
+        }
+        if (lane == 0) W.cnt[sl] = n <= kPoolRing<S> ? n : kPoolLost;
+        __syncwarp();
+    }
+}
 
 // The search of a warp's S queries; lane l < S brings query l (valid or not; T
 // holds its mesh's scale and size) and takes its hit.  hint: a leaf tested first, or -1.  descend: a query without a
@@ -156,40 +208,30 @@ __device__ __forceinline__ Hit pool_search(const Traversal &T, PoolWarp<S, kDeep
             for (int k = 0; k < most; ++k) {
                 const int leaf = pool_id(e) + k;
                 float d2 = INFINITY;
-                bool test = k < cnt;
+                int face = 0;
+                const bool test = k < cnt;
                 if (test) {
                     const float4 *tr = t.tris + 3 * (size_t)leaf;
                     const float4 a = ldg4(tr), b = ldg4(tr + 1), c = ldg4(tr + 2);
                     d2 = tri_distance2(p, xyz(a), xyz(b), xyz(c), b.w != 0.0f);
+                    face = __float_as_int(a.w);
                     atomicMin(&W.dmin[slot], __float_as_uint(d2));
                 }
                 __syncwarp();
+                bool over = false;                           // met, and the ring is full
                 if (test) {
                     float w2, p2;
                     windows(__uint_as_float(W.dmin[slot]), t.tau, qs.w, w2, p2);
                     W.thr[slot] = fminf(W.thr[slot], p2);    // the same value from every lane of the slot
                     if (d2 <= w2) {
                         const int pos = atomicAdd(&W.cnt[slot], 1);
-                        if (pos < kPoolRing<S>) W.ring[slot][pos] = make_uint2(__float_as_uint(d2), (unsigned)leaf);
+                        over = pos >= kPoolRing<S>;
+                        if (!over) W.ring[slot][pos] = make_uint2(__float_as_uint(d2), (unsigned)leaf);
                     }
                 }
                 __syncwarp();
-                // a ring filling up drops the faces the window has left behind
-                if (lane < S) {
-                    const int m = W.cnt[lane];
-                    if (m > kPoolRing<S> / 2 && m <= kPoolRing<S>) {
-                        const Traversal tl = scene_of(lane);
-                        float w2, p2;
-                        windows(__uint_as_float(W.dmin[lane]), tl.tau, W.q[lane].w, w2, p2);
-                        int keep = 0;
-                        for (int j = 0; j < m; ++j) {
-                            const uint2 c = W.ring[lane][j];
-                            if (__uint_as_float(c.x) <= w2) W.ring[lane][keep++] = c;
-                        }
-                        W.cnt[lane] = keep;
-                    }
-                }
-                __syncwarp();
+                if (__any_sync(kFull, over))
+                    pool_absorb<S, kDeep, kScenes>(T.tris, T.tau, W, sc, over, slot, d2, leaf, face);
             }
             continue;
         }
@@ -248,7 +290,7 @@ __device__ __forceinline__ Hit pool_search(const Traversal &T, PoolWarp<S, kDeep
         if (m <= maxd2) {
             const Traversal t = scene_of(lane);
             const int cnt = W.cnt[lane];
-            if (cnt > kPoolRing<S>) {
+            if (cnt >= kPoolLost) {
                 Best B{-1, INFINITY, m, 0.0f, -1.0f};
                 resolve_ties(t, B, q, status);
                 h.leaf = B.leaf;
@@ -263,7 +305,7 @@ __device__ __forceinline__ Hit pool_search(const Traversal &T, PoolWarp<S, kDeep
                     if (f < h.face) { h.face = f; h.leaf = (int)c.y; h.d2 = __uint_as_float(c.x); }
                 }
             }
-            if (h.leaf >= 0 && cnt > kPoolRing<S>) h.face = face_of(t, h.leaf);
+            if (h.leaf >= 0 && cnt >= kPoolLost) h.face = face_of(t, h.leaf);
         }
     }
     return h;

@@ -127,3 +127,57 @@ def test_knn_lists_are_the_k_least_distances(n, k, leaf):
         assert np.array_equal(d2[:m, :c].cpu().numpy(), np.take_along_axis(each, order, 1))
         assert (face[:, c:] == -1).all() and torch.isinf(d2[:, c:]).all()
         assert bvh.status()[0] == 0
+
+
+@pytest.mark.parametrize("lanes", LANES)
+@pytest.mark.parametrize("leaf", [1, 4])
+def test_fronts_of_falling_ids_over_rising_distances(lanes, leaf):
+    """Layers of faces one float32 step apart, the nearer ones with the higher ids: up to 17
+    of them lie inside a tie window and none rules out another, more than the rings of 8, 12
+    and 16 hold (the search is then decided by resolve_ties); with the ids in no order a few
+    remain.  Each layer is three copies, so that many faces are met at once."""
+    base = np.float32(0.99999)
+    z = -(base + np.arange(40, dtype=np.float32) * np.float32(2.0 ** -24))
+    V = np.stack([[[-9, -9, h], [9, -9, h], [0, 9, h]] for h in z]).reshape(-1, 3).astype(np.float32)
+    layers = np.arange(120, dtype=np.int32).reshape(40, 3)
+    rng = np.random.default_rng(2)
+    falling = np.repeat(layers[::-1], 3, 0)               # the nearest layer last
+    for F in (falling, falling[rng.permutation(120)]):
+        bvh = MeshBVH.from_mesh(dev(V), dev(np.ascontiguousarray(F)))
+        bvh.set_leaf_size(leaf)
+        Q = np.zeros((70, 3), np.float32)
+        Q[:, :2] = rng.uniform(-1, 1, (70, 2))
+        Q[::2, 2] = rng.uniform(0, 1, 35)
+        for md in (float("inf"), 1.5):
+            assert_identical(pooled(bvh, dev(Q), md, lanes), one_thread(bvh, dev(Q), md))
+        assert bvh.status()[0] == 0
+
+
+def _best_ms(fn, repeats=12):
+    fn()
+    ts = []
+    for _ in range(repeats):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        fn()
+        b.record()
+        b.synchronize()
+        ts.append(a.elapsed_time(b))
+    return min(ts)
+
+
+def test_tied_faces_are_not_left_to_one_lane():
+    """From 1000 radii away hundreds of faces of a sphere lie inside the tie window: 100 such
+    queries take at most 4 times as long as 100 from 3 radii (they meet more faces; with the
+    ties left to one lane's search they took 11 times as long)."""
+    V, F = icosphere(6)
+    bvh = MeshBVH.from_mesh(dev(V), dev(F))
+    d = np.random.default_rng(0).normal(size=(100, 3))
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    ms = []
+    for r in (3.0, 1000.0):
+        Q = dev((d * r).astype(np.float32))
+        out = bvh.closest_point(Q)
+        assert_identical(out, one_thread(bvh, Q, float("inf")))
+        ms.append(_best_ms(lambda: bvh.closest_point(Q, out=out)))
+    assert ms[1] <= 4 * ms[0], ms
