@@ -44,11 +44,12 @@ constexpr int kPoolLost = 1 << 20;    // a count from which on faces were not re
 // face count less one (3 bits, leaves) and the box distance, its low six bits
 // rounded off: an entry's distance only ever rounds down, so it is never
 // dropped too early.
-template <int S, bool kDeep> struct __align__(16) PoolWarp {
-    // Node entries.  A depth-first search deep inside a mesh defers about 20 siblings, one under a
-    // cutoff few; what the stacks leave of an SM's memory caches the tree.
-    static constexpr int kStack = S == 32 ? 448 : S == 16 ? (kDeep ? 512 : 320) : S == 8 ? (kDeep ? 384 : 256)
-                                  : S == 4 ? (kDeep ? 320 : 192) : kDeep ? 256 : 160;
+template <int S> struct __align__(16) PoolWarp {
+    // Node entries.  A depth-first search deep inside a mesh defers about 20 siblings; a warp whose
+    // stack fills up goes on with fewer lanes, down to one.  What the stacks leave of an SM's memory
+    // caches the tree, but a third less stack for searches under a cutoff gained nothing (1M contacts
+    // 555 us, 539 with these) and made those under a loose one up to 5 times as long.
+    static constexpr int kStack = S == 32 ? 448 : S == 16 ? 512 : S == 8 ? 384 : S == 4 ? 320 : 256;
     float4 q[S];                      // position, float32 error bound of a distance
     uint2 stack[kStack];
     uint2 leaf[kPoolLeaf];
@@ -86,8 +87,8 @@ __device__ __forceinline__ float pool_dist(uint2 e) { return __uint_as_float(e.y
 // search while the warp waits.  On the axis through a vertex of 512 faces 100 queries
 // took 181 us so and 20k 1211, now 46 and 279; 100 queries 1000 radii from a sphere
 // of 82k faces (hundreds of faces tie in float32) 443 us, now 54.
-template <int S, bool kDeep, bool kScenes>
-static __device__ __noinline__ void pool_absorb(const float4 *tris, float tau, PoolWarp<S, kDeep> &W,
+template <int S, bool kScenes>
+static __device__ __noinline__ void pool_absorb(const float4 *tris, float tau, PoolWarp<S> &W,
                                                 const PoolScene<S> *sc, bool over, int slot, float d2, int leaf,
                                                 int face) {
     const unsigned int kFull = 0xffffffffu, kNone = 0xffffffffu;
@@ -126,15 +127,26 @@ static __device__ __noinline__ void pool_absorb(const float4 *tris, float tau, P
     }
 }
 
+// A cutoff is loose when the ball of that radius may hold more faces than a search
+// should meet without a nearer radius: about n r^2 / diag^2 of a surface of n faces,
+// some three times that for a closed one.  Lines at 50, 200 and 1000 measured the same
+// for tight cutoffs (1M signed queries, cutoff 0.05 of a 3.9 diagonal: 302 to 314 us);
+// 50k queries near a 5k-face torus, cutoff 0.7 (160 by this estimate), took 79, 202 and
+// 204 us.  With no rule a loose cutoff cost 2 to 18 times one thread per query (1M
+// queries near the 200k-face torus, cutoff 2.0: 19.9 ms against 1.2; 0.96 now).
+constexpr float kLooseFaces = 50.0f;
+
 // The search of a warp's S queries; lane l < S brings query l (valid or not; T
-// holds its mesh's scale and size) and takes its hit.  hint: a leaf tested first, or -1.  descend: a query without a
-// hint first goes down the nearer children to one leaf, so that the pool
-// starts with a radius for each query (unbounded searches).
+// holds its mesh's scale and size) and takes its hit.  hint: a leaf tested first, or -1.  A query without a
+// hint starts at the first node with two children inside the cutoff (descend: at the
+// root), which ends most misses at once; when the cutoff is loose or there is none
+// (descend) it then goes down the nearer children to one leaf, so that the pool
+// starts with a radius for it.
 // sc: per-query offsets into T's arrays (queries of several scenes), or NULL.
-template <int S, bool kDeep, bool kRange, bool kScenes>
-__device__ __forceinline__ Hit pool_search(const Traversal &T, PoolWarp<S, kDeep> &W, PoolScene<S> *sc, float3 q, bool valid,
+template <int S, bool kRange, bool kScenes>
+__device__ __forceinline__ Hit pool_search(const Traversal &T, PoolWarp<S> &W, PoolScene<S> *sc, float3 q, bool valid,
                                            float maxd2, int hint, bool descend, unsigned int *status) {
-    constexpr int kStack = PoolWarp<S, kDeep>::kStack;
+    constexpr int kStack = PoolWarp<S>::kStack;
     const unsigned int kFull = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const unsigned int lt = (1u << lane) - 1u;
@@ -158,32 +170,56 @@ __device__ __forceinline__ Hit pool_search(const Traversal &T, PoolWarp<S, kDeep
         if constexpr (kScenes) sc->tau[lane] = T.tau;        // base is set by the caller
     }
     __syncwarp();
-    int first = -1, first_cnt = 1;                           // the leaf this query tests first
+    int first = -1, first_cnt = 1, root = -1;                // the leaf this query tests first, the node it starts from
     if (mine) {
-        if (hint >= 0) {
-            first = hint;
-        } else if (T.n == 1) {
+        if (T.n == 1) {
             first = 0;
-        } else if (descend) {
+        } else if (hint >= 0) {
+            first = hint;
+            root = 0;
+        } else {
             const Traversal t = scene_of(lane);
+            const float thr = W.thr[lane];
+            // down to the first node with two children inside the cutoff
             int node = 0;
-            while (true) {
+            while (node >= 0 && !descend) {
                 const float4 *r = t.nodes + 4 * (size_t)node;
                 const float4 l0 = ldg4(r), l1 = ldg4(r + 1), r0 = ldg4(r + 2), r1 = ldg4(r + 3);
-                const float dl = box_d2(q, l0, l1), dr = box_d2(q, r0, r1);
-                bool left = dl < dr;
-                if (dl == dr) left = box_minmax_d2(q, l0, l1) <= box_minmax_d2(q, r0, r1);
-                const int c = __float_as_int(left ? l0.w : r0.w);
-                if (c >= 0) { node = c; continue; }
-                first = -c - 1;
-                if constexpr (kRange) first_cnt = __float_as_int(left ? l1.w : r1.w);
-                break;
+                const bool il = box_d2(q, l0, l1) <= thr, ir = box_d2(q, r0, r1) <= thr;
+                if (il && ir) break;
+                node = -1;
+                if (il || ir) {
+                    const int c = __float_as_int(il ? l0.w : r0.w);
+                    if (c >= 0) {
+                        node = c;
+                    } else {
+                        first = -c - 1;
+                        if constexpr (kRange) first_cnt = __float_as_int(il ? l1.w : r1.w);
+                    }
+                }
+            }
+            root = node;
+            // a radius, where the cutoff leaves many faces: down the nearer children to a leaf
+            const float diag = T.tau * (1.0f / kTieAbs);
+            if (node >= 0 && (descend || maxd2 * (float)T.n > kLooseFaces * diag * diag)) {
+                while (true) {
+                    const float4 *r = t.nodes + 4 * (size_t)node;
+                    const float4 l0 = ldg4(r), l1 = ldg4(r + 1), r0 = ldg4(r + 2), r1 = ldg4(r + 3);
+                    const float dl = box_d2(q, l0, l1), dr = box_d2(q, r0, r1);
+                    bool left = dl < dr;
+                    if (dl == dr) left = box_minmax_d2(q, l0, l1) <= box_minmax_d2(q, r0, r1);
+                    const int c = __float_as_int(left ? l0.w : r0.w);
+                    if (c >= 0) { node = c; continue; }
+                    first = -c - 1;
+                    if constexpr (kRange) first_cnt = __float_as_int(left ? l1.w : r1.w);
+                    break;
+                }
             }
         }
     }
-    const unsigned int fm = __ballot_sync(kFull, first >= 0), rm = __ballot_sync(kFull, mine && T.n > 1);
+    const unsigned int fm = __ballot_sync(kFull, first >= 0), rm = __ballot_sync(kFull, root >= 0);
     if (first >= 0) W.leaf[__popc(fm & lt)] = pool_entry(first, lane, first_cnt - 1, 0.0f);
-    if (mine && T.n > 1) W.stack[__popc(rm & lt)] = pool_entry(0, lane, 0, 0.0f);
+    if (root >= 0) W.stack[__popc(rm & lt)] = pool_entry(root, lane, 0, 0.0f);
     int nleaf = __popc(fm), nstack = __popc(rm);
     bool start = nleaf > 0;                                  // the first leaves are tested before any node
     __syncwarp();
@@ -231,7 +267,7 @@ __device__ __forceinline__ Hit pool_search(const Traversal &T, PoolWarp<S, kDeep
                 }
                 __syncwarp();
                 if (__any_sync(kFull, over))
-                    pool_absorb<S, kDeep, kScenes>(T.tris, T.tau, W, sc, over, slot, d2, leaf, face);
+                    pool_absorb<S, kScenes>(T.tris, T.tau, W, sc, over, slot, d2, leaf, face);
             }
             continue;
         }
@@ -312,12 +348,12 @@ __device__ __forceinline__ Hit pool_search(const Traversal &T, PoolWarp<S, kDeep
 }
 
 // The queries of a warp: S consecutive ones.
-template <int S, bool kDeep, bool kRange>
+template <int S, bool kRange>
 __global__ void __launch_bounds__(32 * kQueryWarps, 32 / kQueryWarps)
 k_pool_closest_point(Traversal T, const Header *__restrict__ hdr, unsigned int *status, const float *__restrict__ Q,
                      int64_t nQ, float maxd2, int *face, float *bary, float *point, float *dist2, const int *hint,
                      const int *__restrict__ iperm) {
-    __shared__ PoolWarp<S, kDeep> s_pool[kQueryWarps];
+    __shared__ PoolWarp<S> s_pool[kQueryWarps];
     pdl_wait();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t i0 = ((int64_t)blockIdx.x * kQueryWarps + wid) * S, i = i0 + lane;
@@ -330,19 +366,19 @@ k_pool_closest_point(Traversal T, const Header *__restrict__ hdr, unsigned int *
         const int hf = hint[i];
         if (hf >= 0 && hf < T.n) hl = __ldg(iperm + hf);
     }
-    const Hit h = pool_search<S, kDeep, kRange, false>(T, s_pool[wid], nullptr, q, valid, maxd2, hl, T.mmd, status);
+    const Hit h = pool_search<S, kRange, false>(T, s_pool[wid], nullptr, q, valid, maxd2, hl, T.mmd, status);
     if (valid) write_hit(T, h, q, i, face, bary, point, dist2);
 }
 
 // Queries of many scenes (mesh_batch_closest_point): each lane finds its query's
 // scene, and the pool's entries carry scene-local nodes.
-template <int S, bool kDeep>
+template <int S>
 __global__ void __launch_bounds__(32 * kQueryWarps, 32 / kQueryWarps)
 k_pool_batch(const float4 *__restrict__ nodes, const float4 *__restrict__ tris, const float4 *__restrict__ scene_box,
              const int *__restrict__ face_off, const int *__restrict__ query_off, int nscenes,
              const float *__restrict__ Q, int64_t nQ, float maxd2, bool mmd, int *face, float *bary, float *point,
              float *dist2, unsigned int *status) {
-    __shared__ PoolWarp<S, kDeep> s_pool[kQueryWarps];
+    __shared__ PoolWarp<S> s_pool[kQueryWarps];
     __shared__ PoolScene<S> s_scene[kQueryWarps];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t i0 = ((int64_t)blockIdx.x * kQueryWarps + wid) * S, i = i0 + lane;
@@ -359,7 +395,7 @@ k_pool_batch(const float4 *__restrict__ nodes, const float4 *__restrict__ tris, 
         q = make_float3(Q[3 * i], Q[3 * i + 1], Q[3 * i + 2]);
     }
     if (lane < S) s_scene[wid].base[lane] = fb;
-    Hit h = pool_search<S, kDeep, false, true>(T, s_pool[wid], &s_scene[wid], q, valid, maxd2, -1, mmd, status);
+    Hit h = pool_search<S, false, true>(T, s_pool[wid], &s_scene[wid], q, valid, maxd2, -1, mmd, status);
     if (!valid) return;
     if (h.leaf >= 0) h.face -= fb;
     T.tris += 3 * (size_t)fb;
@@ -389,7 +425,7 @@ template <int S, bool kRange>
 __global__ void __launch_bounds__(32 * kChamferWarps, 32 / kChamferWarps)
 k_pool_chamfer(ChamferSide A2B, ChamferSide B2A, unsigned int nbA, unsigned int *status, double *partial,
                unsigned int *ticket, double *out) {
-    __shared__ PoolWarp<S, true> s_pool[kChamferWarps];
+    __shared__ PoolWarp<S> s_pool[kChamferWarps];
     __shared__ double s_red[kChamferWarps];
     __shared__ bool s_last;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -407,7 +443,7 @@ k_pool_chamfer(ChamferSide A2B, ChamferSide B2A, unsigned int nbA, unsigned int 
             const int hf = C.hint[i];
             if (hf >= 0 && hf < T.n) hl = __ldg(C.iperm + hf);
         }
-        const Hit h = pool_search<S, true, kRange, false>(T, s_pool[wid], nullptr, q, valid, INFINITY, hl, true, status);
+        const Hit h = pool_search<S, kRange, false>(T, s_pool[wid], nullptr, q, valid, INFINITY, hl, true, status);
         if (valid) {
             write_hit(T, h, q, i, C.face, C.bary, nullptr, C.dist2);
             d2 = h.leaf >= 0 ? (double)h.d2 : 0.0;
@@ -540,20 +576,20 @@ static __device__ __noinline__ float signed_of_hit(const Traversal &T, Hit h, fl
     return (dn >= 0.0f ? 1.0f : -1.0f) * sqrtf(h.d2);
 }
 
-template <int S, bool kDeep, bool kRange>
+template <int S, bool kRange>
 __global__ void __launch_bounds__(32 * kQueryWarps, 32 / kQueryWarps)
 k_pool_signed(Traversal T, const Header *__restrict__ hdr, unsigned int *status, const float *__restrict__ Q,
               int64_t nQ, float maxd2, const int4 *__restrict__ faces, const int *__restrict__ adj,
               const float4 *__restrict__ fnorm, const float4 *__restrict__ verts, int *face, float *bary,
               float *point, float *sdist) {
-    __shared__ PoolWarp<S, kDeep> s_pool[kQueryWarps];
+    __shared__ PoolWarp<S> s_pool[kQueryWarps];
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const int64_t i0 = ((int64_t)blockIdx.x * kQueryWarps + wid) * S, i = i0 + lane;
     if (i0 >= nQ) return;
     const bool valid = lane < S && i < nQ;
     set_scale(T, hdr);
     const float3 q = valid ? make_float3(Q[3 * i], Q[3 * i + 1], Q[3 * i + 2]) : make_float3(0.0f, 0.0f, 0.0f);
-    const Hit h = pool_search<S, kDeep, kRange, false>(T, s_pool[wid], nullptr, q, valid, maxd2, -1, T.mmd, status);
+    const Hit h = pool_search<S, kRange, false>(T, s_pool[wid], nullptr, q, valid, maxd2, -1, T.mmd, status);
     if (!valid) return;
     write_hit(T, h, q, i, face, bary, point, nullptr);
     sdist[i] = h.leaf < 0 ? INFINITY : signed_of_hit(T, h, q, faces, adj, fnorm, verts, status);
@@ -813,10 +849,7 @@ void pool_closest_point(const mesh_bvh *b, Traversal T, const float *Q, int64_t 
                         float *bary, float *point, float *dist2, const int *hint, cudaStream_t s) {
     Header *h = b->hdr();
     pool_dispatch(G, [&](auto S) {
-        auto kern = b->leaf_size > 1 ? (T.mmd ? k_pool_closest_point<S.value, true, true>
-                                              : k_pool_closest_point<S.value, false, true>)
-                                     : (T.mmd ? k_pool_closest_point<S.value, true, false>
-                                              : k_pool_closest_point<S.value, false, false>);
+        auto kern = b->leaf_size > 1 ? k_pool_closest_point<S.value, true> : k_pool_closest_point<S.value, false>;
         kern<<<grid_for(nQ, kQueryWarps * S.value), 32 * kQueryWarps, 0, s>>>(T, h, &h->status, Q, nQ, maxd2, face, bary,
                                                                        point, dist2, hint, b->iperm());
     });
@@ -827,8 +860,7 @@ void pool_signed(const mesh_bvh *b, Traversal T, const float *Q, int64_t nQ, flo
                  float *point, float *sdist, cudaStream_t s) {
     Header *h = b->hdr();
     pool_dispatch(G, [&](auto S) {
-        auto kern = b->leaf_size > 1 ? (T.mmd ? k_pool_signed<S.value, true, true> : k_pool_signed<S.value, false, true>)
-                                     : (T.mmd ? k_pool_signed<S.value, true, false> : k_pool_signed<S.value, false, false>);
+        auto kern = b->leaf_size > 1 ? k_pool_signed<S.value, true> : k_pool_signed<S.value, false>;
         kern<<<grid_for(nQ, kQueryWarps * S.value), 32 * kQueryWarps, 0, s>>>(T, h, &h->status, Q, nQ, maxd2, b->faces(),
                                                                        b->adj(), b->fnorm(), b->verts(), face, bary,
                                                                        point, sdist);
@@ -861,8 +893,7 @@ void pool_chamfer(int G, bool range, const ChamferSide &a2b, const ChamferSide &
 void pool_batch(const mesh_batch *b, const float *Q, const int *query_off, int64_t nQ, float maxd2, bool mmd, int G,
                 int *face, float *bary, float *point, float *dist2, cudaStream_t s) {
     pool_dispatch(G, [&](auto S) {
-        auto kern = mmd ? k_pool_batch<S.value, true> : k_pool_batch<S.value, false>;
-        kern<<<grid_for(nQ, kQueryWarps * S.value), 32 * kQueryWarps, 0, s>>>(
+        k_pool_batch<S.value><<<grid_for(nQ, kQueryWarps * S.value), 32 * kQueryWarps, 0, s>>>(
             b->nodes(), b->tris(), b->scene_box(), b->face_off(), query_off, (int)b->L.n_scenes, Q, nQ, maxd2, mmd,
             face, bary, point, dist2, &b->st()->status);
     });

@@ -181,3 +181,38 @@ def test_tied_faces_are_not_left_to_one_lane():
         assert_identical(out, one_thread(bvh, Q, float("inf")))
         ms.append(_best_ms(lambda: bvh.closest_point(Q, out=out)))
     assert ms[1] <= 4 * ms[0], ms
+
+
+@pytest.mark.parametrize("n", [100, 50_000])
+@pytest.mark.parametrize("signed", [False, True])
+def test_loose_cutoffs_cost_no_more_than_none(n, signed):
+    """A cutoff that every query's answer meets by far prunes nothing by itself: the search
+    takes at most 1.5 times the time of the one without a cutoff (it took 3 to 20 times as
+    long when it started without a radius)."""
+    V, F = icosphere(6)
+    bvh = MeshBVH.from_mesh(dev(V), dev(F))
+    rng = np.random.default_rng(n)
+    Q = dev((V[rng.integers(0, len(V), n)] + rng.normal(size=(n, 3)) * 0.02).astype(np.float32))
+    find = bvh.signed_distance if signed else bvh.closest_point
+    ref = find(Q)
+    free_ms = _best_ms(lambda: find(Q, out=ref))
+    for md in (0.3, 0.7, 2.0):
+        got = find(Q, md)
+        assert_identical(got, ref)
+        assert _best_ms(lambda: find(Q, md, out=got)) <= 1.5 * free_ms
+
+
+def test_searches_under_a_cutoff_from_wherever_they_start():
+    """Cutoffs from none of the mesh to all of it (the search starts at the first node with two
+    children inside, or ends there; a loose cutoff first goes down to a leaf), with and
+    without hints and leaf ranges: the one-thread search's answers."""
+    V, F = displaced_icosphere(4, 0.1, 0.4)
+    for faces, leaf in ((len(F), 1), (len(F), 4), (2, 1), (3, 4)):
+        bvh = MeshBVH.from_mesh(dev(V), dev(np.ascontiguousarray(F[:faces])))
+        bvh.set_leaf_size(leaf)
+        Q = dev(np.concatenate([uniform_box(3000, [-1.5] * 3, [1.5] * 3, seed=4), np.full((3, 3), 1e6)]).astype(np.float32))
+        for md in (0.0, 1e-3, 0.02, 0.1, 0.3, 1.0, 5.0, 1e9):
+            ref = one_thread(bvh, Q, md)
+            for lanes in (-1, 2, 32):
+                assert_identical(pooled(bvh, Q, md, lanes), ref)
+                assert_identical(pooled(bvh, Q, md, lanes, hint=ref["face"]), ref)
