@@ -488,8 +488,11 @@ __device__ __forceinline__ void write_hit(const Traversal &T, const Hit &h, floa
     if (bary || point) write_weights(T, h.leaf, h.d2, q, i, bary, point);
 }
 
-// The pooled search (pool.cu) with G lanes per query (a power of two to 32; 1 =
-// 32 queries per warp).
+// The pooled search (pool.cu) with G lanes per query (a power of two from 2 to 32; the
+// Chamfer kernel also 1, 32 queries per warp).  G = 0: the mesh has at most kFewFaces
+// faces (a batch's scenes on average), each tested by a thread per query; the Chamfer
+// kernel then takes 128 samples per block.
+constexpr int kFewFaces = 24;
 void pool_closest_point(const mesh_bvh *b, Traversal T, const float *Q, int64_t nQ, float maxd2, int G, int *face,
                         float *bary, float *point, float *dist2, const int *hint, cudaStream_t s);
 void pool_signed(const mesh_bvh *b, Traversal T, const float *Q, int64_t nQ, float maxd2, int G, int *face, float *bary,

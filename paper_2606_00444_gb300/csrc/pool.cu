@@ -1,7 +1,7 @@
 // NearestSurface by warps that pool the work of several queries.
 //
-// A warp holds S queries (32 when there are many, fewer when the queries would
-// not fill the GPU) and one stack of (node, query) entries for all of them.
+// A warp holds S queries (16 when there are many, fewer when the queries would
+// not fill the GPU; 32 in the largest calls of mesh_chamfer_noalloc) and one stack of (node, query) entries for all of them.
 // Each step its 32 lanes take the top 32 entries, whoever they belong to: a lane
 // reads one node record (two child boxes), tests both against its entry's query
 // and pruning radius, and the surviving children go back on the stack -- the
@@ -135,6 +135,18 @@ static __device__ __noinline__ void pool_absorb(const float4 *tris, float tau, P
 // 204 us.  With no rule a loose cutoff cost 2 to 18 times one thread per query (1M
 // queries near the 200k-face torus, cutoff 2.0: 19.9 ms against 1.2; 0.96 now).
 constexpr float kLooseFaces = 50.0f;
+
+// Meshes of at most kFewFaces faces: a thread per query tests every face.  A warp
+// of the pool spends more on starting and ending its queries than such a search
+// takes (300k queries of one face: 60 us in the Chamfer kernel's pool, 34 so; figures
+// over sizes at pool_lanes).  Bound by the tests, some 100 instructions each.
+constexpr int kFewThreads = 128;
+
+__device__ __forceinline__ Hit few_search(const Traversal &T, float3 q, float maxd2, unsigned int *status) {
+    Best B = make_best(T, q, maxd2);
+    for (int leaf = 0; leaf < T.n; ++leaf) test_leaf(T, B, leaf, q, maxd2);
+    return finish(T, B, q, status);
+}
 
 // The search of a warp's S queries; lane l < S brings query l (valid or not; T
 // holds its mesh's scale and size) and takes its hit.  hint: a leaf tested first, or -1.  A query without a
@@ -370,18 +382,28 @@ k_pool_closest_point(Traversal T, const Header *__restrict__ hdr, unsigned int *
     if (valid) write_hit(T, h, q, i, face, bary, point, dist2);
 }
 
+__global__ void __launch_bounds__(kFewThreads)
+k_few_closest_point(Traversal T, const Header *__restrict__ hdr, unsigned int *status, const float *__restrict__ Q,
+                    int64_t nQ, float maxd2, int *face, float *bary, float *point, float *dist2) {
+    const int64_t i = (int64_t)blockIdx.x * kFewThreads + threadIdx.x;
+    if (i >= nQ) return;
+    set_scale(T, hdr);
+    const float3 q = make_float3(Q[3 * i], Q[3 * i + 1], Q[3 * i + 2]);
+    write_hit(T, few_search(T, q, maxd2, status), q, i, face, bary, point, dist2);
+}
+
 // Queries of many scenes (mesh_batch_closest_point): each lane finds its query's
 // scene, and the pool's entries carry scene-local nodes.
 template <int S>
-__global__ void __launch_bounds__(32 * kQueryWarps, 32 / kQueryWarps)
+__global__ void __launch_bounds__(32, 32)
 k_pool_batch(const float4 *__restrict__ nodes, const float4 *__restrict__ tris, const float4 *__restrict__ scene_box,
              const int *__restrict__ face_off, const int *__restrict__ query_off, int nscenes,
              const float *__restrict__ Q, int64_t nQ, float maxd2, bool mmd, int *face, float *bary, float *point,
              float *dist2, unsigned int *status) {
-    __shared__ PoolWarp<S> s_pool[kQueryWarps];
-    __shared__ PoolScene<S> s_scene[kQueryWarps];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int64_t i0 = ((int64_t)blockIdx.x * kQueryWarps + wid) * S, i = i0 + lane;
+    __shared__ PoolWarp<S> s_pool;
+    __shared__ PoolScene<S> s_scene;
+    const int lane = threadIdx.x;
+    const int64_t i0 = (int64_t)blockIdx.x * S, i = i0 + lane;
     if (i0 >= nQ) return;
     const bool valid = lane < S && i < nQ;
     Traversal T{nodes, tris, 0, 0.0f, 0.0f, mmd, nullptr};
@@ -394,9 +416,65 @@ k_pool_batch(const float4 *__restrict__ nodes, const float4 *__restrict__ tris, 
         set_scale(T, scene_box[2 * sc], scene_box[2 * sc + 1]);
         q = make_float3(Q[3 * i], Q[3 * i + 1], Q[3 * i + 2]);
     }
-    if (lane < S) s_scene[wid].base[lane] = fb;
-    Hit h = pool_search<S, false, true>(T, s_pool[wid], &s_scene[wid], q, valid, maxd2, -1, mmd, status);
+    if (lane < S) s_scene.base[lane] = fb;
+    Hit h = pool_search<S, false, true>(T, s_pool, &s_scene, q, valid, maxd2, -1, mmd, status);
     if (!valid) return;
+    if (h.leaf >= 0) h.face -= fb;
+    T.tris += 3 * (size_t)fb;
+    write_hit(T, h, q, i, face, bary, point, dist2);
+}
+
+// The same for batches whose scenes have at most kFewFaces faces on average: a thread
+// per query of such a scene; the queries of the others go to the pool, half a warp
+// at a time.
+__global__ void __launch_bounds__(32, 32)
+k_few_batch(const float4 *__restrict__ nodes, const float4 *__restrict__ tris, const float4 *__restrict__ scene_box,
+            const int *__restrict__ face_off, const int *__restrict__ query_off, int nscenes,
+            const float *__restrict__ Q, int64_t nQ, float maxd2, bool mmd, int *face, float *bary, float *point,
+            float *dist2, unsigned int *status) {
+    constexpr int S = 16;
+    __shared__ PoolWarp<S> s_pool;
+    __shared__ PoolScene<S> s_scene;
+    const unsigned int kFull = 0xffffffffu;
+    const int lane = threadIdx.x;
+    const int64_t i = (int64_t)blockIdx.x * 32 + lane;
+    Traversal T{nodes, tris, 0, 0.0f, 0.0f, mmd, nullptr};
+    float3 q = make_float3(0.0f, 0.0f, 0.0f);
+    int fb = 0;
+    if (i < nQ) {
+        const int sc = segment_of(query_off, nscenes, i);
+        fb = __ldg(face_off + sc);
+        T.n = __ldg(face_off + sc + 1) - fb;
+        set_scale(T, scene_box[2 * sc], scene_box[2 * sc + 1]);
+        q = make_float3(Q[3 * i], Q[3 * i + 1], Q[3 * i + 2]);
+    }
+    Hit h{-1, 0x7fffffff, INFINITY};
+    if (T.n > 0 && T.n <= kFewFaces) {
+        Traversal own = T;
+        own.tris += 3 * (size_t)fb;
+        own.nodes += 4 * (size_t)fb;
+        h = few_search(own, q, maxd2, status);
+    }
+    for (int half = 0; half < 2; ++half) {
+        const bool mine = T.n > kFewFaces && lane / S == half;
+        if (!__any_sync(kFull, mine)) continue;
+        const int src = half * S + lane % S;                 // lanes 0 to 15 take the half's queries
+        const bool valid = __shfl_sync(kFull, (int)mine, src) && lane < S;
+        const float3 qh = make_float3(__shfl_sync(kFull, q.x, src), __shfl_sync(kFull, q.y, src),
+                                      __shfl_sync(kFull, q.z, src));
+        Traversal Th = T;
+        Th.n = __shfl_sync(kFull, T.n, src);
+        Th.tau = __shfl_sync(kFull, T.tau, src);
+        Th.vmax = __shfl_sync(kFull, T.vmax, src);
+        const int fh = __shfl_sync(kFull, fb, src);
+        if (lane < S) s_scene.base[lane] = fh;
+        const Hit g = pool_search<S, false, true>(Th, s_pool, &s_scene, qh, valid, maxd2, -1, mmd, status);
+        const int leaf = __shfl_sync(kFull, g.leaf, lane % S), f = __shfl_sync(kFull, g.face, lane % S);
+        const float d2 = __shfl_sync(kFull, g.d2, lane % S);
+        if (mine) h = Hit{leaf, f, d2};
+        __syncwarp();
+    }
+    if (i >= nQ) return;
     if (h.leaf >= 0) h.face -= fb;
     T.tris += 3 * (size_t)fb;
     write_hit(T, h, q, i, face, bary, point, dist2);
@@ -421,29 +499,36 @@ __device__ __forceinline__ double block_sum_d(double x, double *s) {
     return t;
 }
 
+// S = 0: both meshes have few faces, a thread per sample.
 template <int S, bool kRange>
 __global__ void __launch_bounds__(32 * kChamferWarps, 32 / kChamferWarps)
 k_pool_chamfer(ChamferSide A2B, ChamferSide B2A, unsigned int nbA, unsigned int *status, double *partial,
                unsigned int *ticket, double *out) {
-    __shared__ PoolWarp<S> s_pool[kChamferWarps];
+    constexpr int kOwn = S == 0 ? 32 : S;                    // samples of a warp
     __shared__ double s_red[kChamferWarps];
     __shared__ bool s_last;
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const bool first = blockIdx.x < nbA;
     const ChamferSide &C = first ? A2B : B2A;
-    const int64_t i0 = ((int64_t)(first ? blockIdx.x : blockIdx.x - nbA) * kChamferWarps + wid) * S, i = i0 + lane;
-    const bool valid = lane < S && i < C.n;
+    const int64_t i0 = ((int64_t)(first ? blockIdx.x : blockIdx.x - nbA) * kChamferWarps + wid) * kOwn, i = i0 + lane;
+    const bool valid = lane < kOwn && i < C.n;
     double d2 = 0.0;
     if (i0 < C.n) {                                          // uniform in the warp
         Traversal T = C.T;
         set_scale(T, C.hdr);
         const float3 q = valid ? make_float3(C.S[3 * i], C.S[3 * i + 1], C.S[3 * i + 2]) : make_float3(0.0f, 0.0f, 0.0f);
-        int hl = -1;
-        if (valid && C.hint) {
-            const int hf = C.hint[i];
-            if (hf >= 0 && hf < T.n) hl = __ldg(C.iperm + hf);
+        Hit h{-1, 0x7fffffff, INFINITY};
+        if constexpr (S == 0) {
+            if (valid) h = few_search(T, q, INFINITY, status);
+        } else {
+            __shared__ PoolWarp<S> s_pool[kChamferWarps];
+            int hl = -1;
+            if (valid && C.hint) {
+                const int hf = C.hint[i];
+                if (hf >= 0 && hf < T.n) hl = __ldg(C.iperm + hf);
+            }
+            h = pool_search<S, kRange, false>(T, s_pool[wid], nullptr, q, valid, INFINITY, hl, true, status);
         }
-        const Hit h = pool_search<S, kRange, false>(T, s_pool[wid], nullptr, q, valid, INFINITY, hl, true, status);
         if (valid) {
             write_hit(T, h, q, i, C.face, C.bary, nullptr, C.dist2);
             d2 = h.leaf >= 0 ? (double)h.d2 : 0.0;
@@ -591,6 +676,20 @@ k_pool_signed(Traversal T, const Header *__restrict__ hdr, unsigned int *status,
     const float3 q = valid ? make_float3(Q[3 * i], Q[3 * i + 1], Q[3 * i + 2]) : make_float3(0.0f, 0.0f, 0.0f);
     const Hit h = pool_search<S, kRange, false>(T, s_pool[wid], nullptr, q, valid, maxd2, -1, T.mmd, status);
     if (!valid) return;
+    write_hit(T, h, q, i, face, bary, point, nullptr);
+    sdist[i] = h.leaf < 0 ? INFINITY : signed_of_hit(T, h, q, faces, adj, fnorm, verts, status);
+}
+
+__global__ void __launch_bounds__(kFewThreads)
+k_few_signed(Traversal T, const Header *__restrict__ hdr, unsigned int *status, const float *__restrict__ Q,
+             int64_t nQ, float maxd2, const int4 *__restrict__ faces, const int *__restrict__ adj,
+             const float4 *__restrict__ fnorm, const float4 *__restrict__ verts, int *face, float *bary, float *point,
+             float *sdist) {
+    const int64_t i = (int64_t)blockIdx.x * kFewThreads + threadIdx.x;
+    if (i >= nQ) return;
+    set_scale(T, hdr);
+    const float3 q = make_float3(Q[3 * i], Q[3 * i + 1], Q[3 * i + 2]);
+    const Hit h = few_search(T, q, maxd2, status);
     write_hit(T, h, q, i, face, bary, point, nullptr);
     sdist[i] = h.leaf < 0 ? INFINITY : signed_of_hit(T, h, q, faces, adj, fnorm, verts, status);
 }
@@ -833,10 +932,9 @@ k_pool_knn(Traversal T, const Header *__restrict__ hdr, const float *Q, int64_t 
     }
 }
 
-// Calls f with S = 32 / G as a compile-time constant.
+// Calls f with S = 32 / G as a compile-time constant (G of 2 or more).
 template <typename F> static void pool_dispatch(int G, F f) {
     switch (G) {
-        case 1: f(std::integral_constant<int, 32>()); break;
         case 2: f(std::integral_constant<int, 16>()); break;
         case 4: f(std::integral_constant<int, 8>()); break;
         case 8: f(std::integral_constant<int, 4>()); break;
@@ -848,24 +946,34 @@ template <typename F> static void pool_dispatch(int G, F f) {
 void pool_closest_point(const mesh_bvh *b, Traversal T, const float *Q, int64_t nQ, float maxd2, int G, int *face,
                         float *bary, float *point, float *dist2, const int *hint, cudaStream_t s) {
     Header *h = b->hdr();
+    count_launch();
+    if (G == 0) {
+        k_few_closest_point<<<grid_for(nQ, kFewThreads), kFewThreads, 0, s>>>(T, h, &h->status, Q, nQ, maxd2, face, bary,
+                                                                              point, dist2);
+        return;
+    }
     pool_dispatch(G, [&](auto S) {
         auto kern = b->leaf_size > 1 ? k_pool_closest_point<S.value, true> : k_pool_closest_point<S.value, false>;
         kern<<<grid_for(nQ, kQueryWarps * S.value), 32 * kQueryWarps, 0, s>>>(T, h, &h->status, Q, nQ, maxd2, face, bary,
                                                                        point, dist2, hint, b->iperm());
     });
-    count_launch();
 }
 
 void pool_signed(const mesh_bvh *b, Traversal T, const float *Q, int64_t nQ, float maxd2, int G, int *face, float *bary,
                  float *point, float *sdist, cudaStream_t s) {
     Header *h = b->hdr();
+    count_launch();
+    if (G == 0) {
+        k_few_signed<<<grid_for(nQ, kFewThreads), kFewThreads, 0, s>>>(T, h, &h->status, Q, nQ, maxd2, b->faces(), b->adj(),
+                                                                       b->fnorm(), b->verts(), face, bary, point, sdist);
+        return;
+    }
     pool_dispatch(G, [&](auto S) {
         auto kern = b->leaf_size > 1 ? k_pool_signed<S.value, true> : k_pool_signed<S.value, false>;
         kern<<<grid_for(nQ, kQueryWarps * S.value), 32 * kQueryWarps, 0, s>>>(T, h, &h->status, Q, nQ, maxd2, b->faces(),
                                                                        b->adj(), b->fnorm(), b->verts(), face, bary,
                                                                        point, sdist);
     });
-    count_launch();
 }
 
 void pool_knn(const mesh_bvh *b, Traversal T, const float *Q, int64_t nQ, int k, int G, const float *anchor,
@@ -883,21 +991,26 @@ void pool_knn(const mesh_bvh *b, Traversal T, const float *Q, int64_t nQ, int k,
 
 void pool_chamfer(int G, bool range, const ChamferSide &a2b, const ChamferSide &b2a, unsigned nbA, unsigned grid,
                   unsigned *status, double *partial, unsigned *ticket, double *out, cudaStream_t s) {
-    pool_dispatch(G, [&](auto S) {
+    auto go = [&](auto S) {
         auto kern = range ? k_pool_chamfer<S.value, true> : k_pool_chamfer<S.value, false>;
         kern<<<grid, 32 * kChamferWarps, 0, s>>>(a2b, b2a, nbA, status, partial, ticket, out);
-    });
+    };
     count_launch();
+    if (G == 0) k_pool_chamfer<0, false><<<grid, 32 * kChamferWarps, 0, s>>>(a2b, b2a, nbA, status, partial, ticket, out);
+    else if (G == 1) go(std::integral_constant<int, 32>());   // mesh_chamfer_noalloc's largest calls
+    else pool_dispatch(G, go);
 }
 
 void pool_batch(const mesh_batch *b, const float *Q, const int *query_off, int64_t nQ, float maxd2, bool mmd, int G,
                 int *face, float *bary, float *point, float *dist2, cudaStream_t s) {
-    pool_dispatch(G, [&](auto S) {
-        k_pool_batch<S.value><<<grid_for(nQ, kQueryWarps * S.value), 32 * kQueryWarps, 0, s>>>(
-            b->nodes(), b->tris(), b->scene_box(), b->face_off(), query_off, (int)b->L.n_scenes, Q, nQ, maxd2, mmd,
-            face, bary, point, dist2, &b->st()->status);
-    });
     count_launch();
+    auto go = [&](auto kern, int queries) {
+        kern<<<grid_for(nQ, queries), 32, 0, s>>>(b->nodes(), b->tris(), b->scene_box(), b->face_off(), query_off,
+                                                  (int)b->L.n_scenes, Q, nQ, maxd2, mmd, face, bary, point, dist2,
+                                                  &b->st()->status);
+    };
+    if (G == 0) go(k_few_batch, 32);
+    else pool_dispatch(G, [&](auto S) { go(k_pool_batch<S.value>, S.value); });
 }
 
 }  // namespace meshgs

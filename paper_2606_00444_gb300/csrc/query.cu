@@ -668,8 +668,8 @@ void meshgs::wide_refresh(const mesh_bvh *b, cudaStream_t s, bool pdl) {
 
 namespace meshgs {
 
-static size_t chamfer_blocks(int64_t n, int G = 1) {
-    return (size_t)((n * G + kQueryBlock - 1) / kQueryBlock);
+static size_t chamfer_blocks(int64_t n, int G) {         // of 128 / G samples (G = 0: 128)
+    return (size_t)((n * (G > 0 ? G : 1) + kQueryBlock - 1) / kQueryBlock);
 }
 
 // The one-thread searches' weights in their own launch after the search (k_hit_weights).
@@ -704,8 +704,13 @@ static int fill_lanes(int64_t nQ) {
 // took 289 / 267 / 349 us with 32 / 16 / 8 queries per warp under a cutoff and
 // 6.3 / 4.5 / 4.3 ms without; 20k took 97 / 58 / 50 / 40 / 44 / 56 us with 32 ... 1
 // (2 by this rule), 5k 68 ... 27 us (1 by this rule: 27).
-static int pool_lanes(int64_t nQ) {
+// Meshes of few faces do without (0): 12 faces, 300k queries 74 us with it, 35 without (one
+// thread per query of the tree 87), 50k signed distances 54 and 22 (30), 100 queries 13 and
+// 13; 20 faces, 50k queries 36 and 21 (52), 100 queries 11 and 17 (15); 40 faces, 300k
+// queries 74 and 93 (162).
+static int pool_lanes(int64_t nQ, int64_t n_faces) {
     const int G = fill_lanes(nQ);
+    if (n_faces <= (G <= 8 ? kFewFaces : 16)) return 0;
     return G > 2 ? G : 2;
 }
 
@@ -718,7 +723,7 @@ mesh_status launch_signed_query(const mesh_bvh *bvh, const float *d_Q, int64_t n
                                 cudaStream_t s) {
     const bool unbounded = isinf(max_dist);
     pool_signed(bvh, traversal_of(bvh, unbounded), d_Q, nQ, unbounded ? INFINITY : max_dist * max_dist,
-                pool_lanes(nQ), d_face, d_bary, d_point, d_sdist, s);
+                pool_lanes(nQ, bvh->L.n_faces), d_face, d_bary, d_point, d_sdist, s);
     return check_launch();
 }
 
@@ -828,7 +833,10 @@ static void launch_contact(Traversal T, Header *h, const float *d_Q, int64_t nQ,
 
 // Lanes per sample of the Chamfer searches (unbounded), unless the process-wide
 // setting names more than one.
-static int chamfer_lanes(int64_t n) { return g_group_override > 1 ? g_group_override : pool_lanes(n); }
+static int chamfer_lanes(const mesh_bvh *A, const mesh_bvh *B, int64_t n) {
+    const int64_t most = A->L.n_faces > B->L.n_faces ? A->L.n_faces : B->L.n_faces;
+    return g_group_override > 1 ? g_group_override : pool_lanes(n, most);
+}
 
 static mesh_status run_chamfer(const mesh_bvh *A, const float *SA, int64_t nSA, const mesh_bvh *B, const float *SB,
                                int64_t nSB, int G, double *partial, unsigned int *ticket, double *out,
@@ -886,8 +894,8 @@ mesh_status mesh_closest_point_hinted(const mesh_bvh *bvh, const float *d_Q, int
     if (one && variant == 13) ensure_wide(bvh, s);
     Traversal T = traversal_of(bvh, isinf(max_dist));
     if (!one) {
-        pool_closest_point(bvh, T, d_Q, nQ, maxd2, lanes > 1 ? lanes : pool_lanes(nQ), d_face, d_bary, d_point,
-                           d_dist2, d_hint, s);
+        pool_closest_point(bvh, T, d_Q, nQ, maxd2, lanes > 1 ? lanes : pool_lanes(nQ, bvh->L.n_faces), d_face, d_bary,
+                           d_point, d_dist2, d_hint, s);
         return check_launch();
     }
     // the one-thread depth-first searches write face and distance; the weights and
@@ -1024,8 +1032,8 @@ mesh_status mesh_knn_project(const mesh_bvh *bvh, const float *d_Q, int64_t nQ, 
         return MESH_ERR_INVALID_ARG;
     if (nQ == 0) return MESH_OK;
     if (!d_Q || !d_point) return MESH_ERR_INVALID_ARG;
-    pool_knn(bvh, traversal_of(bvh, false), d_Q, nQ, k, pool_lanes(nQ), d_anchor, anchor_weight, d_point, d_face, d_dist2,
-             (cudaStream_t)stream);
+    pool_knn(bvh, traversal_of(bvh, false), d_Q, nQ, k, pool_lanes(nQ, bvh->L.n_faces), d_anchor, anchor_weight, d_point,
+             d_face, d_dist2, (cudaStream_t)stream);
     return check_launch();
 }
 
@@ -1105,7 +1113,7 @@ mesh_status mesh_chamfer_hinted(const mesh_bvh *A, const float *d_SA, int64_t nS
     if (!d_ws || ws_bytes < need || ((uintptr_t)d_ws & 255u)) return MESH_ERR_WORKSPACE;
     double *partial = (double *)d_ws;
     unsigned int *ticket = (unsigned int *)((char *)d_ws + need - 256);
-    return run_chamfer(A, d_SA, nSA, B, d_SB, nSB, chamfer_lanes(nSA + nSB), partial, ticket, d_out, d_hintA, d_hintB,
+    return run_chamfer(A, d_SA, nSA, B, d_SB, nSB, chamfer_lanes(A, B, nSA + nSB), partial, ticket, d_out, d_hintA, d_hintB,
                        d_faceA, d_baryA, d_dist2A, d_faceB, d_baryB, d_dist2B, (cudaStream_t)stream);
 }
 
@@ -1136,8 +1144,8 @@ mesh_status mesh_batch_closest_point(mesh_batch *batch, const float *d_Q,
     if (nQ == 0) return MESH_OK;
     const bool unbounded = isinf(max_dist);
     pool_batch(batch, d_Q, d_query_off, nQ, unbounded ? INFINITY : max_dist * max_dist, unbounded,
-               pool_lanes(nQ), d_face,
-               d_bary, d_point, d_dist2, (cudaStream_t)stream);
+               pool_lanes(nQ, batch->L.n_faces / (batch->L.n_scenes > 0 ? batch->L.n_scenes : 1)), d_face, d_bary,
+               d_point, d_dist2, (cudaStream_t)stream);
     return check_launch();
 }
 
@@ -1256,7 +1264,7 @@ extern "C" mesh_status mesh_chamfer_noalloc(const mesh_bvh *A, const float *d_SA
     if (!A || !B || !d_out || nSA < 0 || nSB < 0 || (nSA > 0 && !d_SA) || (nSB > 0 && !d_SB))
         return MESH_ERR_INVALID_ARG;
     // the lanes per sample mesh_chamfer would use, fewer if its blocks exceed the array
-    int G = chamfer_lanes(nSA + nSB);
+    int G = chamfer_lanes(A, B, nSA + nSB);
     while (G > 1 && chamfer_blocks(nSA, G) + chamfer_blocks(nSB, G) > (size_t)kNoAllocMaxBlocks) G >>= 1;
     size_t nbA = chamfer_blocks(nSA, G), nbB = chamfer_blocks(nSB, G);
     if (nbA + nbB > (size_t)kNoAllocMaxBlocks) return MESH_ERR_WORKSPACE;

@@ -216,3 +216,63 @@ def test_searches_under_a_cutoff_from_wherever_they_start():
             for lanes in (-1, 2, 32):
                 assert_identical(pooled(bvh, Q, md, lanes), ref)
                 assert_identical(pooled(bvh, Q, md, lanes, hint=ref["face"]), ref)
+
+
+@pytest.mark.parametrize("faces", [1, 2, 16, 17, 24, 25])
+def test_meshes_of_few_faces(faces):
+    """Up to 16 faces (24 with many queries) a thread per query tests them all: closest points,
+    signed distances and Chamfer samples equal the one-thread search's, faces tied or not."""
+    from paper_2606_00444_gb300 import chamfer
+    V, F = displaced_icosphere(1, 0.1, 0.4)
+    F = np.ascontiguousarray(F[:faces])
+    for Fm in (F, np.repeat(F[:1], faces, 0)):
+        bvh = MeshBVH.from_mesh(dev(V), dev(np.ascontiguousarray(Fm)))
+        for n in (1, 127, 129, 50_001):
+            Q = dev(uniform_box(n, [-1.5] * 3, [1.5] * 3, seed=n))
+            for md in (float("inf"), 0.5, 0.0):
+                ref = one_thread(bvh, Q, md)
+                assert_identical(bvh.closest_point(Q, md), ref)
+                assert_identical(bvh.signed_distance(Q, md), ref)
+            out, ps = chamfer(bvh, Q, bvh, Q, per_sample=True)
+            ref = one_thread(bvh, Q, float("inf"))
+            assert torch.equal(ps["faceA"], ref["face"]) and torch.equal(ps["dist2B"], ref["dist2"])
+            assert torch.allclose(out, ref["dist2"].double().mean().expand(2), rtol=1e-12)
+        assert bvh.status()[0] & ~8 == 0                   # (8: copies of a face are no manifold)
+
+
+def test_batch_of_mostly_few_faces():
+    """Scenes of few faces on average, some of them large, some without faces: warps
+    that hold queries of several of each."""
+    rng = np.random.default_rng(3)
+    meshes, qs = [], []
+    for k in range(60):
+        V, F = displaced_icosphere(2 if k == 7 else 1, 0.1, 0.1 * k)
+        V = (V * rng.uniform(0.1, 50.0)).astype(np.float32)
+        F = F if k == 7 else F[:[1, 0, 5, 24, 25][k % 5]]
+        meshes.append((V, np.ascontiguousarray(F)))
+        qs.append(uniform_box(int(rng.integers(0, 40)), V.min(0) * 1.2, V.max(0) * 1.2, seed=k))
+    batch = MeshBatch.from_meshes(meshes)
+    assert sum(len(f) for _, f in meshes) <= 17 * len(meshes) and max(len(f) for _, f in meshes) == 320
+    off = dev(np.concatenate([[0], np.cumsum([len(q) for q in qs])]).astype(np.int32))
+    for md in (float("inf"), 0.5):
+        got = batch.closest_point(dev(np.concatenate(qs)), off, md)
+        ref = [one_thread(MeshBVH.from_mesh(dev(v), dev(f)), dev(q), md) for (v, f), q in zip(meshes, qs) if len(q)]
+        assert_identical(got, {k: torch.cat([r[k] for r in ref]) for k in ref[0]})
+    assert batch.status()[0] == 0
+
+
+def test_few_faces_cost_no_more_than_one_thread_per_query():
+    """300k queries of meshes of one and of four faces: at most 1.3 times the one-thread
+    search's time (a warp of the pool per 16 queries: up to 2.5 times for signed distances)."""
+    V, F = icosphere(1)
+    Q = dev(uniform_box(300_000, [-1.5] * 3, [1.5] * 3, seed=1))
+    for faces in (1, 4):
+        bvh = MeshBVH.from_mesh(dev(V), dev(np.ascontiguousarray(F[:faces])))
+        ref = one_thread(bvh, Q, float("inf"))
+        bvh.set_query_config(1, 2)
+        one_ms = _best_ms(lambda: bvh.closest_point(Q, out=ref))
+        bvh.set_query_config(-1, -1)
+        got = bvh.closest_point(Q)
+        assert _best_ms(lambda: bvh.closest_point(Q, out=got)) <= 1.3 * one_ms
+        sd = bvh.signed_distance(Q)
+        assert _best_ms(lambda: bvh.signed_distance(Q, out=sd)) <= 1.3 * one_ms
