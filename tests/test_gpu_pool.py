@@ -262,8 +262,10 @@ def test_batch_of_mostly_few_faces():
 
 
 def test_few_faces_cost_no_more_than_one_thread_per_query():
-    """300k queries of meshes of one and of four faces: at most 1.3 times the one-thread
-    search's time (a warp of the pool per 16 queries: up to 2.5 times for signed distances)."""
+    """300k queries of meshes of one and of four faces, and 300k Chamfer samples a side: at most
+    1.3 times the one-thread search's time for as many queries (a warp of the pool per 16
+    samples: twice)."""
+    from paper_2606_00444_gb300 import Workspace, chamfer
     V, F = icosphere(1)
     Q = dev(uniform_box(300_000, [-1.5] * 3, [1.5] * 3, seed=1))
     for faces in (1, 4):
@@ -274,5 +276,51 @@ def test_few_faces_cost_no_more_than_one_thread_per_query():
         bvh.set_query_config(-1, -1)
         got = bvh.closest_point(Q)
         assert _best_ms(lambda: bvh.closest_point(Q, out=got)) <= 1.3 * one_ms
-        sd = bvh.signed_distance(Q)
-        assert _best_ms(lambda: bvh.signed_distance(Q, out=sd)) <= 1.3 * one_ms
+        ws, cd = Workspace(Q.device), torch.empty(2, dtype=torch.float64, device="cuda")
+        assert _best_ms(lambda: chamfer(bvh, Q, bvh, Q, ws=ws, out=cd)) <= 1.3 * 2 * one_ms
+
+
+@pytest.mark.parametrize("faces", [1, 3, 16, 17, 24, 25])
+@pytest.mark.parametrize("n", [1, 33, 50_001])
+def test_knn_of_few_or_tied_faces(n, faces):
+    """Meshes of few faces (a lane per query tests them all) and many tied faces (copies, at
+    a query's own distance): the lists are the k least (distance, id)."""
+    V, F = icosphere(1)
+    rng = np.random.default_rng(n)
+    Qn = rng.normal(size=(n, 3)).astype(np.float32)
+    Qn[0] = 0.0
+    for Fs in (F[:faces], np.concatenate([F[:faces], F[:faces][::-1]])):
+        Fs = np.ascontiguousarray(Fs)
+        bvh = MeshBVH.from_mesh(dev(V), dev(Fs))
+        m = min(n, 100)
+        each = torch.stack([one_thread(MeshBVH.from_mesh(dev(V), dev(Fs[f:f + 1])), dev(Qn[:m]), float("inf"))["dist2"]
+                            for f in range(len(Fs))], 1).cpu().numpy()
+        order = np.lexsort((np.broadcast_to(np.arange(len(Fs)), each.shape), each), axis=1)
+        for k in (1, 4, 8):
+            p, face, d2 = bvh.knn_project(dev(Qn), k=k, want_faces=True)
+            c = min(k, len(Fs))
+            assert np.array_equal(face[:m, :c].cpu().numpy(), order[:, :c])
+            assert np.array_equal(d2[:m, :c].cpu().numpy(), np.take_along_axis(each, order[:, :c], 1))
+            assert (face[:, c:] == -1).all() and torch.isinf(d2[:, c:]).all() and torch.isfinite(p).all()
+        assert bvh.status()[0] == 0
+
+
+def test_knn_of_tied_faces_costs_no_more_than_the_nearest():
+    """50k queries at the centre of a cube whose sides are 8 nearest faces each: the nearest face
+    by k-NN takes at most 3 times the unbounded closest point's time (inserting every
+    tied face took 5 times); of 4 faces, the 4 nearest at most 3 times (9)."""
+    g = np.arange(41)
+    u, v = (x.ravel() for x in np.meshgrid(g, g, indexing="ij"))
+    i, j = (x.ravel() for x in np.meshgrid(g[:-1], g[:-1], indexing="ij"))
+    q = [(i + a) * 41 + j + b for a, b in ((0, 0), (1, 0), (1, 1), (0, 1))]
+    side = np.concatenate([np.stack([q[0], q[1], q[2]], 1), np.stack([q[0], q[2], q[3]], 1)])
+    V = np.concatenate([np.roll(np.stack([u / 20 - 1, v / 20 - 1, 0 * u + s], 1), k, axis=1)
+                        for k in range(3) for s in (-1.0, 1.0)]).astype(np.float32)
+    F = np.concatenate([side + 1681 * k for k in range(6)]).astype(np.int32)
+    Vs, Fs = icosphere(1)
+    for (Vm, Fm, k, n) in ((V, F, 1, 50_000), (Vs, np.ascontiguousarray(Fs[:4]), 4, 300_000)):
+        bvh = MeshBVH.from_mesh(dev(Vm), dev(Fm))
+        Q = torch.zeros(n, 3, device="cuda")
+        out, p = bvh.closest_point(Q), bvh.knn_project(Q, k=k)
+        cp_ms = _best_ms(lambda: bvh.closest_point(Q, out=out))
+        assert _best_ms(lambda: bvh.knn_project(Q, k=k, out=p)) <= 3 * cp_ms
