@@ -16,6 +16,7 @@
 
 #include "common.cuh"
 #include "gauss_math.cuh"
+#include "sort_shape.h"
 
 namespace meshgs {
 
@@ -29,8 +30,6 @@ mesh_status check_launch() {
 
 constexpr int kBlock = 256;
 constexpr int kRadix = 256;
-constexpr int kSortTileMin = 1024;    // keys per sort tile: 1024, 2048, 4096 or 8192 (sort_shape)
-constexpr int kSortTilesMax = 512;    // tiles whose counts a pass sums itself
 constexpr int kScanThreads = 256;     // one block per digit; also scans the 256 digit totals
 
 // ---------------------------------------------------------------------------
@@ -1100,24 +1099,6 @@ static BuildWs build_ws_layout(char *base, int64_t nF) {
     w.ticket = (unsigned int *)take(4);
     w.bytes = off;
     return w;
-}
-
-// Threads and keys per thread of a sort of n keys: f gets them as compile-time
-// constants.  Tiles grow with n: a pass reads every tile's 256 counts in every
-// block, 1 KB x tiles^2 in all, against 8 B x n of keys -- at most about 250 tiles
-// up to 2M keys.  Smaller tiles than these spread the ranking over more SMs.
-template <typename F> static void sort_shape(int n, F f) {
-    using std::integral_constant;
-    if (n <= 160 * 1024) f(integral_constant<int, 256>(), integral_constant<int, 4>());
-    else if (n <= 480 * 1024) f(integral_constant<int, 256>(), integral_constant<int, 8>());
-    else if (n <= 1024 * 1024) f(integral_constant<int, 512>(), integral_constant<int, 8>());
-    else f(integral_constant<int, 512>(), integral_constant<int, 16>());
-}
-
-static int sort_tiles(int n) {
-    int T = 0;
-    sort_shape(n, [&](auto th, auto it) { T = (n + th.value * it.value - 1) / (th.value * it.value); });
-    return T;
 }
 
 // The later passes' counts lie over the centroids (16 B per key; three more
