@@ -246,7 +246,9 @@ k_gs_render(mesh_camera cam, int gx, const int *__restrict__ order, const int2 *
     const unsigned int lt = (1u << lane) - 1u;
     const int2 rg = range[tile];
     float T = 1.0f, C0 = 0.0f, C1 = 0.0f, C2 = 0.0f;
-    auto gaussian = [&](int b) { return b + lane < rg.y ? gid[b + lane] : -1; };
+    // (unsigned: the steps ahead may pass INT_MAX)
+    const unsigned int end = (unsigned)rg.y;
+    auto gaussian = [&](unsigned int b) { return b + lane < end ? gid[b + lane] : -1; };
     auto box = [&](int g) {
         return g >= 0 ? reach[g] : make_float4(INFINITY, -INFINITY, INFINITY, -INFINITY);
     };
@@ -271,14 +273,15 @@ k_gs_render(mesh_camera cam, int gx, const int *__restrict__ order, const int2 *
             s_col[wid][buf][at] = nl;
         }
     };
-    int g1 = gaussian(rg.x + 32), g2 = gaussian(rg.x + 64);
+    const unsigned int begin = (unsigned)rg.x;
+    int g1 = gaussian(begin + 32), g2 = gaussian(begin + 64);
     {
-        const int g0 = gaussian(rg.x);
+        const int g0 = gaussian(begin);
         fetch(g0, box(g0));
     }
     float4 r1 = box(g1);
     int buf = 0;
-    for (int b0 = rg.x; b0 < rg.y; b0 += 32, buf ^= 1) {
+    for (unsigned int b0 = begin; b0 < end; b0 += 32, buf ^= 1) {
         if (__all_sync(0xffffffffu, done)) break;
         stage(buf);
         const int n = __popc(next);
