@@ -227,3 +227,11 @@ def test_equal_keys_sort_in_the_time_of_others():
     equal_ms, order = _order_ms(P)
     assert torch.equal(order, torch.arange(len(P), dtype=torch.int32, device="cuda"))
     assert equal_ms <= 0.85 * random_ms, (equal_ms, random_ms)
+
+
+def test_sorts_of_twice_the_keys_take_at_most_twice_as_long():
+    """2M and 4M random points, on either side of where k_sort_scan sums the tiles' counts."""
+    g = torch.Generator(device="cuda")
+    g.manual_seed(4)
+    P = torch.rand(4_000_000, 3, generator=g, device="cuda")
+    assert _order_ms(P)[0] <= 2 * _order_ms(P[:2_000_000])[0]
