@@ -18,6 +18,7 @@
 #include <math.h>
 
 #include <cstring>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -141,15 +142,29 @@ __global__ void k_emd_resolve(int n, float *price, int *owner, int *assign, unsi
 // their distances, still holds the best two as long as the best listed value
 // is above T and the second is not below it (everything outside is at most T).
 // Such a bid reads kListMax entries instead of n objects.  The threshold is the
-// second-best value at that time less a margin, adapted per point so that
-// about 160 objects qualify.  A list that no longer decides is made again by
-// a scan of all objects; one that cannot (more than kListMax objects within the
-// margin, e.g. coincident points) gives way to an exact scan for that bid.
+// second-best value at that time less a margin, scaled per point by the count it
+// gave so that about 160 objects qualify.  A list that no longer decides is made
+// again by a scan of all objects, which also gives the bid.
+//
+// A list pays when it outlives a few bids -- fewer the more objects a scan reads --
+// and every bid raises a price by at least eps: where the margin that holds 160 objects
+// is below list_margin (the coarse phases; many points in one place, of which no
+// margin is small enough), a point makes none and bids by one exact scan.  Lists everywhere, with the margin changed by a quarter
+// at a time, cost up to 6 times the scans alone (10k points in one place 17.9 s against
+// 3.1, 2.6 so; 10k points of a plane and of a cube, eps 1e-2, 106 ms against 60, 53 so).
 // Either way the bid is the one a full scan gives, bit for bit: the same
 // distances, the same subtraction, ties to the lowest object id.
 // ---------------------------------------------------------------------------
 constexpr int kListMax = 256;                        // entries; eight per lane
 constexpr int kListLow = 120, kListHigh = 208;       // entries aimed for
+constexpr float kListAim = 160.0f;
+
+// Least margin of a list at a phase's eps.  Multiples of 2, 3, 4 and 6 eps were timed at 1000
+// to 10000 points on surfaces, volumes and clusters: 10000 points in a cube, eps 1e-2, take
+// 75, 120, 123 and 123 ms (scans 115); 5000 of a 3-D normal and its image 1.25 apart 58,
+// 56, 55, 56 (scans 50); 5000 in a cube 40, 40, 59, 64 (56); 3000 in a cube 19, 19, 19, 28
+// (24).  Below 3333 points 4, at 10000 2.
+inline float list_margin(int n, double eps) { return (float)(eps * fmin(4.0, 1.0 + 1e4 / (double)n)); }
 
 struct EmdLists {
     int4 *entry;       // [n][kListMax / 2], two (object, distance bits) pairs each
@@ -209,10 +224,14 @@ __device__ __forceinline__ bool list_qualifies(float d2, float price, float T) {
     return r > 0.0f && d2 <= r * r * 1.000002f;
 }
 
-__device__ __forceinline__ void list_append(const EmdLists &L, int i, int *cnt, int j, float d2) {
+// Lists an object and takes it into the (best, second best) values met.  The two best of
+// all objects qualify, so a list's scan gives the bid.
+__device__ __forceinline__ void list_append(const EmdLists &L, int i, int *cnt, int j, float d2, float price, float &b1,
+                                            int &j1, float &b2) {
     const int pos = atomicAdd(cnt, 1);
-    if (pos < kListMax)
-        reinterpret_cast<int2 *>(L.entry)[(size_t)i * kListMax + pos] = make_int2(j, __float_as_int(sqrtf(d2)));
+    const float d = sqrtf(d2);
+    if (pos < kListMax) reinterpret_cast<int2 *>(L.entry)[(size_t)i * kListMax + pos] = make_int2(j, __float_as_int(d));
+    merge2(b1, j1, b2, -d - price, j, -INFINITY);
 }
 
 // Closes a list of cnt entries: the rest padded with entries of value -inf
@@ -222,10 +241,12 @@ __device__ __forceinline__ void list_close(const EmdLists &L, int i, int cnt, in
     for (int k = cnt + t; k < kListMax; k += nt)
         reinterpret_cast<int2 *>(L.entry)[(size_t)i * kListMax + k] = make_int2(0, 0x7f800000);
     if (t != 0) return;
-    if (cnt > kListMax) { T = INFINITY; margin *= 0.5f; }            // too many: no list
+    if (cnt < n && (cnt < kListLow || cnt > kListHigh))              // about r^2 objects within r
+        margin *= fminf(4.0f, fmaxf(0.25f, sqrtf(kListAim / fmaxf((float)cnt, 1.0f))));
+    else if (cnt > kListMax)                                         // (and every object)
+        margin *= 0.25f;
+    if (cnt > kListMax) T = INFINITY;                                // too many: no list
     else if (cnt == n) T = -INFINITY;                                // every object is listed
-    else if (cnt > kListHigh) margin *= 0.8f;
-    else if (cnt < kListLow) margin *= 1.25f;
     L.hdr[i] = make_float2(T, margin);
 }
 
@@ -244,17 +265,17 @@ __global__ void k_emd_lists_init(int n, EmdLists L, float margin) {
 
 // One round of bids with lists (n <= kTailMaxN): one warp per unassigned point
 // reads its list; the block then scans the objects for the points whose lists
-// did not decide, two at a time, and those bid from their new lists.  B4 holds
-// the prices in w.
+// did not decide: two at a time those that get a new list, up to four at a time
+// those that make none.  B4 holds the prices in w.
 __global__ void __launch_bounds__(kEmdBlock)
 k_emd_bid_lists(int n, const float4 *__restrict__ A4, const float4 *__restrict__ B4, const int *__restrict__ assign,
-                unsigned long long *bids, EmdLists L, float eps, unsigned *active) {
-    __shared__ int s_point[kEmdWarps], s_miss;
-    __shared__ float s_b1[2][kEmdWarps], s_b2[2][kEmdWarps];
-    __shared__ int s_cnt[2];
+                unsigned long long *bids, EmdLists L, float eps, float least, unsigned *active) {
+    __shared__ int s_list[kEmdWarps], s_lists, s_scan[kEmdWarps], s_scans;
+    __shared__ float s_b1[4][kEmdWarps], s_b2[4][kEmdWarps];
+    __shared__ int s_j[4][kEmdWarps], s_cnt[2];
     pdl_wait();
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (threadIdx.x == 0) s_miss = 0;
+    if (threadIdx.x == 0) { s_lists = 0; s_scans = 0; }
     __syncthreads();
     auto price = [&](int j) { return __ldcg(&B4[j].w); };
     auto place = [&](int i, float b1, int j1, float b2) {
@@ -280,16 +301,65 @@ k_emd_bid_lists(int n, const float4 *__restrict__ A4, const float4 *__restrict__
     };
     {
         const int i = blockIdx.x * kEmdWarps + wid;
-        if (i < n && assign[i] < 0 && !bid_from_list(i) && lane == 0) s_point[atomicAdd(&s_miss, 1)] = i;
+        if (i < n && assign[i] < 0 && !bid_from_list(i) && lane == 0) {
+            if (L.hdr[i].y >= least) s_list[atomicAdd(&s_lists, 1)] = i;
+            else s_scan[atomicAdd(&s_scans, 1)] = i;
+        }
     }
     __syncthreads();
-    const int misses = s_miss;
-    for (int m0 = 0; m0 < misses; m0 += 2) {
-        const int two = min(2, misses - m0);
-        const int pt[2] = {s_point[m0], s_point[m0 + two - 1]};
+    const int lists = s_lists, scans = s_scans;
+    // the block's best two values of K points, from its threads'
+    auto block_best2 = [&](auto K, float *b1, int *j1, float *b2) {
+#pragma unroll
+        for (int k = 0; k < K.value; ++k) {
+            warp_best2(b1[k], j1[k], b2[k]);
+            if (lane == 0) { s_b1[k][wid] = b1[k]; s_b2[k][wid] = b2[k]; s_j[k][wid] = j1[k]; }
+        }
+        __syncthreads();
+    };
+    auto of_block = [&](int k, float &b1, int &j1, float &b2) {
+        b1 = lane < kEmdWarps ? s_b1[k][lane] : -INFINITY;
+        b2 = lane < kEmdWarps ? s_b2[k][lane] : -INFINITY;
+        j1 = lane < kEmdWarps ? s_j[k][lane] : 0x7fffffff;
+        warp_best2(b1, j1, b2);
+    };
+    // exact scans for K points of s_scan
+    auto scan = [&](auto K, int m0) {
+        float4 a[K.value];
+        float b1[K.value], b2[K.value];
+        int j1[K.value];
+#pragma unroll
+        for (int k = 0; k < K.value; ++k) {
+            a[k] = A4[s_scan[min(m0 + k, scans - 1)]];
+            b1[k] = b2[k] = -INFINITY;
+            j1[k] = 0x7fffffff;
+        }
+        for (int j = threadIdx.x; j < n; j += kEmdBlock) {
+            const float4 b = __ldcg(&B4[j]);
+#pragma unroll
+            for (int k = 0; k < K.value; ++k)
+                merge2(b1[k], j1[k], b2[k], -sqrtf(emd_d2(a[k], b.x, b.y, b.z)) - b.w, j, -INFINITY);
+        }
+        block_best2(K, b1, j1, b2);
+        if (wid < K.value && m0 + wid < scans) {
+            of_block(wid, b1[0], j1[0], b2[0]);
+            place(s_scan[m0 + wid], b1[0], j1[0], b2[0]);
+        }
+        __syncthreads();
+    };
+    for (int m0 = 0; m0 < scans; m0 += 4) {
+        if (scans - m0 > 2) scan(std::integral_constant<int, 4>(), m0);
+        else if (scans - m0 == 2) scan(std::integral_constant<int, 2>(), m0);
+        else scan(std::integral_constant<int, 1>(), m0);
+    }
+    for (int m0 = 0; m0 < lists; m0 += 2) {
+        const std::integral_constant<int, 2> two;
+        const int cnt = min(2, lists - m0);
+        const int pt[2] = {s_list[m0], s_list[m0 + cnt - 1]};
         const float4 a[2] = {A4[pt[0]], A4[pt[1]]};
         const float margin[2] = {L.hdr[pt[0]].y, L.hdr[pt[1]].y};
         float b1[2] = {-INFINITY, -INFINITY}, b2[2] = {-INFINITY, -INFINITY};
+        int j1[2] = {lane, lane};                     // (which object does not matter here)
         for (int j = threadIdx.x; j < n; j += kEmdBlock) {
             const float4 b = __ldcg(&B4[j]);
 #pragma unroll
@@ -299,14 +369,8 @@ k_emd_bid_lists(int n, const float4 *__restrict__ A4, const float4 *__restrict__
                 b1[k] = fmaxf(b1[k], v);
             }
         }
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            int dummy = lane;
-            warp_best2(b1[k], dummy, b2[k]);
-            if (lane == 0) { s_b1[k][wid] = b1[k]; s_b2[k][wid] = b2[k]; }
-        }
         if (threadIdx.x < 2) s_cnt[threadIdx.x] = 0;
-        __syncthreads();
+        block_best2(two, b1, j1, b2);
         float T[2];
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
@@ -314,33 +378,38 @@ k_emd_bid_lists(int n, const float4 *__restrict__ A4, const float4 *__restrict__
             int dummy = lane;
             warp_best2(c1, dummy, c2);
             T[k] = c2 - margin[k];
+            b1[k] = b2[k] = -INFINITY;
+            j1[k] = 0x7fffffff;
         }
         for (int j = threadIdx.x; j < n; j += kEmdBlock) {
             const float4 b = __ldcg(&B4[j]);
 #pragma unroll
             for (int k = 0; k < 2; ++k) {
-                if (k >= two) break;
+                if (k >= cnt) break;
                 const float d2 = emd_d2(a[k], b.x, b.y, b.z);
-                if (list_qualifies(d2, b.w, T[k])) list_append(L, pt[k], &s_cnt[k], j, d2);
+                if (list_qualifies(d2, b.w, T[k])) list_append(L, pt[k], &s_cnt[k], j, d2, b.w, b1[k], j1[k], b2[k]);
             }
         }
-        __syncthreads();
+        __syncthreads();                              // the counts, and the thresholds' values are read
 #pragma unroll
         for (int k = 0; k < 2; ++k)
-            if (k < two) list_close(L, pt[k], s_cnt[k], n, T[k], margin[k], threadIdx.x, kEmdBlock);
-        __syncthreads();
-        if (wid < two) {
+            if (k < cnt) list_close(L, pt[k], s_cnt[k], n, T[k], margin[k], threadIdx.x, kEmdBlock);
+        block_best2(two, b1, j1, b2);
+        if (wid < cnt) {
             const int i = pt[wid];
-            if (!bid_from_list(i)) {                  // exact scan by the warp
-                float c1 = -INFINITY, c2 = -INFINITY;
-                int j1 = 0x7fffffff;
+            float c1, c2;
+            int jb;
+            of_block(wid, c1, jb, c2);
+            if (!(c1 > T[wid] && c2 >= T[wid])) {     // (rounding of the threshold) exact scan by the warp
+                c1 = c2 = -INFINITY;
+                jb = 0x7fffffff;
                 for (int j = lane; j < n; j += 32) {
                     const float4 b = __ldcg(&B4[j]);
-                    merge2(c1, j1, c2, -sqrtf(emd_d2(a[wid], b.x, b.y, b.z)) - b.w, j, -INFINITY);
+                    merge2(c1, jb, c2, -sqrtf(emd_d2(a[wid], b.x, b.y, b.z)) - b.w, j, -INFINITY);
                 }
-                warp_best2(c1, j1, c2);
-                place(i, c1, j1, c2);
+                warp_best2(c1, jb, c2);
             }
+            place(i, c1, jb, c2);
         }
         __syncthreads();
     }
@@ -377,9 +446,10 @@ __global__ void k_emd_resolve_lists(int n, float4 *__restrict__ B4, int *owner, 
 // memory, as are the owners), as long as they decide it: prices only rise, so
 // what was left out stays below.  The head of the queue, with no bid since its
 // list was read, bids from the whole list.  A point whose list no longer decides
-// gets a new one from a scan by all other warps, which hold the objects'
-// coordinates in registers, two points at a time.
-// 10k points, eps 1e-4: 259 ms with one list at a time, 191 ms so (531 with scans).
+// bids from a scan by all other warps, which hold the objects' coordinates in
+// registers: one that makes a new list, for it and for the next point that needs
+// one, or an exact scan for a point that makes none.
+// 10k points, eps 1e-4: 259 ms with one list at a time, 178 ms so (531 with scans).
 constexpr int kTailThreads = 768;                    // 80 registers each: 48 of coordinates
 constexpr int kTailQueue = 256;
 constexpr int kTailAhead = 16;
@@ -400,7 +470,8 @@ __device__ __forceinline__ void bar_sync(int id, int threads) {
 struct TailAhead {
     float d[kTailAhead][32];
     int j[kTailAhead][32];
-    float rest[kTailAhead];            // -inf: the list does not decide
+    float rest[kTailAhead];            // -inf: the list does not decide; NaN: to be read again
+    bool wants[kTailAhead];            // a new list pays (list_margin)
     float b1, b2;                      // the head's bid from its whole list
     int j1;
 };
@@ -417,7 +488,7 @@ __device__ __forceinline__ void least2(float c, int j, float &c1, int &j1, float
 
 __global__ void __launch_bounds__(kTailThreads, 1)
 k_emd_tail(int n, const float4 *__restrict__ A4, float4 *B4, float *price, int *owner, int *assign, EmdLists L,
-           float eps, int max_bids, unsigned *active) {
+           float eps, float least, int max_bids, unsigned *active) {
     extern __shared__ float sp[];                    // prices, then owners
     int *s_own = reinterpret_cast<int *>(sp + n);
     __shared__ TailAhead s_ahead;
@@ -425,6 +496,7 @@ k_emd_tail(int n, const float4 *__restrict__ A4, float4 *B4, float *price, int *
     __shared__ float r1[2][32], r2[2][32];
     __shared__ int rj[32], s_wcnt[32];
     __shared__ int s_len, s_mode, s_head, s_point[2], s_cnt[2];
+    __shared__ float s_T;
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const bool lists = L.entry != nullptr;
     for (int j = tid; j < n; j += kTailThreads) { sp[j] = price ? price[j] : B4[j].w; s_own[j] = owner[j]; }
@@ -474,54 +546,84 @@ k_emd_tail(int n, const float4 *__restrict__ A4, float4 *B4, float *price, int *
             bar_sync(1, kTailThreads);
             if (mode != kTailDone) bar_sync(1, kTailThreads);
         };
-        bool fresh = false;                          // the head's list was just made
+        // a scan's best two, from the other warps'
+        auto scanned = [&](float &b1, int &j1, float &b2) {
+            const bool in = lane > 0 && lane < kTailThreads / 32;
+            b1 = in ? r1[0][lane] : -INFINITY;
+            b2 = in ? r2[0][lane] : -INFINITY;
+            j1 = in ? rj[lane] : 0x7fffffff;
+            warp_best2(b1, j1, b2);
+        };
+        int ahead = 0, done = 0;                     // bids read ahead, and used
         while (bids < max_bids && len > 0) {
+            bool list = false;
             if (lists) {
-                step(kTailRead);
-                const int ahead = min(len, kTailAhead);
-                int done = 0;
-                if (s_ahead.rest[0] >= 0.0f) {       // the head, from its whole list
-                    const float b1 = s_ahead.b1, b2 = s_ahead.b2;
-                    commit(queue[head % kTailQueue], b2 == -INFINITY ? 0.0f : b1 - b2, s_ahead.j1);
-                    done = 1;
+                if (done == ahead) {
+                    step(kTailRead);
+                    ahead = min(len, kTailAhead);
+                    done = 0;
+                    if (s_ahead.rest[0] >= 0.0f) {   // the head, from its whole list
+                        const float b1 = s_ahead.b1, b2 = s_ahead.b2;
+                        commit(queue[head % kTailQueue], b2 == -INFINITY ? 0.0f : b1 - b2, s_ahead.j1);
+                        done = 1;
+                        continue;
+                    }
                 }
-                float d = s_ahead.d[1][lane];        // the next entries, one bid ahead of their use
-                int j = s_ahead.j[1][lane];
-                while (done > 0 && done < ahead && bids < max_bids) {
-                    const float rest = s_ahead.rest[done];
-                    if (!(rest >= 0.0f)) break;      // (its entries need not be written)
+                const int before = done;
+                bool again = false;                  // an entry whose 32 costs do not decide
+                float rest = s_ahead.rest[done];
+                float d = s_ahead.d[done][lane];     // the next entries, one bid ahead of their use
+                int j = s_ahead.j[done][lane];
+                while (rest >= 0.0f && bids < max_bids) {
                     const float nd = d + sp[j];
                     const int i = queue[head % kTailQueue], nj = j;
-                    if (done + 1 < ahead) { d = s_ahead.d[done + 1][lane]; j = s_ahead.j[done + 1][lane]; }
+                    const float limit = rest;
+                    if (done + 1 < ahead) {
+                        d = s_ahead.d[done + 1][lane];
+                        j = s_ahead.j[done + 1][lane];
+                        rest = s_ahead.rest[done + 1];
+                    }
                     float c1, c2;
                     int j1;
                     least2(nd, nj, c1, j1, c2);
-                    if (!(c1 < rest && c2 <= rest)) break;
+                    again = !(c1 < limit && c2 <= limit);
+                    if (again) break;
                     commit(i, c2 == INFINITY ? 0.0f : c2 - c1, j1);
-                    ++done;
+                    if (++done == ahead) break;
                 }
-                if (done > 0) { fresh = false; continue; }
-            }
-            if (lists && !fresh) {                   // new lists for the head and the next that needs one
-                const int ahead = min(len, kTailAhead);
-                const unsigned need = __ballot_sync(0xffffffffu, lane > 0 && lane < ahead && s_ahead.rest[lane < kTailAhead ? lane : 0] < 0.0f);
+                if (again || (done == before && done > 0 && !(rest < 0.0f))) {
+                    ahead = done;                    // read its whole list, as the head's
+                    continue;
+                }
+                if (done > before) continue;
+                list = s_ahead.wants[done];
+                const int q = lane < kTailAhead ? lane : 0;
+                const unsigned need = __ballot_sync(0xffffffffu, list && lane > done && lane < ahead &&
+                                                                     s_ahead.rest[q] < 0.0f && s_ahead.wants[q]);
                 if (lane == 0) {
-                    s_point[0] = queue[head % kTailQueue];
-                    s_point[1] = need ? queue[(head + __ffs(need) - 1) % kTailQueue] : -1;
+                    s_point[1] = -1;
+                    if (need) {                      // the next that needs one: its list is read again
+                        const int next = __ffs(need) - 1;
+                        s_point[1] = queue[(head + next - done) % kTailQueue];
+                        s_ahead.rest[next] = NAN;
+                    }
                 }
-                step(kTailList);
-                fresh = true;
-                continue;
             }
             if (lane == 0) s_point[0] = queue[head % kTailQueue];
-            step(kTailExact);
-            float b1 = lane > 0 && lane < kTailThreads / 32 ? r1[0][lane] : -INFINITY;
-            float b2 = lane > 0 && lane < kTailThreads / 32 ? r2[0][lane] : -INFINITY;
-            int j1 = lane > 0 && lane < kTailThreads / 32 ? rj[lane] : 0x7fffffff;
-            warp_best2(b1, j1, b2);
+            float b1, b2;
+            int j1;
+            if (list) {
+                step(kTailList);
+                scanned(b1, j1, b2);
+                list = b1 > s_T && b2 >= s_T;
+            }
+            if (!list) {
+                step(kTailExact);
+                scanned(b1, j1, b2);
+            }
             if ((unsigned)j1 >= (unsigned)n) break;  // no comparable value (NaN input): leave the point queued
             commit(s_point[0], b2 == -INFINITY ? 0.0f : b1 - b2, j1);
-            fresh = false;
+            if (lists) ++done;
         }
         step(kTailDone);
         if (lane == 0) *active = (unsigned)len;
@@ -534,6 +636,20 @@ k_emd_tail(int n, const float4 *__restrict__ A4, float4 *B4, float *price, int *
             const float4 b = j < n ? B4[j] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
             bx[k] = b.x; by[k] = b.y; bz[k] = b.z;
         }
+        // calls f for each object this thread holds; few slots for few objects (1000 points' call
+        // from scans 15.7 ms with all 16, 11.2 so)
+        auto objects = [&](auto f) {
+            auto run = [&](auto slots) {
+#pragma unroll
+                for (int k = 0; k < slots.value; ++k) {
+                    const int j = t + k * kScanThreads;
+                    if (j < n) f(j, bx[k], by[k], bz[k]);
+                }
+            };
+            if (n <= 2 * kScanThreads) run(std::integral_constant<int, 2>());
+            else if (n <= 7 * kScanThreads) run(std::integral_constant<int, 7>());
+            else run(std::integral_constant<int, kScanPer>());
+        };
         while (true) {
             bar_sync(1, kTailThreads);
             const int mode = s_mode;
@@ -542,7 +658,9 @@ k_emd_tail(int n, const float4 *__restrict__ A4, float4 *B4, float *price, int *
                 const int q = wid - 1;
                 if (q < min(s_len, kTailAhead)) {
                     const int i = queue[(s_head + q) % kTailQueue];
-                    const float T = L.hdr[i].x;
+                    const float2 hdr = L.hdr[i];
+                    const float T = hdr.x;
+                    if (lane == 0) s_ahead.wants[q] = hdr.y >= least;
                     int4 e[4];
                     list_load(L, i, lane, e);
                     if (T == INFINITY) {             // no list (its entries are not read)
@@ -585,11 +703,9 @@ k_emd_tail(int n, const float4 *__restrict__ A4, float4 *B4, float *price, int *
                 const float4 a = A4[s_point[0]];
                 float b1 = -INFINITY, b2 = -INFINITY;
                 int j1 = 0x7fffffff;
-#pragma unroll
-                for (int k = 0; k < kScanPer; ++k) {
-                    const int j = t + k * kScanThreads;
-                    if (j < n) merge2(b1, j1, b2, -sqrtf(emd_d2(a, bx[k], by[k], bz[k])) - sp[j], j, -INFINITY);
-                }
+                objects([&](int j, float x, float y, float z) {
+                    merge2(b1, j1, b2, -sqrtf(emd_d2(a, x, y, z)) - sp[j], j, -INFINITY);
+                });
                 warp_best2(b1, j1, b2);
                 if (lane == 0) { r1[0][wid] = b1; r2[0][wid] = b2; rj[wid] = j1; }
                 bar_sync(1, kTailThreads);
@@ -601,19 +717,15 @@ k_emd_tail(int n, const float4 *__restrict__ A4, float4 *B4, float *price, int *
             const float margin0 = L.hdr[i0].y, margin1 = L.hdr[i1 >= 0 ? i1 : i0].y;
             if (t < 2) s_cnt[t] = 0;
             float b1 = -INFINITY, b2 = -INFINITY, e1 = -INFINITY, e2 = -INFINITY;
-#pragma unroll
-            for (int k = 0; k < kScanPer; ++k) {
-                const int j = t + k * kScanThreads;
-                if (j < n) {
-                    const float p = sp[j];
-                    float v = value_approx(emd_d2(a0, bx[k], by[k], bz[k]), p);
-                    b2 = fmaxf(b2, fminf(b1, v));
-                    b1 = fmaxf(b1, v);
-                    v = value_approx(emd_d2(a1, bx[k], by[k], bz[k]), p);
-                    e2 = fmaxf(e2, fminf(e1, v));
-                    e1 = fmaxf(e1, v);
-                }
-            }
+            objects([&](int j, float x, float y, float z) {
+                const float p = sp[j];
+                float v = value_approx(emd_d2(a0, x, y, z), p);
+                b2 = fmaxf(b2, fminf(b1, v));
+                b1 = fmaxf(b1, v);
+                v = value_approx(emd_d2(a1, x, y, z), p);
+                e2 = fmaxf(e2, fminf(e1, v));
+                e1 = fmaxf(e1, v);
+            });
             int dummy = lane;
             warp_best2(b1, dummy, b2);
             dummy = lane;
@@ -630,22 +742,22 @@ k_emd_tail(int n, const float4 *__restrict__ A4, float4 *B4, float *price, int *
             dummy = lane;
             warp_best2(e1, dummy, e2);
             const float T0 = b2 - margin0, T1 = e2 - margin1;
-#pragma unroll
-            for (int k = 0; k < kScanPer; ++k) {
-                const int j = t + k * kScanThreads;
-                if (j < n) {
-                    const float p = sp[j];
-                    const float d0 = emd_d2(a0, bx[k], by[k], bz[k]);
-                    if (list_qualifies(d0, p, T0)) list_append(L, i0, &s_cnt[0], j, d0);
-                    if (i1 >= 0) {
-                        const float d1 = emd_d2(a1, bx[k], by[k], bz[k]);
-                        if (list_qualifies(d1, p, T1)) list_append(L, i1, &s_cnt[1], j, d1);
-                    }
+            b1 = b2 = e1 = e2 = -INFINITY;               // now of the objects listed
+            int j1 = 0x7fffffff, e1j = 0x7fffffff;
+            objects([&](int j, float x, float y, float z) {
+                const float p = sp[j], d0 = emd_d2(a0, x, y, z);
+                if (list_qualifies(d0, p, T0)) list_append(L, i0, &s_cnt[0], j, d0, p, b1, j1, b2);
+                if (i1 >= 0) {
+                    const float d1 = emd_d2(a1, x, y, z);
+                    if (list_qualifies(d1, p, T1)) list_append(L, i1, &s_cnt[1], j, d1, p, e1, e1j, e2);
                 }
-            }
+            });
             bar_sync(2, kScanThreads);
             list_close(L, i0, s_cnt[0], n, T0, margin0, t, kScanThreads);
             if (i1 >= 0) list_close(L, i1, s_cnt[1], n, T1, margin1, t, kScanThreads);
+            warp_best2(b1, j1, b2);
+            if (lane == 0) { r1[0][wid] = b1; r2[0][wid] = b2; rj[wid] = j1; }
+            if (t == 0) s_T = T0;
             bar_sync(1, kTailThreads);
         }
     }
@@ -785,8 +897,10 @@ mesh_status mesh_emd(const float *d_A, const float *d_B, int64_t n, float eps_re
     static std::atomic<unsigned long long> tail_smem{0};
     if (!allow_smem(k_emd_tail, 8 * (size_t)kTailMaxN, tail_smem)) return MESH_ERR_CUDA;
     if (lists) {
-        // a first guess of the margin: about 1 % of the box diagonal's objects at 10k points
-        k_emd_lists_init<<<grid_for(N, 256), 256, 0, s>>>(N, w.L, (float)(0.25 * C * sqrt(160.0 / (double)N)));
+        // a first guess of the margin: about 1 % of the box diagonal's objects at 10k points;
+        // every object where a list holds them all (such a list decides every bid)
+        const float margin = N <= kListMax ? 1e30f : (float)(0.25 * C * sqrt((double)kListAim / (double)N));
+        k_emd_lists_init<<<grid_for(N, 256), 256, 0, s>>>(N, w.L, margin);
         count_launch();
     }
     int64_t iters = 0;
@@ -802,7 +916,8 @@ mesh_status mesh_emd(const float *d_A, const float *d_B, int64_t n, float eps_re
                 if (lists) {
                     const bool after_kernel = k != 0 && k != kEmdCheck - 1;
                     launch_ex(after_kernel, k_emd_bid_lists, bid_grid, kEmdBlock, 0, s, N, (const float4 *)w.A4,
-                              (const float4 *)w.B4, (const int *)w.assign, w.bids, w.L, (float)eps, w.active);
+                              (const float4 *)w.B4, (const int *)w.assign, w.bids, w.L, (float)eps,
+                              list_margin(N, eps), w.active);
                     pdl_launch(k_emd_resolve_lists, grid_for(N, 256), 256, 0, s, N, w.B4, w.owner, w.assign, w.bids);
                 } else {
                     k_emd_bid<<<bid_grid, kEmdBlock, 0, s>>>(N, w.A4, w.B4, w.price, w.assign, w.bids, (float)eps,
@@ -821,7 +936,7 @@ mesh_status mesh_emd(const float *d_A, const float *d_B, int64_t n, float eps_re
                 int64_t left = max_iters > iters ? max_iters - iters : 1;
                 int cap = (int)(left < (int64_t)(1 << 24) ? left : (int64_t)(1 << 24));
                 k_emd_tail<<<1, kTailThreads, 8 * (size_t)N, s>>>(N, w.A4, w.B4, lists ? nullptr : w.price, w.owner,
-                                                                  w.assign, w.L, (float)eps, cap, w.active);
+                                                                  w.assign, w.L, (float)eps, list_margin(N, eps), cap, w.active);
                 count_launch();
                 if (cudaMemcpyAsync(&act, w.active, sizeof(unsigned), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
                     cudaStreamSynchronize(s) != cudaSuccess)

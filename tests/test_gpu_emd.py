@@ -95,3 +95,63 @@ def test_emd_candidate_lists_leave_every_bid_unchanged(n, kind_a, kind_b):
         assert st == 0
         got.append((host(out), host(sigma), it.value))
     assert got[0][2] == got[1][2] and np.array_equal(got[0][1], got[1][1]) and np.array_equal(got[0][0], got[1][0])
+
+
+def _call(A, B, eps, nbytes, max_iters=100_000):
+    import ctypes as C
+    from paper_2606_00444_gb300._abi import lib
+    n = A.shape[0]
+    ws = torch.empty(lib().mesh_emd_workspace_bytes(n), dtype=torch.uint8, device="cuda")
+    out = torch.empty(1, dtype=torch.float64, device="cuda")
+    sigma = torch.empty(n, dtype=torch.int32, device="cuda")
+    it = C.c_int64(0)
+
+    def go():
+        return lib().mesh_emd(A.data_ptr(), B.data_ptr(), n, eps, max_iters, ws.data_ptr(),
+                              ws.numel() if nbytes is None else nbytes, out.data_ptr(), sigma.data_ptr(), C.byref(it),
+                              torch.cuda.current_stream().cuda_stream)
+
+    st = go()
+    torch.cuda.synchronize()
+    return st, host(out), host(sigma), it.value, go
+
+
+@pytest.mark.parametrize("kind_a,kind_b,eps", [("normal", "clusters", 1e-2), ("one", "one", 1e-2), ("plane", "normal", 1e-2),
+                                               ("normal", "affine", 1e-2), ("normal", "normal", 1e-2)])
+def test_emd_lists_cost_no_more_than_scans(kind_a, kind_b, eps):
+    """Where no list pays -- many points in one place, a coarse eps -- a call with room for lists
+    takes at most 1.25 times the call without (lists for every point: 1.3 to 6 times), and the
+    result is the same bit for bit."""
+    import time
+    from paper_2606_00444_gb300._abi import lib
+    n = 3000
+    rng = np.random.default_rng(n)
+    A = _points_of("normal" if kind_a == "plane" else kind_a, n, rng)
+    if kind_a == "plane":
+        A[:, 2] = 0
+    A = dev(A)
+    B = A * 0.8 + 0.3 if kind_b == "affine" else dev(_points_of(kind_b, n, rng))
+    best, got = [], []
+    for nbytes in (None, lib().mesh_emd_workspace_bytes(n) - 1):
+        st, out, sigma, it, go = _call(A, B, eps, nbytes)
+        assert st == 0
+        got.append((out, sigma, it))
+        ts = []
+        for _ in range(4):
+            t0 = time.perf_counter()
+            go()
+            torch.cuda.synchronize()
+            ts.append(time.perf_counter() - t0)
+        best.append(min(ts))
+    assert all(np.array_equal(x, y) for x, y in zip(*got))
+    assert best[0] <= 1.25 * best[1], best
+
+
+def test_emd_without_comparable_values_ends():
+    """A point with a NaN coordinate never bids: the call ends at max_iters with an error."""
+    rng = np.random.default_rng(5)
+    A, B = rng.normal(size=(2, 700, 3)).astype(np.float32)
+    A[3, 1] = np.nan
+    for nbytes in (None, 1 << 20):
+        st = _call(dev(A), dev(B), 1e-2, nbytes, max_iters=60)[0]
+        assert st != 0
