@@ -324,3 +324,67 @@ def test_knn_of_tied_faces_costs_no_more_than_the_nearest():
         out, p = bvh.closest_point(Q), bvh.knn_project(Q, k=k)
         cp_ms = _best_ms(lambda: bvh.closest_point(Q, out=out))
         assert _best_ms(lambda: bvh.knn_project(Q, k=k, out=p)) <= 3 * cp_ms
+
+
+@pytest.mark.parametrize("n", [6_000, 25_000, 50_000, 100_000, 200_000])
+def test_batch_warps_of_every_width_span_scenes(n):
+    """Widths of 1, 2, 4, 8 and 16 queries per warp (by the query count) over 300 scenes of
+    different sizes and scales, some without faces or without queries."""
+    rng = np.random.default_rng(n)
+    meshes, qs = [], []
+    for k in range(300):
+        V, F = displaced_icosphere(int(rng.integers(1, 4)), 0.1, 0.1 * k)
+        V = (V * rng.uniform(0.1, 50.0) + rng.uniform(-5, 5, 3)).astype(np.float32)
+        F = F[:0] if k % 17 == 5 else F
+        meshes.append((V, np.ascontiguousarray(F)))
+        m = 0 if k % 11 == 3 else int(rng.integers(0, n // 136))
+        qs.append(uniform_box(m, V.min(0) - 0.1, V.max(0) + 0.1, seed=k))
+    batch = MeshBatch.from_meshes(meshes)
+    off = dev(np.concatenate([[0], np.cumsum([len(q) for q in qs])]).astype(np.int32))
+    Q = dev(np.concatenate(qs))
+    singles = [MeshBVH.from_mesh(dev(v), dev(f)) for v, f in meshes]
+    for md in (float("inf"), 0.5):
+        got = batch.closest_point(Q, off, md)
+        ref = [one_thread(b, dev(q), md) for b, q in zip(singles, qs) if len(q)]
+        assert_identical(got, {k: torch.cat([r[k] for r in ref]) for k in ref[0]})
+    assert batch.status()[0] == 0
+
+
+@pytest.mark.parametrize("n", [25_003, 50_003])
+@pytest.mark.parametrize("k,leaf", [(4, 1), (8, 4)])
+def test_knn_of_two_and_four_queries_per_warp(n, k, leaf):
+    V, F = icosphere(1)
+    bvh = MeshBVH.from_mesh(dev(V), dev(F))
+    bvh.set_leaf_size(leaf)
+    Qn = np.random.default_rng(n + k).normal(size=(n, 3)).astype(np.float32)
+    Qn[:12] = V[:12]                                      # on vertices: ties of five faces
+    pick = np.r_[0:100, n - 100:n]
+    p, face, d2 = bvh.knn_project(dev(Qn), k=k, want_faces=True)
+    Q = dev(Qn[pick])
+    each = torch.stack([one_thread(MeshBVH.from_mesh(dev(V), dev(np.ascontiguousarray(F[f:f + 1]))), Q, float("inf"))["dist2"]
+                        for f in range(len(F))], 1).cpu().numpy()
+    order = np.lexsort((np.broadcast_to(np.arange(len(F)), each.shape), each), axis=1)[:, :k]
+    assert np.array_equal(face.cpu().numpy()[pick], order)
+    assert np.array_equal(d2.cpu().numpy()[pick], np.take_along_axis(each, order, 1))
+    assert torch.isfinite(p).all() and bvh.status()[0] == 0
+
+
+def test_chamfer_of_32_samples_per_warp():
+    """mesh_chamfer_noalloc with more samples than its scratch holds blocks of 64 for: 32 queries
+    per warp, the per-sample results of mesh_chamfer."""
+    from paper_2606_00444_gb300 import chamfer
+    from paper_2606_00444_gb300._abi import check, lib
+    V, F = displaced_icosphere(3, 0.1, 0.4)
+    bvh = MeshBVH.from_mesh(dev(V), dev(F))
+    nA, nB = 600_011, 500_003
+    assert (nA + nB) * 2 > 16384 * 128 > nA + nB
+    SA, SB = (dev(uniform_box(n, [-1.2] * 3, [1.2] * 3, seed=n)) for n in (nA, nB))
+    ref, ps = chamfer(bvh, SA, bvh, SB, per_sample=True)
+    out = torch.empty(2, dtype=torch.float64, device="cuda")
+    got = {k: torch.empty_like(v) for k, v in ps.items()}
+    check(lib().mesh_chamfer_noalloc(bvh.handle, SA.data_ptr(), nA, bvh.handle, SB.data_ptr(), nB, out.data_ptr(),
+                                     *(got[k].data_ptr() for k in ("faceA", "baryA", "dist2A", "faceB", "baryB", "dist2B")),
+                                     torch.cuda.current_stream().cuda_stream), "mesh_chamfer_noalloc")
+    for k in ps:
+        assert torch.equal(got[k], ps[k]), k
+    assert torch.allclose(out, ref, rtol=1e-12)
