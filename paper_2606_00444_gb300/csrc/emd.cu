@@ -65,6 +65,14 @@ __global__ void k_emd_unassign(int n, int *owner, int *assign) {
     assign[i] = -1;
 }
 
+// Squared distance of a point and an object: the one expression every path values with,
+// its roundings written out -- a list's entry and a scan's value of the same object are
+// compiled in different kernels and must be the same float.
+__device__ __forceinline__ float emd_d2(float4 a, float bx, float by, float bz) {
+    const float dx = a.x - bx, dy = a.y - by, dz = a.z - bz;
+    return __fmaf_rn(dz, dz, __fmaf_rn(dx, dx, __fmul_rn(dy, dy)));
+}
+
 // (best, second best) of a lane merged with another lane's
 __device__ __forceinline__ void merge2(float &b1, int &j1, float &b2, float o1, int oj, float o2) {
     if (o1 > b1 || (o1 == b1 && oj < j1)) {
@@ -97,10 +105,8 @@ k_emd_bid(int n, const float4 *__restrict__ A4, const float4 *__restrict__ B4, c
         __syncthreads();
         if (mine) {
             for (int t = lane; t < m; t += 32) {
-                float4 b = sb[t];
-                float dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z;
-                float v = -sqrtf(dx * dx + dy * dy + dz * dz) - sp[t];
-                merge2(b1, j1, b2, v, t0 + t, -INFINITY);
+                const float4 b = sb[t];
+                merge2(b1, j1, b2, -sqrtf(emd_d2(a, b.x, b.y, b.z)) - sp[t], t0 + t, -INFINITY);
             }
         }
         __syncthreads();
@@ -170,12 +176,6 @@ struct EmdLists {
     int4 *entry;       // [n][kListMax / 2], two (object, distance bits) pairs each
     float2 *hdr;       // [n] (threshold, margin); threshold +inf: no list yet
 };
-
-// Distance of a point and an object: the one expression every path values with.
-__device__ __forceinline__ float emd_d2(float4 a, float bx, float by, float bz) {
-    float dx = a.x - bx, dy = a.y - by, dz = a.z - bz;
-    return dx * dx + dy * dy + dz * dz;
-}
 
 __device__ __forceinline__ float warp_max(float v) { return ord2f_emd(__reduce_max_sync(0xffffffffu, f2ord_emd(v))); }
 

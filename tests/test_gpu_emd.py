@@ -155,3 +155,17 @@ def test_emd_without_comparable_values_ends():
     for nbytes in (None, 1 << 20):
         st = _call(dev(A), dev(B), 1e-2, nbytes, max_iters=60)[0]
         assert st != 0
+
+
+@pytest.mark.parametrize("n", [11417, 11418])
+def test_emd_at_the_largest_size_with_lists(n):
+    """The largest n that takes lists (every slot of the scan's registers is used) and one more:
+    the same result with and without room for lists, within eps of each other's cost."""
+    rng = np.random.default_rng(n)
+    A, B = (rng.normal(size=(n, 3)).astype(np.float32) for _ in range(2))
+    eps = 3e-2
+    got = [_call(dev(A), dev(B), eps, nbytes) for nbytes in (None, 1 << 21)]
+    for st, out, sigma, it, _ in got:
+        assert st == 0 and it == got[0][3]
+        assert np.array_equal(out, got[0][1]) and np.array_equal(sigma, got[0][2])
+        assert np.array_equal(np.sort(sigma), np.arange(n))
