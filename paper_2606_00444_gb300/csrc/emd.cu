@@ -455,7 +455,7 @@ constexpr int kTailQueue = 256;
 constexpr int kTailAhead = 16;
 constexpr int kScanThreads = kTailThreads - 32;      // all but warp 0
 constexpr int kScanPer = 16;                         // objects a scanning thread holds
-constexpr int kTailMaxN = 11417;                     // largest n taken (16 + 4 B of shared memory each would fit)
+constexpr int kTailMaxN = 11417;                     // largest n taken: every object in a scanning thread's registers
 static_assert(kScanThreads * kScanPer >= kTailMaxN, "every object is held by a thread");
 static_assert(kTailAhead < kTailThreads / 32, "a warp per list, beside warp 0");
 
@@ -851,7 +851,10 @@ extern "C" {
 
 size_t mesh_emd_workspace_bytes(int64_t n) {
     if (n < 0 || n > ((int64_t)1 << 26)) return 0;
-    return emd_ws(nullptr, n).bytes;
+    // never less than for fewer points: past kTailMaxN a call takes no lists, but the same
+    // workspace then serves smaller calls, with theirs
+    const size_t own = emd_ws(nullptr, n).bytes, lists = n > kTailMaxN ? emd_ws(nullptr, kTailMaxN).bytes : 0;
+    return own > lists ? own : lists;
 }
 
 mesh_status mesh_emd(const float *d_A, const float *d_B, int64_t n, float eps_rel, int64_t max_iters,

@@ -113,3 +113,11 @@ def test_status_strings():
         assert len(L.mesh_status_string(s)) > 3
     with pytest.raises(_abi.MeshError):
         _abi.check(1, "x")
+
+
+def test_emd_workspace_never_shrinks_with_more_points():
+    """A workspace sized for the largest call serves every smaller one, lists and all."""
+    L = lib()
+    sizes = [L.mesh_emd_workspace_bytes(n) for n in (0, 1, 1000, 11416, 11417, 11418, 20000, 1 << 20, 1 << 26)]
+    assert sizes == sorted(sizes) and sizes[0] > 0
+    assert L.mesh_emd_workspace_bytes((1 << 26) + 1) == 0
