@@ -249,12 +249,11 @@ def gpu_arm(args, rank, world, local_rank):
     S0 = fixed.interpolate(cdf, cdb)
     tuned_cd = tune_chamfer(fixed, S0, rest, rest_S, step=True)
     Vin = torch.empty(nV, 3, device=dev)
-    # the contact step's workspace carries each particle's work class to the next frame
+    # (with a one-thread variant the contact step's workspace carries each particle's work
+    # class to the next frame)
     ct_ws = Workspace(dev)
     # contact faces persist from frame to frame: each frame's contact step (mesh_contact)
-    # is warm-started with the previous frame's faces and runs the particles in the
-    # order of the previous frame's work classes (the same answers up to near ties
-    # whose kept face depends on the order faces are met)
+    # is warm-started with the previous frame's faces (the same answers, bit for bit)
     contact = dict(face=torch.full((N_PART,), -1, dtype=torch.int32, device=dev),
                    bary=torch.empty(N_PART, 3, device=dev), point=torch.empty(N_PART, 3, device=dev),
                    dist2=torch.empty(N_PART, device=dev))
@@ -263,9 +262,8 @@ def gpu_arm(args, rank, world, local_rank):
     S_def = torch.empty(N_CD, 3, device=dev)
     cd_out = torch.empty(2, dtype=torch.float64, device=dev)
     # The frame's Chamfer runs as a step of the sequence (mesh_chamfer_step): warm-started
-    # from the previous frame's per-sample faces, each side's samples run heaviest first
-    # by the costs the previous frame left in its workspace (per-sample results those of
-    # mesh_chamfer, bit for bit); the plain call is timed beside it
+    # from the previous frame's per-sample faces (the results of mesh_chamfer, bit for
+    # bit); the plain call is timed beside it
     cd_ps = dict(faceA=torch.full((N_CD,), -1, dtype=torch.int32, device=dev),
                  baryA=torch.empty(N_CD, 3, device=dev), dist2A=torch.empty(N_CD, device=dev),
                  faceB=torch.full((N_CD,), -1, dtype=torch.int32, device=dev),
@@ -1140,7 +1138,7 @@ def fit_measure(n_steps):
     V = t(VT).requires_grad_(True)
     opt = torch.optim.Adam([V], lr=1e-3)
     # the Chamfer of each step is a step of the sequence (mesh_chamfer_step): warm-started
-    # from the previous step's faces, samples heaviest first by the previous step's costs
+    # from the previous step's faces
     state = chamfer_state(ns, ns, dev)
 
     def loss_of(Vx, grad):
@@ -1264,9 +1262,11 @@ def main():
     # particles stay in L2, so its bytes are bounded by L2, not HBM, bandwidth: the
     # headline fraction is its algorithmic bytes (44 B of query I/O, 64 B per node
     # visit = both children's 32-byte boxes, or 128 B per 4-wide record with
-    # traversal variant 13, 48 B per triangle test, counted by the
-    # counting form of the same traversal) over the L2 read bandwidth measured in
-    # this run.  Beside it, from the committed ncu capture of the same launch: DRAM
+    # traversal variant 13, 48 B per triangle test, as the counting form of the
+    # one-thread depth-first search counts them for the same queries: the pooled
+    # search visits some 3 % more nodes and tests 10 to 15 % more faces, so its
+    # fraction is a lower bound) over the L2 read bandwidth measured in this run.
+    # Beside it, from the committed ncu capture of the same launch: DRAM
     # bytes over the measured HBM peak, L2 bytes over the L2 peak, and the FP32 pipe.
     # Counters, time and ncu record all belong to the same launch: the search without
     # a warm start on frame ROOF_FRAME.
@@ -1289,6 +1289,7 @@ def main():
                            "L2-resident buffer, best of 20",
             "traffic": dram,
             "bytes_per_query": per_query,
+            "counted_by": "the one-thread depth-first search of the same queries",
             "per_query": {"io": CONTACT_BYTES, "node_visits": vis, "triangle_tests": tst,
                           "node_bytes": nb, "triangle_bytes": TRI_BYTES},
             "algorithmic_over_hbm_peak": achieved / hbm,

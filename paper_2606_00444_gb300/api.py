@@ -253,7 +253,8 @@ class MeshBVH:
         return out
 
     def closest_point_stats(self, Q: torch.Tensor, max_dist: float = math.inf) -> dict:
-        """Traversal work for these queries: node visits, triangle tests, hits (totals)."""
+        """Traversal work for these queries: node visits, triangle tests, hits (totals), as the
+        one-thread depth-first search meets them (mesh_closest_point_stats)."""
         Q = _f32(Q, 3, "Q")
         c = torch.zeros(3, dtype=torch.int64, device=Q.device)
         check(lib().mesh_closest_point_stats(self.handle, Q.data_ptr(), Q.shape[0], float(max_dist),
@@ -309,7 +310,7 @@ class MeshBVH:
 
     def set_query_config(self, lanes: int = -1, variant: int = -1, block: int | None = None) -> None:
         """Traversal choice for this handle's closest-point calls (-1 = process-wide);
-        `block`: threads per block of the one-thread variants 0, 2, 3 (32, 64, 128)."""
+        `block`: threads per block of the one-thread variants 2, 3, 13 (32, 64, 128)."""
         check(lib().mesh_bvh_set_query_config(self.handle, int(lanes), int(variant)),
               "mesh_bvh_set_query_config")
         if block is not None:
@@ -724,7 +725,7 @@ def set_query_group(lanes: int) -> None:
 
 
 def set_traversal(variant: int) -> None:
-    """One-thread traversal variant 0..12 (see mesh_set_traversal in include/meshgs.h)."""
+    """Search 0..13: 0 pooled, 1..13 one thread per query (mesh_set_traversal in include/meshgs.h)."""
     check(lib().mesh_set_traversal(int(variant)), "mesh_set_traversal")
 
 

@@ -25,7 +25,7 @@ struct mesh_bvh_impl {
     mesh_bvh_layout L;
     int cfg_lanes = -1;      // per-handle traversal choice; -1 = process-wide setting
     int cfg_variant = -1;
-    int cfg_block = 128;     // threads per block of the one-thread traversal (variants 0, 2, 3)
+    int cfg_block = 128;     // threads per block of the one-thread traversal (variants 2, 3, 13)
     int leaf_size = 1;       // faces per collapsed leaf, written by the next build / refit
     mutable bool wide_valid = false;   // the 4-wide records match the node records
     Header *hdr() const { return reinterpret_cast<Header *>(base + L.off_header); }
@@ -48,8 +48,7 @@ struct mesh_bvh_impl {
 struct BatchStatus {
     unsigned int status;
     unsigned int n_degenerate;
-    unsigned int work;       // not used
-    unsigned int pad;
+    unsigned int pad[2];
 };
 
 struct mesh_batch_impl {

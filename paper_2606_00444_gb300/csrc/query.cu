@@ -587,8 +587,8 @@ k_closest_point_persistent(Traversal T, const Header *__restrict__ hdr, unsigned
     }
 }
 
-// Counting form of the one-thread depth-first traversal (same visiting order
-// as variants 0, 2 and 3): node visits, triangle tests and hits, summed over
+// Counting form of the one-thread depth-first traversal (the visiting order of
+// variants 2 and 3; the pooled search of variant 0 visits a few per cent more): node visits, triangle tests and hits, summed over
 // all queries.  Separate instantiation; the timed kernels carry no counters.
 // kWide: the traversal over the 4-wide records (its visits count records).
 template <bool kRange, bool kWide = false>
@@ -682,8 +682,8 @@ bool wide_wanted(const mesh_bvh *b) {
     return (b->cfg_variant >= 0 ? b->cfg_variant : g_traversal) == 13 && b->cfg_lanes <= 1;
 }
 
-// Lanes per query that fill the GPU (2048 lanes per SM): 1 with enough queries,
-// else a power of two up to 32.
+// Lanes per query that fill 2048 lanes per SM (twice what the search kernels hold at a
+// time): 1 with enough queries, else a power of two up to 32.
 static int fill_lanes(int64_t nQ) {
     static int sms = 0;
     if (sms == 0) {
@@ -703,7 +703,7 @@ static int fill_lanes(int64_t nQ) {
 // lanes busy and take stack from the L1 cache: 1M queries of the 200k-face torus
 // took 289 / 267 / 349 us with 32 / 16 / 8 queries per warp under a cutoff and
 // 6.3 / 4.5 / 4.3 ms without; 20k took 97 / 58 / 50 / 40 / 44 / 56 us with 32 ... 1
-// (2 by this rule), 5k 68 ... 27 us (1 by this rule: 27).
+// (2 by this rule; 4, the best, would be a single fill), 5k 68 ... 27 us (1 by this rule: 27).
 // Meshes of few faces do without (0): 12 faces, 300k queries 74 us with it, 35 without (one
 // thread per query of the tree 87), 50k signed distances 54 and 22 (30), 100 queries 13 and
 // 13; 20 faces, 50k queries 36 and 21 (52), 100 queries 11 and 17 (15); 40 faces, 300k
