@@ -15,9 +15,9 @@
 // tests a face in nearly every step with three or four lanes on; 8 of 32 lanes
 // did useful work.  Here a lane is idle only while the pool holds fewer entries
 // than lanes, and the tail of one long search is shared by the whole warp: 26 of
-// 32 lanes on, 174 warp instructions per warm-started contact query.  Bound by
-// the mix of issue (a warp eligible in 63 % of cycles) and the reads of scattered
-// 64-byte records (L1 throughput 60 %) at 24 resident warps per SM.  1M contact queries of the
+// 32 lanes on, 172 warp instructions per warm-started contact query.  Bound by
+// the mix of issue (60 % of the slots) and the reads of scattered 64-byte records
+// (L1 throughput 65 %) at some 24 resident warps per SM.  1M contact queries of the
 // 200k-face torus: 549 -> 309 us cold, 380 -> 255 us warm-started (the one-thread
 // form with its work classes); unbounded 12.7 -> 4.5 ms; 20k queries 117 -> 44 us.
 //
