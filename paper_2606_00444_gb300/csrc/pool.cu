@@ -129,12 +129,12 @@ static __device__ __noinline__ void pool_absorb(const float4 *tris, float tau, P
 
 // A cutoff is loose when the ball of that radius may hold more faces than a search
 // should meet without a nearer radius: about n r^2 / diag^2 of a surface of n faces,
-// some three times that for a closed one.  Lines at 50, 200 and 1000 measured the same
-// for tight cutoffs (1M signed queries, cutoff 0.05 of a 3.9 diagonal: 302 to 314 us);
-// 50k queries near a 5k-face torus, cutoff 0.7 (160 by this estimate), took 79, 202 and
-// 204 us.  With no rule a loose cutoff cost 2 to 18 times one thread per query (1M
+// some three times that for a closed one.  With lines at 50, 150 and 200: two contact
+// steps of 943k particles, 80k faces, cutoff 0.1 (54 by this estimate) 696 us above the
+// line, 675 below it; 50k queries near a 5k-face torus, cutoff 0.7 (160) 79 above, 99
+// below.  With no line a loose cutoff cost 2 to 18 times one thread per query (1M
 // queries near the 200k-face torus, cutoff 2.0: 19.9 ms against 1.2; 0.96 now).
-constexpr float kLooseFaces = 50.0f;
+constexpr float kLooseFaces = 150.0f;
 
 // Meshes of at most kFewFaces faces: a thread per query tests every face.  A warp
 // of the pool spends more on starting and ending its queries than such a search
