@@ -153,7 +153,10 @@ __device__ __forceinline__ Hit few_search(const Traversal &T, float4 lo, float4 
 // The search of a warp's S queries; lane l < S brings query l (valid or not; T
 // holds its mesh's scale and size) and takes its hit.  hint: a leaf tested first, or -1.  A query without a
 // hint starts at the first node with two children inside the cutoff (descend: at the
-// root), which ends most misses at once; when the cutoff is loose or there is none
+// root), which ends most misses at once (from the root, timed over 792 calls: 2 % more in
+// two contact steps or signed distances of 1M ordered particles, 10 to 15 % more where
+// most miss; only 1M queries close to the surface and in no order were faster, 977
+// against 1076 us); when the cutoff is loose or there is none
 // (descend) it then goes down the nearer children to one leaf, so that the pool
 // starts with a radius for it.
 // sc: per-query offsets into T's arrays (queries of several scenes), or NULL.
